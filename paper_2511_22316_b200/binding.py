@@ -109,25 +109,27 @@ def _check(code: int, where: str) -> None:
 
 def _ptr(t) -> Optional[int]:
     """Device (torch tensor) or host (numpy array) pointer; None stays NULL."""
-    if t is None:
-        return None
-    if isinstance(t, np.ndarray):
-        return t.ctypes.data
-    if isinstance(t, int):
+    try:
+        return t.data_ptr()             # the usual argument first: a decode step is bound by its host calls
+    except AttributeError:
+        pass
+    if t is None or isinstance(t, int):
         return t
-    return t.data_ptr()
+    return t.ctypes.data
 
 
-_torch = None
+_current_device = _raw_stream = None
 
 
 def _stream(stream) -> Optional[int]:
+    # The raw handle of the current stream without a Stream object around it: 0.3 us instead of 3.2 us, of
+    # some 10 us that a whole sq_linear call took on the host.
     if stream is None:
-        global _torch
-        if _torch is None:
+        global _current_device, _raw_stream
+        if _raw_stream is None:
             import torch
-            _torch = torch
-        return _torch.cuda.current_stream().cuda_stream or None
+            _current_device, _raw_stream = torch.cuda.current_device, torch._C._cuda_getCurrentRawStream
+        return _raw_stream(_current_device()) or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
