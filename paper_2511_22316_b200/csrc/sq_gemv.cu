@@ -34,11 +34,32 @@ w4a4_gemv_kernel(const uint8_t* __restrict__ Xq, const __half* __restrict__ sx, 
                  const __half* __restrict__ sw, int M, int N, int K, __half* __restrict__ Y,
                  int32_t* __restrict__ accdbg) {
   griddep_launch_dependents();                           // a rotate kernel launched behind this one may set itself up
-  griddep_wait();                                        // Xq and sx may come from the kernel launched before this one
   extern __shared__ __align__(16) uint32_t xs[];
   constexpr int GV_ROWS = GvRows<MT>::value;
   const int kw = K / 8;                                  // packed words per row
   const int nchunk = K / 32;                             // 16-byte pieces per row
+  const int lane = threadIdx.x & 31;
+  const int warps_per_cta = blockDim.x >> 5;
+  const long long ntask = (N + GV_ROWS - 1) / GV_ROWS;
+  const long long wstride = static_cast<long long>(gridDim.x) * warps_per_cta;
+  // task index interleaved over CTAs first, so that the warps of all SMs work on neighbouring rows
+  long long task = static_cast<long long>(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  uint4 wv[GV_UNROLL][GV_ROWS];
+  auto load_w = [&](long long tk, int c0) {
+    const int row0 = static_cast<int>(tk) * GV_ROWS;
+#pragma unroll
+    for (int r = 0; r < GV_ROWS; ++r) {
+      const uint4* wrow = reinterpret_cast<const uint4*>(Wq + static_cast<size_t>(min(row0 + r, N - 1)) * (K / 2)) + c0;
+#pragma unroll
+      for (int u = 0; u < GV_UNROLL; ++u)
+        wv[u][r] = (c0 + 32 * u < nchunk) ? __ldcs(wrow + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  // The warp's first pieces of weights are requested before the predecessor is awaited, like the first blocks of the
+  // tensor-core kernels: over a 29 MB layer that is half of all, in flight while the tokens are still being rotated
+  // (1 x 4096 -> 14336: layer 13.4 -> 11.8 us, product alone 8.0 -> 7.0; 4096 -> 4096: layer 8.8 -> 7.5).
+  if (task < ntask) load_w(task, lane);
+  griddep_wait();                                        // Xq and sx may come from the kernel launched before this one
   // tokens -> shared memory, four 16-byte pieces per thread in flight
   for (int i0 = threadIdx.x; i0 < MT * nchunk; i0 += 4 * blockDim.x) {
     uint4 w[4];
@@ -64,31 +85,15 @@ w4a4_gemv_kernel(const uint8_t* __restrict__ Xq, const __half* __restrict__ sx, 
   }
   __syncthreads();
 
-  const int lane = threadIdx.x & 31;
-  const int warps_per_cta = blockDim.x >> 5;
-  const long long ntask = (N + GV_ROWS - 1) / GV_ROWS;
-  const long long wstride = static_cast<long long>(gridDim.x) * warps_per_cta;
-  // task index interleaved over CTAs first, so that the warps of all SMs work on neighbouring rows
-  for (long long task = static_cast<long long>(threadIdx.x >> 5) * gridDim.x + blockIdx.x; task < ntask; task += wstride) {
+  for (bool first = true; task < ntask; task += wstride, first = false) {
     const int row0 = static_cast<int>(task) * GV_ROWS;
     int acc[GV_ROWS][MT];
 #pragma unroll
     for (int r = 0; r < GV_ROWS; ++r)
 #pragma unroll
       for (int t = 0; t < MT; ++t) acc[r][t] = 0;
-    const uint4* wrow[GV_ROWS];
-#pragma unroll
-    for (int r = 0; r < GV_ROWS; ++r)
-      wrow[r] = reinterpret_cast<const uint4*>(Wq + static_cast<size_t>(min(row0 + r, N - 1)) * (K / 2));
     for (int c0 = lane; c0 < nchunk; c0 += 32 * GV_UNROLL) {
-      uint4 wv[GV_UNROLL][GV_ROWS];
-#pragma unroll
-      for (int u = 0; u < GV_UNROLL; ++u) {
-        const int c = c0 + 32 * u;
-#pragma unroll
-        for (int r = 0; r < GV_ROWS; ++r)
-          wv[u][r] = (c < nchunk) ? __ldcs(wrow[r] + c) : make_uint4(0u, 0u, 0u, 0u);
-      }
+      if (!first || c0 != lane) load_w(task, c0);
 #pragma unroll
       for (int u = 0; u < GV_UNROLL; ++u) {
         const int c = c0 + 32 * u;
