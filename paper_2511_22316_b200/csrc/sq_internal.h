@@ -30,6 +30,7 @@ struct sq_rotation {
   // tensor-core rotate+quant: shared-memory images of the split factors (device), if supported
   void* dA1img = nullptr;
   void* dB2img = nullptr;
+  void* dMmaImg = nullptr; // operand images of the warp-level kernel (sq_rotate_quant_mma.cu), if supported
   bool tc_ready = false;   // images for the single-CTA kernel (n1 <= 128)
   bool tc_pair = false;    // images for the CTA-pair kernel (128 < n1 <= 256)
   // structured application of R2 (sq_rotate_quant_st.cu): composition and kernel coefficients
@@ -127,16 +128,21 @@ sq_status_t build_factors_host(const float* calib, int64_t T, int64_t n, int32_t
 sq_status_t launch_rotate_quant(const float* dR1, const float* dR2, int n1, int n2, const void* X,
                                 int64_t rows, void* Xq, void* scales, float* Zdbg, cudaStream_t s, int qmax = 7);
 
-// Tensor-core variant of steps 1+2 (sq_rotate_quant_tc.cu).
+// Tensor-core variant of steps 1+2 (sq_rotate_quant_tc.cu).  qmax as in launch_rotate_quant, also below.
 bool rotate_quant_tc_supported(int n1, int n2);
 bool rotate_quant_tc_prepare(sq_rotation* h);
 sq_status_t launch_rotate_quant_tc(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
-                                   float* Zdbg, cudaStream_t s, bool f16out = false);
+                                   float* Zdbg, cudaStream_t s, int qmax = 7);
 // Tensor-core variant for 128 < n1 <= 256 on CTA pairs (sq_rotate_quant_pair.cu).
 bool rotate_quant_pair_supported(int n1, int n2);
 bool rotate_quant_pair_prepare(sq_rotation* h);
 sq_status_t launch_rotate_quant_pair(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
-                                     float* Zdbg, cudaStream_t s, bool f16out = false);
+                                     float* Zdbg, cudaStream_t s, int qmax = 7);
+// Warp-level variant (sq_rotate_quant_mma.cu): n2 = 32.  qmax as in launch_rotate_quant.
+bool rotate_quant_mma_supported(int n1, int n2);
+bool rotate_quant_mma_prepare(sq_rotation* h);
+sq_status_t launch_rotate_quant_mma(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales, float* Zdbg,
+                                    cudaStream_t s, int qmax = 7);
 // Steps 1+2 with R2 applied through its structure (sq_rotate_quant_st.cu): R1^T on the tensor cores,
 // then the Hadamard butterflies and the two rotation chains of URT in registers.
 bool rotate_quant_st_prepare(sq_rotation* h);
@@ -150,7 +156,7 @@ sq_status_t launch_linear_fused(const sq_rotation* h, const void* X, int64_t M, 
                                 int64_t N, int64_t K, void* Xq, void* sx, void* Y, cudaStream_t s);
 // Picks the tensor-core kernel when the handle has its images, else the generic fp32 kernel.
 sq_status_t rotate_quant_dispatch(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
-                                  float* Zdbg, cudaStream_t s);
+                                  float* Zdbg, cudaStream_t s, int qmax = 7);
 
 // Step 1 alone with fp16 rows out (the rotation-only form of the kernels above).
 sq_status_t rotate_f16_dispatch(const sq_rotation* h, const void* X, int64_t rows, void* Z16, cudaStream_t s);

@@ -146,6 +146,18 @@ def test_rotate_quant_small_and_ragged(sq, n1, n2, M):
     check_rotate_quant(sq, X, R1, R2)
 
 
+# The warp-level kernel (n2 = 32): every n1 class and its edges, several tokens per CTA; n1 = 129 takes the fp32 kernel.
+MMA_ROT = [(1, 32, 3), (15, 32, 2), (16, 32, 1300), (17, 32, 5), (33, 32, 4), (64, 32, 9), (65, 32, 4), (81, 32, 2), (97, 32, 3),
+           (128, 32, 700), (129, 32, 2)]
+
+
+@pytest.mark.parametrize("n1,n2,M", MMA_ROT)
+def test_rotate_quant_warp_level(sq, n1, n2, M):
+    X = wl.make_activations(wl.small(f"rm{n1}x{n2}", M, n1, n2, 8, seed=n1 * 11 + n2))
+    R1, R2 = ora.build_rotation(X.astype(np.float32), n1, n2, seed=2)
+    check_rotate_quant(sq, X, R1, R2)
+
+
 def test_rotate_quant_tiny_config(sq):
     w = wl.TINY
     X = wl.make_activations(w)
