@@ -21,6 +21,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "sq_internal.h"
 #include "sq_ptx.cuh"
@@ -667,7 +668,8 @@ wo_gemm_tmem_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
 // the N operand).  An MMA then does 128 cycles of arithmetic per 4 KB of A, and a CTA reads 128 tokens per
 // 256 tokens' worth of work.  The accumulator (128 lanes x 256 columns per CTA) is single-buffered: the
 // operand ring needs the other 256 columns; eight epilogue warps (two per lane quarter, 128 columns
-// each) hand it back after their last read.
+// each) hand it back after their last read.  The tile's token width is the host's choice (wo_pair_tile_m); 256 above
+// stands for the widest.
 //   warp 0        TMA: packed weights of this CTA's channels (staging ring), this CTA's tokens (ring
 //                 stage s = four 64-channel k-blocks)
 //   warps 2..9    two converter groups, alternating stages: staging -> registers -> tensor-memory ring
@@ -702,7 +704,7 @@ struct WoPairSmem {
 template <int SS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(WP_THREADS, 1)
 wo_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_constant__ CUtensorMap tmap_w,
-                    const __half* __restrict__ sw, int M, int N, int K, __half* __restrict__ Y) {
+                    const __half* __restrict__ sw, int M, int N, int K, int tile_m, __half* __restrict__ Y) {
   using L = WoPairSmem<SS>;
   griddep_launch_dependents();
   extern __shared__ unsigned char smem_dyn[];
@@ -724,7 +726,7 @@ wo_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
   const int num_sb = (num_kb + 3) / 4;                // stages per tile (the last may hold fewer than four k-blocks)
   // channel tiles run fastest: the pairs at work at one time share a few token tiles, which stay in L2
   const int tiles_n = (N + 255) / 256;
-  const int num_tiles = tiles_n * ((M + 255) / 256);
+  const int num_tiles = tiles_n * ((M + tile_m - 1) / tile_m);
   const uint32_t limit = wait_limit();
 
   // The weights do not depend on the kernel before this one: the first ring-full of them is requested
@@ -776,7 +778,7 @@ wo_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
       bool ok = true;
       for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
         const int ch0 = (tile % tiles_n) * 256 + static_cast<int>(rank) * 128;
-        const int tok0 = (tile / tiles_n) * 256 + static_cast<int>(rank) * 128;
+        const int tok0 = (tile / tiles_n) * tile_m + static_cast<int>(rank) * (tile_m / 2);
         for (int sb = 0; sb < num_sb && ok; ++sb, ++it) {
           if (it >= static_cast<uint32_t>(pre)) {
             const int ss = it % SS;
@@ -789,7 +791,7 @@ wo_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
           const int nk = (num_kb - 4 * sb) < 4 ? (num_kb - 4 * sb) : 4;
           ok = mbar_wait(&empty[s], ((it / WP_S) & 1) ^ 1, WP_EMPTY_T, limit);
           if (!ok) break;
-          mbar_arrive_expect_tx(&t_full[s], static_cast<uint32_t>(nk * L::T_KB));
+          mbar_arrive_expect_tx(&t_full[s], static_cast<uint32_t>(nk * (tile_m / 2) * 128));
           for (int h = 0; h < nk; ++h)
             tma_load_2d(smem + L::OFF_T + s * L::T_TILE + h * L::T_KB, &tmap_z, &t_full[s], (4 * sb + h) * 64, tok0);
         }
@@ -798,7 +800,7 @@ wo_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
   } else if (warp == 1) {
     // ------------------------------ MMA issuer (leader CTA) -------------------------------
     if (rank == 0 && elect_one()) {
-      constexpr uint32_t idesc = umma_idesc(/*c=f32*/ 1, /*a=f16*/ 0, /*b=f16*/ 0, 256, 256);
+      const uint32_t idesc = umma_idesc(/*c=f32*/ 1, /*a=f16*/ 0, /*b=f16*/ 0, 256, static_cast<uint32_t>(tile_m));
       const uint64_t t_desc0 = umma_desc_sw128(smem_u32(smem + L::OFF_T));
       uint32_t it = 0, tcount = 0;
       bool ok = true;
@@ -885,23 +887,25 @@ wo_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
   } else {
     // ------------------------------ epilogue warps ------------------------------------------
     const int q = warp & 3;                             // TMEM lane quarter this warp may read
-    const int half = (warp - (2 + WOD_CONV_WARPS)) >> 2;  // its 128 of the 256 token columns
+    // its part of the token columns, in chunks of 16: the first half (rounded up) or the rest
+    const int half = (warp - (2 + WOD_CONV_WARPS)) >> 2;
+    const int c_all = tile_m / 16, c_first = half ? (c_all + 1) / 2 : 0, c_end = half ? c_all : (c_all + 1) / 2;
     uint32_t tcount = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += npairs, ++tcount) {
       const int ch = (tile % tiles_n) * 256 + static_cast<int>(rank) * 128 + q * 32 + lane;
-      const int tok0 = (tile / tiles_n) * 256 + half * 128;
+      const int tok0 = (tile / tiles_n) * tile_m;
       const float swv = (ch < N) ? __half2float(sw[ch]) : 0.0f;
       ok = mbar_wait(tmem_full, tcount & 1, WP_TMEM_FULL, limit);
       if (!ok) break;
       tc_fence_after_sync();
-      const uint32_t tmem_d = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + half * 128;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
+      const uint32_t tmem_d = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
+#pragma unroll 1
+      for (int c = c_first; c < c_end; ++c) {
         uint32_t r[16];
         tmem_ld_32x32b_x16(tmem_d + c * 16, r);
         tmem_wait_ld();
-        if (c == 7) {                                   // last read of this warp: hand the accumulator back
+        if (c == c_end - 1) {                                   // last read of this warp: hand the accumulator back
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(tmem_empty, 0);
@@ -1146,6 +1150,27 @@ sq_status_t launch_wo_decode(const void* Z16, const void* Wq, const void* sw, in
   return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SQ_OK : SQ_ERR_CUDA;
 }
 
+// Token width of the CTA-pair kernel's tiles, a multiple of 16 from 64 to 256.  A tile of width w takes a time of about
+// w + 144 (fit of eleven widths on 777 x 11008 x 4096: 14.4 us at 96, 18.6 at 160, 24.4 at 256; the constant is the weights'
+// share of the operand supply and the hand-overs), and a batch that is no multiple of 256 tokens, or whose tiles do not
+// divide by the pairs, wastes part of the wide ones: 777 x 11008 x 4096 72 us in three waves of 256 (two thirds of the last
+// wave empty), 56 us in three full waves of 160.  The cost is waves x (w + 144), mixed with the same sum without rounding
+// up: what the chip as a whole has to move (2048 x 4096 x 4096: two waves of 240 measure 53.6 us, two of 256 50.9).
+int wo_pair_tile_m(int M, int N, int pairs) {
+  const double ch_tiles = (N + 255) / 256;
+  int best = 256;
+  double best_cost = 0.0;
+  for (int w = 256; w >= 64; w -= 16) {
+    const double load = ch_tiles * ((M + w - 1) / w) / pairs, waves = std::ceil(load);
+    const double cost = (0.6 * waves + 0.4 * load) * (w + 144);
+    if (w == 256 || cost < best_cost) {
+      best = w;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 template <int SS>
 sq_status_t launch_wo_pair(const void* Z16, const void* Wq, const void* sw, int M, int N, int K, void* Y, cudaStream_t s) {
   using L = WoPairSmem<SS>;
@@ -1155,7 +1180,10 @@ sq_status_t launch_wo_pair(const void* Z16, const void* Wq, const void* sw, int 
   CUtensorMap mz, mw;
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(K), static_cast<cuuint64_t>(M)};
   const cuuint64_t strides[1] = {static_cast<cuuint64_t>(K) * 2};
-  const cuuint32_t box[2] = {64, 128};
+  const int sms = sm_count();
+  if (sms <= 0) return SQ_ERR_CUDA;
+  const int tile_m = wo_pair_tile_m(M, N, sms / 2);
+  const cuuint32_t box[2] = {64, static_cast<cuuint32_t>(tile_m / 2)};
   const cuuint32_t estr[2] = {1, 1};
   if (enc(&mz, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(Z16), dims, strides, box, estr,
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1164,12 +1192,10 @@ sq_status_t launch_wo_pair(const void* Z16, const void* Wq, const void* sw, int 
   if (!make_packed_map(&mw, Wq, N, K / 2, 128)) return SQ_ERR_CUDA;
   auto kern = wo_gemm_pair_kernel<SS>;
   if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), L::DYN_BYTES)) return SQ_ERR_CUDA;
-  const int sms = sm_count();
-  if (sms <= 0) return SQ_ERR_CUDA;
-  const int tiles = ((N + 255) / 256) * ((M + 255) / 256);
+  const int tiles = ((N + 255) / 256) * ((M + tile_m - 1) / tile_m);
   const int pairs = tiles < sms / 2 ? tiles : sms / 2;
   const cudaError_t err = launch_maybe_pdl(kern, dim3(2 * pairs), dim3(WP_THREADS), L::DYN_BYTES, s, mz, mw,
-                                           static_cast<const __half*>(sw), M, N, K, static_cast<__half*>(Y));
+                                           static_cast<const __half*>(sw), M, N, K, tile_m, static_cast<__half*>(Y));
   count_launch();
   return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SQ_OK : SQ_ERR_CUDA;
 }
@@ -1213,8 +1239,14 @@ sq_status_t launch_wo_gemm(const void* Z16, const void* Wq, const void* sw, int6
     // operand cost no shared-memory traffic at all, which is what bounds the kernel below (2048 x 4096 x
     // 4096: 76 us there).  From 256 channels on, two channel tiles share every token block (half the
     // token traffic out of L2 per flop: 65 -> 61 us on that shape, 1.85 -> 1.65 ms on 4096 x 28672 x 8192).
-    // Above 128 tokens: CTA pairs on 256 x 256 tiles (an MMA's 4 KB of A then feed twice the arithmetic).
-    if (M > 128 && N >= 256) return launch_wo_pair<4>(Z16, Wq, sw, (int)M, (int)N, (int)K, Y, s);
+    // CTA pairs (an MMA's 4 KB of A then feed twice the arithmetic) above 128 tokens, and from 65 on where they do
+    // not take twice as many waves of channel tiles as the single-CTA form: 100 x 4096 x 4096 31.0 -> 16.5 us,
+    // 128 x 4096 x 14336 92 -> 49; with two waves against one, 100 x 32000 x 4096, 33.7 -> 36.5.
+    const int sms = sm_count();
+    if (sms <= 0) return SQ_ERR_CUDA;
+    const int64_t ch_tiles = (N + 255) / 256, pairs = sms / 2;
+    if (N >= 256 && pairs > 0 && (M > 128 || (ch_tiles + pairs - 1) / pairs < 2 * ((ch_tiles + sms - 1) / sms)))
+      return launch_wo_pair<4>(Z16, Wq, sw, (int)M, (int)N, (int)K, Y, s);
     if (N >= 256) return launch_wo_decode<128, 2, 4, 2>(Z16, Wq, sw, (int)M, (int)N, (int)K, Y, s);
     return launch_wo_decode<128, 2, 4>(Z16, Wq, sw, (int)M, (int)N, (int)K, Y, s);
   }

@@ -42,7 +42,7 @@ linear_decode_fused_kernel(const __grid_constant__ CUtensorMap tmap_xin, const _
   uint32_t* done = counters + 1;         // GEMM CTAs that have finished
   const int cta = static_cast<int>(blockIdx.x);
   if (cta < rot_ctas) {
-    rotate_quant_tc_body<N2, 2>(tmap_xin, L, a1_img, b2_img, n1, M, Xq, sx, nullptr, 7, cta, rot_ctas);
+    rotate_quant_tc_body<N2, 2>(tmap_xin, L, a1_img, b2_img, n1, M, Xq, sx, nullptr, cta, rot_ctas);
     // every thread's stores precede the block barrier at the end of the body; the release is cumulative
     if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ready) : "memory");
   } else {

@@ -75,7 +75,7 @@ template <int N2, int CW, bool F16OUT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((2 + 4 * CW * (256 / N2)) * 32, 1)
 rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsigned char* __restrict__ a1_img,
                          const unsigned char* __restrict__ b2_img, int n1, long long rows,
-                         uint8_t* __restrict__ Xq, __half* __restrict__ scales, float* __restrict__ Zdbg, int qmax) {
+                         uint8_t* __restrict__ Xq, __half* __restrict__ scales, float* __restrict__ Zdbg) {
   constexpr int S = 256 / N2;
   constexpr int SLOT_COLS = 2 * N2;
   const RqPairLayout L = rq_pair_layout(n1, N2);
@@ -343,7 +343,7 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
       amax = fmaxf(amax, amax_peer[w * 2 + ph]);
       __half delta;
       float inv;
-      row_scale(amax, delta, inv, qmax);
+      row_scale(amax, delta, inv);
       const float inv_un = inv * un;
       const bool clamp = __half2float(delta) < 6.103515625e-05f;
       uint8_t* orow = Xq + token * (n / 2) + static_cast<long long>(pp) * (N2 / 2) + cp * (HC / 2);
@@ -357,7 +357,7 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
           t[e] = __fadd_rn(__fmul_rn(__uint_as_float(r[e]), inv_un), 0.5f);
-          if (clamp) t[e] = fminf(fmaxf(t[e], -1.0f - qmax), qmax + 0.5f);
+          if (clamp) t[e] = fminf(fmaxf(t[e], -8.0f), 7.5f);
         }
         uint2 pk;
         pk.x = pack8_codes(t);
@@ -475,7 +475,7 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
       amax = fmaxf(amax, amax_peer[w * 2 + ph]);
       __half delta;
       float inv;
-      row_scale(amax, delta, inv, qmax);
+      row_scale(amax, delta, inv);
       const float inv_un = inv * un;
       const bool clamp = __half2float(delta) < 6.103515625e-05f;   // see sq_rotate_quant_tc.cu
       uint8_t* orow = Xq + token * (n / 2) + static_cast<long long>(pp) * (N2 / 2);
@@ -489,7 +489,7 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
 #pragma unroll
         for (int e = 0; e < 32; ++e) {
           t[e] = __fadd_rn(__fmul_rn(__uint_as_float(r[e]), inv_un), 0.5f);
-          if (clamp) t[e] = fminf(fmaxf(t[e], -1.0f - qmax), qmax + 0.5f);
+          if (clamp) t[e] = fminf(fmaxf(t[e], -8.0f), 7.5f);
         }
         uint4 pk;
         pk.x = pack8_codes(t);
@@ -565,8 +565,7 @@ bool rotate_quant_pair_prepare(sq_rotation* h) {
 }
 
 sq_status_t launch_rotate_quant_pair(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
-                                     float* Zdbg, cudaStream_t s, int qmax) {
-  const bool f16out = qmax == 0;
+                                     float* Zdbg, cudaStream_t s, bool f16out) {
   const int n1 = h->n1, n2 = h->n2;
   const RqPairLayout L = rq_pair_layout(n1, n2);
   EncodeTiledFn enc = get_encode_fn();
@@ -591,14 +590,14 @@ sq_status_t launch_rotate_quant_pair(const sq_rotation* h, const void* X, int64_
     auto kern = f16out ? rotate_quant_pair_kernel<64, 1, true> : rotate_quant_pair_kernel<64, 1, false>;
     if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem)) return SQ_ERR_CUDA;
     if (launch_dependent(kern, dim3(grid), dim3((2 + 4 * 4) * 32), static_cast<size_t>(smem), s, mx, a1, b2, n1, rows,
-                         static_cast<uint8_t*>(Xq), static_cast<__half*>(scales), Zdbg, qmax) != cudaSuccess)
+                         static_cast<uint8_t*>(Xq), static_cast<__half*>(scales), Zdbg) != cudaSuccess)
       return SQ_ERR_CUDA;
   } else {
     // two slots of eight warps (18 warps in the CTA instead of 10)
     auto kern = f16out ? rotate_quant_pair_kernel<128, 2, true> : rotate_quant_pair_kernel<128, 2, false>;
     if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem)) return SQ_ERR_CUDA;
     if (launch_dependent(kern, dim3(grid), dim3((2 + 4 * 2 * 2) * 32), static_cast<size_t>(smem), s, mx, a1, b2, n1, rows,
-                         static_cast<uint8_t*>(Xq), static_cast<__half*>(scales), Zdbg, qmax) != cudaSuccess)
+                         static_cast<uint8_t*>(Xq), static_cast<__half*>(scales), Zdbg) != cudaSuccess)
       return SQ_ERR_CUDA;
   }
   count_launch();

@@ -135,7 +135,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
                                                      const unsigned char* __restrict__ a1_img,
                                                      const unsigned char* __restrict__ b2_img, int n1, int rows,
                                                      uint8_t* __restrict__ Xq, __half* __restrict__ scales,
-                                                     float* __restrict__ Zdbg, int qmax, int cta, int ncta) {
+                                                     float* __restrict__ Zdbg, int cta, int ncta) {
   constexpr int TM_COLS = S * 2 * N2;             // 256 or 512
   constexpr int XQ = N2 / 64;
   constexpr int SLOT_COLS = 2 * N2;              // D1 (N2 columns) + D2 (N2 columns)
@@ -406,7 +406,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       for (int x = 1; x < wpt; ++x) amax = fmaxf(amax, fmaxf(amax_w[(q0 + x) * 2], amax_w[(q0 + x) * 2 + 1]));
       __half delta;
       float inv;
-      row_scale(amax, delta, inv, qmax);
+      row_scale(amax, delta, inv);
       const float inv_un = inv * un;
       const bool live = (pp < n1) && (token < rows);
       const bool clamp = __half2float(delta) < 6.103515625e-05f;
@@ -421,7 +421,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
           t[e] = __fadd_rn(__fmul_rn(__uint_as_float(r[e]), inv_un), 0.5f);
-          if (clamp) t[e] = fminf(fmaxf(t[e], -1.0f - qmax), qmax + 0.5f);
+          if (clamp) t[e] = fminf(fmaxf(t[e], -8.0f), 7.5f);
         }
         uint2 pk;
         pk.x = pack8_codes(t);
@@ -541,10 +541,10 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       for (int x = 1; x < wpt; ++x) amax = fmaxf(amax, amax_w[q0 + x]);
       __half delta;
       float inv;
-      row_scale(amax, delta, inv, qmax);
+      row_scale(amax, delta, inv);
       const float inv_un = inv * un;                 // exact: un is a power of two
       const bool live = (pp < n1) && (token < rows);
-      // Delta >= 2^-14 (a normal fp16) bounds |z / Delta| by qmax (1 + 2^-11): no clamp is needed then.
+      // Delta >= 2^-14 (a normal fp16) bounds |z / Delta| by 7 (1 + 2^-11): no clamp is needed then.
       const bool clamp = __half2float(delta) < 6.103515625e-05f;
       uint8_t* orow = Xq + token * (n / 2) + pp * (N2 / 2);
       float* zrow = (Zdbg != nullptr && live) ? Zdbg + token * n + pp * N2 : nullptr;
@@ -557,7 +557,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
 #pragma unroll
         for (int e = 0; e < 32; ++e) {
           t[e] = __fadd_rn(__fmul_rn(__uint_as_float(r[e]), inv_un), 0.5f);
-          if (clamp) t[e] = fminf(fmaxf(t[e], -1.0f - qmax), qmax + 0.5f);
+          if (clamp) t[e] = fminf(fmaxf(t[e], -8.0f), 7.5f);
         }
         uint4 pk;
         pk.x = pack8_codes(t);
@@ -593,9 +593,9 @@ template <int N2, int S, int CW = 1, bool F16OUT = false>
 __global__ void __launch_bounds__((2 + 4 * S * CW) * 32, (S * 2 * N2 <= 256) ? 2 : 1)
 rotate_quant_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ RqLayout L,
                        const unsigned char* __restrict__ a1_img, const unsigned char* __restrict__ b2_img, int n1,
-                       int rows, uint8_t* __restrict__ Xq, __half* __restrict__ scales, float* __restrict__ Zdbg, int qmax) {
-  rotate_quant_tc_body<N2, S, CW, F16OUT>(tmap_x, L, a1_img, b2_img, n1, rows, Xq, scales, Zdbg, qmax,
-                                          static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x));
+                       int rows, uint8_t* __restrict__ Xq, __half* __restrict__ scales, float* __restrict__ Zdbg) {
+  rotate_quant_tc_body<N2, S, CW, F16OUT>(tmap_x, L, a1_img, b2_img, n1, rows, Xq, scales, Zdbg, static_cast<int>(blockIdx.x),
+                              static_cast<int>(gridDim.x));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -656,8 +656,7 @@ bool rotate_quant_tc_prepare(sq_rotation* h) {
 }
 
 sq_status_t launch_rotate_quant_tc(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
-                                   float* Zdbg, cudaStream_t s, int qmax) {
-  const bool f16out = qmax == 0;
+                                   float* Zdbg, cudaStream_t s, bool f16out) {
   const int n1 = h->n1, n2 = h->n2;
   if (rows > 0x7FFFFFFF) return SQ_ERR_UNSUPPORTED;   // the kernel counts token groups in 32 bits
   // n2 = 64 with images small enough: two CTAs per SM, two accumulator slots each.
@@ -687,7 +686,7 @@ sq_status_t launch_rotate_quant_tc(const sq_rotation* h, const void* X, int64_t 
     const unsigned grid = static_cast<unsigned>(std::min<long long>(ngroups, static_cast<long long>(sms) * ctas_per_sm));
     return launch_dependent(kern, dim3(grid), dim3((2 + 4 * slots * cw) * 32), static_cast<size_t>(smem), s, mx, L, a1, b2, n1,
                             static_cast<int>(rows), static_cast<uint8_t*>(Xq), static_cast<__half*>(scales),
-                            Zdbg, qmax) == cudaSuccess;
+                            Zdbg) == cudaSuccess;
   };
   bool ok;
   // n2 = 128 (one CTA per SM, two slots): eight warps per slot, 18 in all instead of 10 -- measured 10 %

@@ -187,6 +187,15 @@ def test_wo_gemm_full_size_bit_exact_on_sampled_rows(sq, M, N, K):
         assert np.array_equal(Yg[rows, c0:c0 + 4096].view(np.uint16), Yo.view(np.uint16))
 
 
+# Token widths of the CTA-pair kernel's tiles from 64 up (one tile as wide as the batch, ragged last tiles, several waves),
+# and both sides of its line to the single-CTA form between 65 and 128 tokens.
+@pytest.mark.parametrize("M,N,K", [(65, 256, 64), (81, 264, 320), (97, 520, 256), (128, 4096, 128), (145, 256, 512),
+                                   (161, 264, 64), (177, 512, 192), (209, 256, 256), (241, 392, 128), (513, 4096, 128),
+                                   (777, 11008, 64), (100, 18944, 64), (100, 18952, 64)])
+def test_wo_gemm_tile_widths_bit_exact(sq, M, N, K):
+    test_wo_gemm_is_bit_exact_on_small_integers(sq, M, N, K)
+
+
 def test_wo_gemm_random_shapes_bit_exact(sq):
     """Forty-eight seeded random shapes over every kernel of the product (dot products, the single-CTA
     form with and without the K split and with one or two channel tiles, the CTA-pair form, the plain
