@@ -83,18 +83,18 @@ __global__ void bounded_wait_probe_kernel(uint32_t polls) {
 
 namespace sq {
 sq_status_t rotate_quant_dispatch(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
-                                  float* Zdbg, cudaStream_t s, int qmax) {
-  if (h->st_ready && qmax == 7) return launch_rotate_quant_st(h, X, rows, Xq, scales, Zdbg, s);
-  if (h->dMmaImg) return launch_rotate_quant_mma(h, X, rows, Xq, scales, Zdbg, s, qmax);
-  if (h->tc_ready) return launch_rotate_quant_tc(h, X, rows, Xq, scales, Zdbg, s, qmax);
-  if (h->tc_pair) return launch_rotate_quant_pair(h, X, rows, Xq, scales, Zdbg, s, qmax);
-  return launch_rotate_quant(h->dR1, h->dR2, h->n1, h->n2, X, rows, Xq, scales, Zdbg, s, qmax);
+                                  float* Zdbg, cudaStream_t s) {
+  if (h->st_ready) return launch_rotate_quant_st(h, X, rows, Xq, scales, Zdbg, s);
+  if (h->dMmaImg) return launch_rotate_quant_mma(h, X, rows, Xq, scales, Zdbg, s);
+  if (h->tc_ready) return launch_rotate_quant_tc(h, X, rows, Xq, scales, Zdbg, s);
+  if (h->tc_pair) return launch_rotate_quant_pair(h, X, rows, Xq, scales, Zdbg, s);
+  return launch_rotate_quant(h->dR1, h->dR2, h->n1, h->n2, X, rows, Xq, scales, Zdbg, s);
 }
 // Step 1 alone, fp16 rows out (weight-only variant): the same kernels in their rotation-only form.
 sq_status_t rotate_f16_dispatch(const sq_rotation* h, const void* X, int64_t rows, void* Z16, cudaStream_t s) {
   if (h->dMmaImg) return launch_rotate_quant_mma(h, X, rows, Z16, nullptr, nullptr, s, 0);
-  if (h->tc_ready) return launch_rotate_quant_tc(h, X, rows, Z16, nullptr, nullptr, s, 0);
-  if (h->tc_pair) return launch_rotate_quant_pair(h, X, rows, Z16, nullptr, nullptr, s, 0);
+  if (h->tc_ready) return launch_rotate_quant_tc(h, X, rows, Z16, nullptr, nullptr, s, true);
+  if (h->tc_pair) return launch_rotate_quant_pair(h, X, rows, Z16, nullptr, nullptr, s, true);
   return launch_rotate_quant(h->dR1, h->dR2, h->n1, h->n2, X, rows, Z16, nullptr, nullptr, s, 0);
 }
 }  // namespace sq
@@ -487,8 +487,13 @@ sq_status_t sq_pack_weight_wo(const sq_rotation_t* rot_or_null, const void* W, i
   const int qmax = (1 << (bits - 1)) - 1;
   if (!rot_or_null)
     st = sq::launch_rotate_quant(nullptr, nullptr, 1, static_cast<int>(K), W, N, Wq, sw, nullptr, s, qmax);
+  else if (bits == 4)
+    st = sq::rotate_quant_dispatch(rot_or_null, W, N, Wq, sw, nullptr, s);
+  else if (rot_or_null->dMmaImg)      // other widths: the kernels that take the number of levels as an argument
+    st = sq::launch_rotate_quant_mma(rot_or_null, W, N, Wq, sw, nullptr, s, qmax);
   else
-    st = sq::rotate_quant_dispatch(rot_or_null, W, N, Wq, sw, nullptr, s, qmax);
+    st = sq::launch_rotate_quant(rot_or_null->dR1, rot_or_null->dR2, rot_or_null->n1, rot_or_null->n2, W, N, Wq, sw,
+                                 nullptr, s, qmax);
   if (st != SQ_OK) return st;
   return sq::launch_interleave_nibbles(Wq, N, K, s);
 }

@@ -128,16 +128,16 @@ sq_status_t build_factors_host(const float* calib, int64_t T, int64_t n, int32_t
 sq_status_t launch_rotate_quant(const float* dR1, const float* dR2, int n1, int n2, const void* X,
                                 int64_t rows, void* Xq, void* scales, float* Zdbg, cudaStream_t s, int qmax = 7);
 
-// Tensor-core variant of steps 1+2 (sq_rotate_quant_tc.cu).  qmax as in launch_rotate_quant, also below.
+// Tensor-core variant of steps 1+2 (sq_rotate_quant_tc.cu).
 bool rotate_quant_tc_supported(int n1, int n2);
 bool rotate_quant_tc_prepare(sq_rotation* h);
 sq_status_t launch_rotate_quant_tc(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
-                                   float* Zdbg, cudaStream_t s, int qmax = 7);
+                                   float* Zdbg, cudaStream_t s, bool f16out = false);
 // Tensor-core variant for 128 < n1 <= 256 on CTA pairs (sq_rotate_quant_pair.cu).
 bool rotate_quant_pair_supported(int n1, int n2);
 bool rotate_quant_pair_prepare(sq_rotation* h);
 sq_status_t launch_rotate_quant_pair(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
-                                     float* Zdbg, cudaStream_t s, int qmax = 7);
+                                     float* Zdbg, cudaStream_t s, bool f16out = false);
 // Warp-level variant (sq_rotate_quant_mma.cu): n2 = 32.  qmax as in launch_rotate_quant.
 bool rotate_quant_mma_supported(int n1, int n2);
 bool rotate_quant_mma_prepare(sq_rotation* h);
@@ -156,7 +156,7 @@ sq_status_t launch_linear_fused(const sq_rotation* h, const void* X, int64_t M, 
                                 int64_t N, int64_t K, void* Xq, void* sx, void* Y, cudaStream_t s);
 // Picks the tensor-core kernel when the handle has its images, else the generic fp32 kernel.
 sq_status_t rotate_quant_dispatch(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
-                                  float* Zdbg, cudaStream_t s, int qmax = 7);
+                                  float* Zdbg, cudaStream_t s);
 
 // Step 1 alone with fp16 rows out (the rotation-only form of the kernels above).
 sq_status_t rotate_f16_dispatch(const sq_rotation* h, const void* X, int64_t rows, void* Z16, cudaStream_t s);
