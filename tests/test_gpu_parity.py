@@ -372,7 +372,14 @@ GEMM_SHAPES = [
 ]
 
 
-@pytest.mark.parametrize("M,N,K", GEMM_SHAPES)
+# The CTA-pair kernel's narrow form (two converter groups, two accumulators): one block, an odd k-block, fewer blocks than
+# groups and ring stages, ragged tokens and channels, several tiles per pair (both accumulators reused), both sides of the
+# line to the wide form; and the first batch size that goes to the pair kernel.
+PAIR_NARROW = [(65, 128, 128), (129, 136, 1152), (70, 264, 4096), (200, 1000, 1408), (512, 520, 4096), (333, 4096, 1024),
+               (257, 9480, 2560), (300, 9480, 2560), (130, 18952, 2304), (2048, 1280, 5120)]
+
+
+@pytest.mark.parametrize("M,N,K", GEMM_SHAPES + PAIR_NARROW)
 def test_gemm_accumulators_bit_exact(sq, M, N, K):
     rng = np.random.default_rng(M * 1000003 + N * 101 + K)
     Xc, Wc = random_codes(rng, M, K), random_codes(rng, N, K)
