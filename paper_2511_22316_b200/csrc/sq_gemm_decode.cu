@@ -15,7 +15,7 @@
 // them to its own rows, dequantises and writes fp16.  Integer addition makes the result
 // independent of any order; no partial tile, counter or scratch exists in global memory.
 //
-// Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer, warps 2..9 = two groups of weight
+// Warp roles: warp 0 = weight loads, warp 22 = token loads, warp 1 = MMA issuer, warps 2..9 = two groups of weight
 // converters and warps 10..13 = two groups of token unpackers (a group takes every other block:
 // a block costs a warp several hundred cycles of waits and fences whatever its size), warps
 // 14..21 = epilogue: all eight work on every tile, each on a quarter of the channels and half of
@@ -34,15 +34,15 @@ namespace {
 constexpr int D_CONV_GROUPS = 2;          // converter groups; group g takes the blocks g, g + 2, ...
 constexpr int D_A_WARPS = 4 * D_CONV_GROUPS, D_B_WARPS = 2 * D_CONV_GROUPS;
 constexpr int D_EPI_GROUPS = 2, D_EPI_WARPS = 4 * D_EPI_GROUPS;
-constexpr int D_THREADS = (2 + D_A_WARPS + D_B_WARPS + D_EPI_WARPS) * 32;
-constexpr int D_S_OP = 4;                // operand stages (TMEM A ring: 4 x 64 columns)
-constexpr int D_A_COL0 = 256;
+constexpr int D_EPI_WARP0 = 2 + D_A_WARPS + D_B_WARPS;
+constexpr int D_X_WARP = D_EPI_WARP0 + D_EPI_WARPS;      // the token loads have a warp of their own
+constexpr int D_THREADS = (D_X_WARP + 1) * 32;
 constexpr int D_MAX_SPLITS = 8;            // largest cluster (the portable limit)
-constexpr int D_ACCS = 4;                 // accumulators in TMEM (columns 0 .. 4 * NT)
+constexpr int D_ACCS = 4;                 // accumulators in TMEM (columns 0 .. 4 * NT - 1, the operand ring behind them)
 
 enum DecSite : uint32_t {
-  DSITE_ST_EMPTY = 64, DSITE_ST_FULL_A, DSITE_ST_FULL_B, DSITE_EMPTY_A, DSITE_EMPTY_B, DSITE_FULL,
-  DSITE_TMEM_FULL, DSITE_TMEM_EMPTY, DSITE_RED_FULL, DSITE_RED_EMPTY, DSITE_TOKENS
+  DSITE_W_EMPTY = 64, DSITE_W_FULL, DSITE_X_FULL, DSITE_EMPTY_A, DSITE_EMPTY_B, DSITE_FULL,
+  DSITE_TMEM_FULL, DSITE_TMEM_EMPTY, DSITE_RED_FULL, DSITE_RED_EMPTY, DSITE_TOKENS, DSITE_X_EMPTY
 };
 
 // Bounded wait until the counter at `flag` (device memory, bumped with release semantics by the CTAs
@@ -64,7 +64,15 @@ __device__ __forceinline__ bool wait_counter(const uint32_t* flag, uint32_t targ
 
 template <int NT>
 struct DecSmem {
-  static constexpr int S_ST = NT == 64 ? 5 : 6;      // staging stages (256 channels each); deeper rings measured no faster
+  // Stages of 256 channels: packed weights, packed tokens, int8 operands (weights in TMEM, tokens in shared memory).
+  // Weights and tokens have rings of their own: the weights come in, and are converted as far as the operand ring goes,
+  // before the tokens exist.  Deeper is not better: the weights that stream in meanwhile hold up the rotate kernel's own
+  // loads.  Layer 16 x 4096 -> 14336 with 5 / 6 / 8 / 10 stages: 10.9 / 10.7 / 10.7 / 11.2 us (12.2 with one ring of six
+  // for both); 16 x 8192 -> 28672: 29.3 / 28.4 / 27.3 / 27.7 (31.0).
+  static constexpr int S_W = NT == 64 ? 5 : 8;
+  static constexpr int S_X = NT == 64 ? 5 : 8;
+  static constexpr int S_OP = 4;
+  static constexpr int A_COL0 = D_ACCS * 64;         // first column of the operand ring, 64 a stage
   static_assert(NT == 16 || NT == 32 || NT == 64, "token-count classes");
   static constexpr int W_ST = 128 * 128;             // packed weight rows, two k-blocks
   static constexpr int X_ST = NT * 128;              // packed token rows, two k-blocks
@@ -72,12 +80,12 @@ struct DecSmem {
   // Reduce-scatter slots of one epilogue group: (s - 1) sources x 128 / s rows x NT int32, largest at s = 8.
   static constexpr int RED_GROUP = 128 * NT * 4 / D_MAX_SPLITS * (D_MAX_SPLITS - 1);
   static constexpr int OFF_X_OP = 0;
-  static constexpr int OFF_W_ST = OFF_X_OP + D_S_OP * X_OP;
-  static constexpr int OFF_X_ST = OFF_W_ST + S_ST * W_ST;
-  static constexpr int OFF_RED = OFF_X_ST + S_ST * X_ST;
+  static constexpr int OFF_W_ST = OFF_X_OP + S_OP * X_OP;
+  static constexpr int OFF_X_ST = OFF_W_ST + S_W * W_ST;
+  static constexpr int OFF_RED = OFF_X_ST + S_X * X_ST;
   static constexpr int OFF_OUT = OFF_RED + RED_GROUP;     // per epilogue warp: 16 tokens x 32 channels fp16
   static constexpr int OFF_BAR = OFF_OUT + D_EPI_WARPS * 1024;
-  static constexpr int NUM_BARS = 2 * S_ST + 2 * D_S_OP + 2 * D_ACCS + 2 * D_EPI_GROUPS + 1;
+  static constexpr int NUM_BARS = 2 * S_W + 2 * S_X + 2 * S_OP + 2 * D_ACCS + 2 * D_EPI_GROUPS + 1;
   static constexpr int OFF_MISC = (OFF_BAR + NUM_BARS * 8 + 15) / 16 * 16;   // the scales below are read as float4
   static constexpr int TOTAL = OFF_MISC + 32 + NT * 4;   // TMEM address, then the tokens' scales as floats
   static constexpr int DYN_BYTES = TOTAL + 1024;
@@ -139,16 +147,18 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
                                                       const uint32_t* tokens_ready, uint32_t tokens_target,
                                                       const DecGroups* G = nullptr) {
   using L = DecSmem<NT>;
-  constexpr int S_ST = L::S_ST;
+  constexpr int S_W = L::S_W, S_X = L::S_X, S_OP = L::S_OP;
   griddep_launch_dependents();          // a rotate kernel launched behind this one may set itself up on the idle SMs
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);
-  uint64_t* st_full = bars;
-  uint64_t* st_empty = bars + S_ST;
-  uint64_t* full = bars + 2 * S_ST;
-  uint64_t* empty = bars + 2 * S_ST + D_S_OP;
-  uint64_t* tmem_full = bars + 2 * S_ST + 2 * D_S_OP;        // [D_ACCS]
+  uint64_t* w_full = bars;                                    // [S_W]
+  uint64_t* w_empty = w_full + S_W;                           // [S_W]  a converter group has read them
+  uint64_t* x_full = w_empty + S_W;                           // [S_X]
+  uint64_t* x_empty = x_full + S_X;                           // [S_X]  an unpacker group has read them
+  uint64_t* full = x_empty + S_X;                             // [S_OP]
+  uint64_t* empty = full + S_OP;                              // [S_OP]
+  uint64_t* tmem_full = empty + S_OP;                         // [D_ACCS]
   uint64_t* tmem_empty = tmem_full + D_ACCS;                  // [D_ACCS]
   uint64_t* red_full = tmem_empty + D_ACCS;                   // the others' rows have arrived in this CTA's slots (entry 0; entry 1 unused)
   uint64_t* red_empty = red_full + D_EPI_GROUPS;              // the others have read what this CTA sent them
@@ -170,29 +180,18 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
   const int b0 = static_cast<int>(crank * static_cast<uint32_t>(num_sb) / static_cast<uint32_t>(splits));
   const int b1 = static_cast<int>((crank + 1u) * static_cast<uint32_t>(num_sb) / static_cast<uint32_t>(splits));
 
-  // The producer's walk over (tile, block); `budget` blocks are issued per call (waiting for the
-  // staging stage of each, except on the first lap of the ring, when every stage is free and the
-  // "empty" barriers may not exist yet).  The weights do not depend on the kernel before this
-  // one, the tokens do: with `defer_x` only the weights are requested and the blocks are noted.
-  int p_tile = cid, p_sb = b0, pre_n = 0;
-  int pre_sb[S_ST], pre_row[S_ST];
+  // The walk of the weight loads over (tile, block), `budget` blocks per call; on the first lap of the ring every stage is
+  // free, and the "empty" barriers may not exist yet.  The weights do not depend on the kernel before this one.
+  int p_tile = cid, p_sb = b0;
   uint32_t p_it = 0;
-  auto produce = [&](uint32_t budget, bool defer_x) -> bool {
+  auto produce_w = [&](uint32_t budget) -> bool {
     while (budget > 0 && p_tile < tiles) {
-      const int ss = p_it % S_ST;
-      if (p_it >= static_cast<uint32_t>(S_ST) &&
-          !mbar_wait(&st_empty[ss], ((p_it / S_ST) & 1) ^ 1, DSITE_ST_EMPTY, limit)) return false;
-      mbar_arrive_expect_tx(&st_full[ss], L::W_ST + L::X_ST);
-      const int pg = GROUPED ? p_tile / tiles_pe : 0;                  // expert of the tile
-      const int xrow = GROUPED ? G->r0[pg] : 0;                        // its first token row
-      tma_load_2d(smem + L::OFF_W_ST + ss * L::W_ST, GROUPED ? &G->wmap[pg] : &tmap_w, &st_full[ss], p_sb * 128,
+      const int ss = p_it % S_W;
+      if (p_it >= static_cast<uint32_t>(S_W) &&
+          !mbar_wait(&w_empty[ss], ((p_it / S_W) & 1) ^ 1, DSITE_W_EMPTY, limit)) return false;
+      mbar_arrive_expect_tx(&w_full[ss], L::W_ST);
+      tma_load_2d(smem + L::OFF_W_ST + ss * L::W_ST, GROUPED ? &G->wmap[p_tile / tiles_pe] : &tmap_w, &w_full[ss], p_sb * 128,
                   (GROUPED ? p_tile % tiles_pe : p_tile) * 128);
-      if (defer_x) {
-        pre_sb[pre_n] = p_sb;
-        pre_row[pre_n++] = xrow;
-      } else {
-        tma_load_2d(smem + L::OFF_X_ST + ss * L::X_ST, &tmap_x, &st_full[ss], p_sb * 128, xrow);
-      }
       ++p_it;
       --budget;
       if (++p_sb >= b1) {
@@ -205,12 +204,16 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
 
   if (threadIdx.x == 0) {
     // First of all the weights of the whole staging ring: nothing else is on the critical path.
-    for (int s = 0; s < S_ST; ++s) mbar_init(&st_full[s], 1);
+    for (int s = 0; s < S_W; ++s) mbar_init(&w_full[s], 1);
     mbar_fence_init();
-    produce(S_ST, true);
+    produce_w(S_W);
     tma_prefetch_desc(&tmap_x);
-    for (int s = 0; s < S_ST; ++s) mbar_init(&st_empty[s], 6);   // one converter group + one unpacker group
-    for (int s = 0; s < D_S_OP; ++s) {
+    for (int s = 0; s < S_W; ++s) mbar_init(&w_empty[s], 4);     // one converter group
+    for (int s = 0; s < S_X; ++s) {
+      mbar_init(&x_full[s], 1);
+      mbar_init(&x_empty[s], 2);                                 // one unpacker group
+    }
+    for (int s = 0; s < S_OP; ++s) {
       mbar_init(&full[s], 6);
       mbar_init(&empty[s], 1);
     }
@@ -239,17 +242,29 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
   if (splits > 1) cluster_arrive_release();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  if (tokens_ready == nullptr) griddep_wait();         // the tokens and their scales come from the kernel before
 
   if (warp == 0) {
-    // ------------------------------ TMA producer ------------------------------------------------
-    // In the fused form this one thread polls the counter of the token-producing CTAs for the whole
-    // CTA; the epilogue warps, which read the token steps, wait for its arrival on a local barrier.
+    // ------------------------------ weight loads ------------------------------------------------
+    if (lane == 0) produce_w(0xFFFFFFFFu);
+  } else if (warp == D_X_WARP) {
+    // ------------------------------ token loads -------------------------------------------------
+    // The tokens come from the kernel before this one; in the fused form this one thread polls the counter of the CTAs
+    // that make them, and the epilogue warps, which read the token steps, wait for its arrival on a local barrier.
+    if (tokens_ready == nullptr) griddep_wait();
     if (lane == 0 && (tokens_ready == nullptr || wait_counter(tokens_ready, tokens_target, DSITE_TOKENS, limit))) {
       if (tokens_ready != nullptr) mbar_arrive(tok_seen);
-      for (int i = 0; i < pre_n; ++i)
-        tma_load_2d(smem + L::OFF_X_ST + i * L::X_ST, &tmap_x, &st_full[i], pre_sb[i] * 128, pre_row[i]);
-      produce(0xFFFFFFFFu, false);
+      uint32_t it = 0;
+      bool ok = true;
+      for (int tile = cid; tile < tiles && ok; tile += ncl) {
+        const int xrow = GROUPED ? G->r0[tile / tiles_pe] : 0;         // the expert's first token row
+        for (int sb = b0; sb < b1; ++sb, ++it) {
+          const int ss = it % S_X;
+          ok = mbar_wait(&x_empty[ss], ((it / S_X) & 1) ^ 1, DSITE_X_EMPTY, limit);
+          if (!ok) break;
+          mbar_arrive_expect_tx(&x_full[ss], L::X_ST);
+          tma_load_2d(smem + L::OFF_X_ST + ss * L::X_ST, &tmap_x, &x_full[ss], sb * 128, xrow);
+        }
+      }
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer --------------------------------------------------
@@ -269,11 +284,11 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * NT;
         for (int sb = b0; sb < b1; ++sb, ++it) {
-          const uint32_t s = it % D_S_OP;
-          ok = mbar_wait(&full[s], (it / D_S_OP) & 1, DSITE_FULL, limit);
+          const uint32_t s = it % S_OP;
+          ok = mbar_wait(&full[s], (it / S_OP) & 1, DSITE_FULL, limit);
           if (!ok) break;
           tc_fence_after_sync();
-          const uint32_t a_tmem = tmem_base + D_A_COL0 + s * 64;
+          const uint32_t a_tmem = tmem_base + L::A_COL0 + s * 64;
           const uint64_t bd = b_desc0 + static_cast<uint64_t>(s * (L::X_OP >> 4));
           umma_i8_ts(d_tmem, a_tmem, bd, idesc, sb > b0 ? 1u : 0u);
           umma_i8_ts(d_tmem, a_tmem + 8, bd + 2, idesc, 1u);
@@ -301,15 +316,15 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
     for (int tile = cid; tile < tiles && ok; tile += ncl) {
       for (int sb = b0; sb < b1 && ok; ++sb, ++it) {
         if ((it % D_CONV_GROUPS) != static_cast<uint32_t>(grp)) continue;
-        const int ss = it % S_ST, s = it % D_S_OP;
-        ok = mbar_wait(&st_full[ss], (it / S_ST) & 1, DSITE_ST_FULL_A, limit);
+        const int ss = it % S_W, s = it % S_OP;
+        ok = mbar_wait(&w_full[ss], (it / S_W) & 1, DSITE_W_FULL, limit);
         if (!ok) break;
         const unsigned char* row = smem + L::OFF_W_ST + ss * L::W_ST + r * 128;
         const int nh = (2 * sb + 1 < num_kb) ? 2 : 1;
         uint4 w[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) w[c] = *reinterpret_cast<const uint4*>(row + ((c ^ (r & 7)) << 4));
-        ok = mbar_wait(&empty[s], ((it / D_S_OP) & 1) ^ 1, DSITE_EMPTY_A, limit);
+        ok = mbar_wait(&empty[s], ((it / S_OP) & 1) ^ 1, DSITE_EMPTY_A, limit);
         if (!ok) break;
         tc_fence_after_sync();
 #pragma unroll
@@ -324,7 +339,7 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
               v[4 * j + 2] = (x.z << 4) & 0xF0F0F0F0u; v[16 + 4 * j + 2] = x.z & 0xF0F0F0F0u;
               v[4 * j + 3] = (x.w << 4) & 0xF0F0F0F0u; v[16 + 4 * j + 3] = x.w & 0xF0F0F0F0u;
             }
-            tmem_st_32x32b_x32(tmem_base + lane_addr + D_A_COL0 + s * 64 + h * 32, v);
+            tmem_st_32x32b_x32(tmem_base + lane_addr + L::A_COL0 + s * 64 + h * 32, v);
           }
         }
         tmem_wait_st();
@@ -332,11 +347,11 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(&full[s]);
-          mbar_arrive(&st_empty[ss]);
+          mbar_arrive(&w_empty[ss]);
         }
       }
     }
-  } else if (warp < 2 + D_A_WARPS + D_B_WARPS) {
+  } else if (warp < D_EPI_WARP0) {
     // ------------------------------ token unpackers: staging -> operand ring ----------------------
     const int grp = (warp - (2 + D_A_WARPS)) >> 1;
     const int t = (threadIdx.x - (2 + D_A_WARPS) * 32) & 63;
@@ -345,16 +360,16 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
     for (int tile = cid; tile < tiles && ok; tile += ncl) {
       for (int sb = b0; sb < b1 && ok; ++sb, ++it) {
         if ((it % D_CONV_GROUPS) != static_cast<uint32_t>(grp)) continue;
-        const int ss = it % S_ST, s = it % D_S_OP;
-        ok = mbar_wait(&st_full[ss], (it / S_ST) & 1, DSITE_ST_FULL_B, limit) &&
-             mbar_wait(&empty[s], ((it / D_S_OP) & 1) ^ 1, DSITE_EMPTY_B, limit);
+        const int ss = it % S_X, s = it % S_OP;
+        ok = mbar_wait(&x_full[ss], (it / S_X) & 1, DSITE_X_FULL, limit) &&
+             mbar_wait(&empty[s], ((it / S_OP) & 1) ^ 1, DSITE_EMPTY_B, limit);
         if (!ok) break;
         unpack_rows<NT>(smem + L::OFF_X_ST + ss * L::X_ST, smem + L::OFF_X_OP + s * L::X_OP, t, 2 * sb + 1 < num_kb);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(&full[s]);
-          mbar_arrive(&st_empty[ss]);
+          mbar_arrive(&x_empty[ss]);
         }
       }
     }
@@ -363,11 +378,12 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
     // Eight warps share every tile: warp q of group eg reads the TMEM lanes 32 q .. 32 q + 31 (all a
     // warp may touch) of the columns [eg * NT / 2, (eg + 1) * NT / 2) -- a single warp per scheduler
     // is bound by its own instruction issue, so the columns are spread over as many as there are.
+    if (tokens_ready == nullptr) griddep_wait();                     // the token steps come from the kernel before, which may still read Y
     constexpr int HALF = NT / 2;                                     // columns (tokens) per group
     constexpr int CH = HALF >= 16 ? 16 : 8;                          // columns per TMEM load
     const int q = warp & 3;
-    const int eg = (warp - (2 + D_A_WARPS + D_B_WARPS)) >> 2;
-    const int et = static_cast<int>(threadIdx.x) - (2 + D_A_WARPS + D_B_WARPS) * 32;   // 0 .. 255
+    const int eg = (warp - D_EPI_WARP0) >> 2;
+    const int et = static_cast<int>(threadIdx.x) - D_EPI_WARP0 * 32;   // 0 .. 255
     const int rowl = q * 32 + lane;                                  // row of the tile = TMEM lane
     // Reduce-scatter geometry: CTA `owner` finishes this thread's row; this CTA finishes the rows
     // [crank * rows_per, (crank + 1) * rows_per).  Slots are [source][4-column chunk][row][4] int32:
@@ -386,7 +402,7 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
     // its registers, Y has the channels contiguous.  A chunk of CH tokens x 32 channels is turned in
     // shared memory -- written as words of two tokens, [token pair][channel] -- so that a thread
     // stores 8 channels (16 bytes) of one token.
-    uint32_t* outw = reinterpret_cast<uint32_t*>(smem + L::OFF_OUT + (warp - (2 + D_A_WARPS + D_B_WARPS)) * 1024);
+    uint32_t* outw = reinterpret_cast<uint32_t*>(smem + L::OFF_OUT + (warp - D_EPI_WARP0) * 1024);
     const int piece = lane & 3, prow = lane >> 2;                    // reader: channels 8 * piece .., token prow (+ 8)
     const bool piece_mine = static_cast<uint32_t>((q * 32 + piece * 8) / rows_per) == crank;
     const uint32_t pick = (prow & 1) ? 0x7632u : 0x5410u;            // the odd or the even token of a pair
@@ -548,7 +564,7 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
   if (splits > 1) {
     // Nobody leaves while another CTA may still store or arrive here.  No memory is ordered by
     // this barrier: what crossed CTAs was handed over by the red_* barriers.
-    if (warp < 2 + D_A_WARPS + D_B_WARPS) cluster_wait_acquire();      // the set-up barrier, long complete
+    if (warp < D_EPI_WARP0 || warp == D_X_WARP) cluster_wait_acquire();        // the set-up barrier, long complete
     cluster_arrive_relaxed();
     cluster_wait_acquire();
   }

@@ -92,9 +92,9 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
   static_assert(NTT % 2 == 0, "whole k-steps");
   constexpr int B1_BYTES = KJ * NTT * 512, A2_BYTES = RM_SLICES * RM_A2_SLICE;
   constexpr int T_BYTES = PW > 1 ? RM_SLICES * 2 * KJ * 512 : 0;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  uint4* b1s = reinterpret_cast<uint4*>(smem_raw);
-  unsigned char* a2s = smem_raw + B1_BYTES;
+  extern __shared__ __align__(128) unsigned char rm_smem_raw[];
+  uint4* b1s = reinterpret_cast<uint4*>(rm_smem_raw);
+  unsigned char* a2s = rm_smem_raw + B1_BYTES;
   uint2* ts = reinterpret_cast<uint2*>(a2s + A2_BYTES);                    // [slice][hi, lo][k-step][half][lane]
   float* zmax = reinterpret_cast<float*>(a2s + A2_BYTES + T_BYTES);        // [2][WARPS]: of the token
   float* tmax = zmax + 16;                                                 // [WARPS]: of T (PW > 1)
@@ -112,7 +112,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
     mbar_arrive_expect_tx(bar, B1_BYTES + A2_BYTES);
     bulk_load_1d(a2s, a2_img, A2_BYTES, bar);
     for (int o = 0; o < B1_BYTES; o += 16384)
-      bulk_load_1d(smem_raw + o, reinterpret_cast<const unsigned char*>(b1_img) + o,
+      bulk_load_1d(rm_smem_raw + o, reinterpret_cast<const unsigned char*>(b1_img) + o,
                    static_cast<uint32_t>(B1_BYTES - o < 16384 ? B1_BYTES - o : 16384), bar);
   }
   griddep_wait();
