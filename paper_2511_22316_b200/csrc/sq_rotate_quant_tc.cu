@@ -50,10 +50,11 @@ struct RqLayout {
   int off_a1, off_b2, off_x, off_misc, total;
 };
 
-__host__ __device__ inline RqLayout rq_layout(int n1, int n2, int budget = kMaxDynSmem) {
+// `one_token`: one token per accumulator (the other lanes stay zero) instead of as many as fit.
+__host__ __device__ inline RqLayout rq_layout(int n1, int n2, int budget = kMaxDynSmem, bool one_token = false) {
   RqLayout L;
   L.LS = n1 <= 32 ? 32 : (n1 <= 64 ? 64 : 128);   // TMEM lanes per token
-  L.G = 128 / L.LS;                               // tokens per accumulator
+  L.G = one_token ? 1 : 128 / L.LS;               // tokens per accumulator
   L.N1 = (n1 + 15) & ~15;                         // K of stage 1, padded to the MMA's K = 16
   L.KA1 = (L.N1 + 63) / 64;                       // 64-wide K atoms of stage 1
   L.XQ = n2 / 64;                                 // 64-wide column blocks of a token
@@ -363,7 +364,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       tc_fence_after_sync();
       if constexpr (F16OUT) {
         // rotation only: the rotated row leaves as fp16 (weight-only variant), nothing is quantised
-        const bool live16 = (pp < n1) && (token < rows);
+        const bool live16 = (pp < n1) && (tk < G) && (token < rows);
         __half* zrow16 = reinterpret_cast<__half*>(Xq) + token * n + pp * N2 + cp * HC;
 #pragma unroll
         for (int c = 0; c < HC / 16; ++c) {
@@ -408,7 +409,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       float inv;
       row_scale(amax, delta, inv);
       const float inv_un = inv * un;
-      const bool live = (pp < n1) && (token < rows);
+      const bool live = (pp < n1) && (tk < G) && (token < rows);
       const bool clamp = __half2float(delta) < 6.103515625e-05f;
       uint8_t* orow = Xq + token * (n / 2) + pp * (N2 / 2) + cp * (HC / 2);
       float* zrow = (Zdbg != nullptr && live) ? Zdbg + token * n + pp * N2 + cp * HC : nullptr;
@@ -504,7 +505,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       tc_fence_after_sync();
       if constexpr (F16OUT) {
         // rotation only: the rotated row leaves as fp16 (weight-only variant), nothing is quantised
-        const bool live16 = (pp < n1) && (token < rows);
+        const bool live16 = (pp < n1) && (tk < G) && (token < rows);
         __half* zrow16 = reinterpret_cast<__half*>(Xq) + token * n + pp * N2;
 #pragma unroll
         for (int c = 0; c < N2 / 32; ++c) {
@@ -543,7 +544,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       float inv;
       row_scale(amax, delta, inv);
       const float inv_un = inv * un;                 // exact: un is a power of two
-      const bool live = (pp < n1) && (token < rows);
+      const bool live = (pp < n1) && (tk < G) && (token < rows);
       // Delta >= 2^-14 (a normal fp16) bounds |z / Delta| by 7 (1 + 2^-11): no clamp is needed then.
       const bool clamp = __half2float(delta) < 6.103515625e-05f;
       uint8_t* orow = Xq + token * (n / 2) + pp * (N2 / 2);
@@ -590,7 +591,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
 // S accumulator slots (= compute groups) per CTA.  With S * 2 * N2 = 256 TMEM columns two CTAs share
 // an SM (each with its own producer and MMA issuer); with 512 a CTA has the SM to itself.
 template <int N2, int S, int CW = 1, bool F16OUT = false>
-__global__ void __launch_bounds__((2 + 4 * S * CW) * 32, (S * 2 * N2 <= 256) ? 2 : 1)
+__global__ void __launch_bounds__((2 + 4 * S * CW) * 32, (CW == 1 && S * 2 * N2 <= 256) ? 2 : 1)
 rotate_quant_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ RqLayout L,
                        const unsigned char* __restrict__ a1_img, const unsigned char* __restrict__ b2_img, int n1,
                        int rows, uint8_t* __restrict__ Xq, __half* __restrict__ scales, float* __restrict__ Zdbg) {
@@ -662,7 +663,13 @@ sq_status_t launch_rotate_quant_tc(const sq_rotation* h, const void* X, int64_t 
   // n2 = 64 with images small enough: two CTAs per SM, two accumulator slots each.
   const RqLayout Lh = rq_layout(n1, n2, kHalfDynSmem);
   const bool dual = (n2 == 64) && Lh.XS >= 2;
-  const RqLayout L = dual ? Lh : rq_layout(n1, n2);
+  // A handful of tokens: latency is all there is.  One token per accumulator (a group's stage 1 is half or a quarter as
+  // long) and eight warps on it also with n2 = 64; the sums are the same, in the same order.  Not beyond 32 tokens: every
+  // CTA here keeps one of the product's off its SM.  16 x 4096 (64 x 64): 4.57 -> 3.86 us, layer to 14336 11.5 -> 10.7.
+  // The quantising form asks for an SM of its own (120 KB: the layer for one token 11.1 us without, 9.9 with), the fp16
+  // form does not (18.4 without, 25 with: the dot-product kernel behind it then doubles up on another SM).
+  const bool few = rows <= 32;
+  const RqLayout L = few ? rq_layout(n1, n2, kMaxDynSmem, true) : (dual ? Lh : rq_layout(n1, n2));
   EncodeTiledFn enc = get_encode_fn();
   if (!enc) return SQ_ERR_CUDA;
   CUtensorMap mx;
@@ -692,7 +699,10 @@ sq_status_t launch_rotate_quant_tc(const sq_rotation* h, const void* X, int64_t 
   // n2 = 128 (one CTA per SM, two slots): eight warps per slot, 18 in all instead of 10 -- measured 10 %
   // faster on 4096 x 8192 (39.7 -> 35.5 us) and 0.8 us on the decode batches (6.6 -> 5.8 us).  With n2 = 64
   // and two CTAs per SM the same split leaves 56 registers per thread and was slower (12.0 -> 15.9 us).
-  if (f16out) {
+  if (few) {
+    if (f16out) ok = n2 == 64 ? launch(rotate_quant_tc_kernel<64, 1, 2, true>, 1, 2, 2) : launch(rotate_quant_tc_kernel<128, 1, 2, true>, 1, 2, 2);
+    else ok = n2 == 64 ? launch(rotate_quant_tc_kernel<64, 1, 2>, 1, 1, 2) : launch(rotate_quant_tc_kernel<128, 1, 2>, 1, 1, 2);
+  } else if (f16out) {
     // rotation only: Xq receives the rotated rows as fp16 [rows x n], `scales` is not touched
     if (n2 == 64 && dual) ok = launch(rotate_quant_tc_kernel<64, 2, 1, true>, 2, 2);
     else if (n2 == 64) ok = launch(rotate_quant_tc_kernel<64, 4, 1, true>, 4, 1);
