@@ -440,13 +440,17 @@ w4a4_gemm_pair_grouped_kernel(const __grid_constant__ PairGroups G, const __grid
   w4a4_gemm_pair_body<L, true>(tmap_x, G.wmap[0], G.ymap[0], sx, nullptr, 0, N, K, nullptr, &G);
 }
 
-// Estimated time in microseconds of `tiles` tiles of `num_sb` 256-channel blocks on `pairs` CTA pairs.  Measured: a wave of
-// wide tiles takes 0.75 a block and a launch 2.4 more, a wave of narrow ones 0.40 and 5.1 (333 x 4096 x 4096, one wave of
-// either: 14.4 wide, 11.2 narrow; 2048 x 4096 x 4096, two waves against four: 26.4 and 28.7; 333 x 11008 x 4096, two
-// against three: 25.6 and 22.8; 200 x 4096 x 11008, one of either: 29.5 and 19.6).
-double pair_estimate_us(long long tiles, int num_sb, int pairs, bool narrow) {
-  const long long waves = (tiles + pairs - 1) / pairs;
-  return static_cast<double>(waves) * num_sb * (narrow ? 0.40 : 0.75) + (narrow ? 5.1 : 2.4);
+// Whether the narrow form is the faster one for so many tiles of `num_sb` 256-channel blocks on `pairs` CTA pairs.  Fit to
+// both forms on 72 shapes (100 to 1400 tokens, the layer shapes of the configurations): a wave of wide tiles takes
+// 0.57 us a block + 1.8, a launch 3.5 more; a wave of narrow ones 0.34 a block + 0.6, a launch 5.5 (one wave of either, 16
+// blocks: 14.4 and 11.2 us measured, 112 blocks: 70.3 and 48.7; 300 x 11008 x 4096, two waves against three: 25.6 and 22.5;
+// 300 x 28672 x 8192, four against seven: 83.9 and 88.8).  The wide form moves the tokens half as often, which a chip full
+// of tiles repays: the narrow one has to promise five per cent.
+bool pair_prefers_narrow(long long wide_tiles, long long narrow_tiles, int num_sb, int pairs) {
+  const long long ww = (wide_tiles + pairs - 1) / pairs, wn = (narrow_tiles + pairs - 1) / pairs;
+  const double wide = static_cast<double>(ww) * (0.57 * num_sb + 1.8) + 3.5;
+  const double narrow = static_cast<double>(wn) * (0.34 * num_sb + 0.6) + 5.5;
+  return narrow < 0.95 * wide;
 }
 template <class L>
 long long pair_tiles(int64_t rows, int64_t N) {
@@ -524,8 +528,7 @@ sq_status_t launch_w4a4_gemm_pair_grouped(const void* Xq, const void* sx, int64_
     wide += pair_tiles<PairWide>(rows[g], N);
     narrow += pair_tiles<PairNarrow>(rows[g], N);
   }
-  const int sb = pair_blocks(K);
-  if (pair_estimate_us(narrow, sb, sms / 2, true) < pair_estimate_us(wide, sb, sms / 2, false))
+  if (pair_prefers_narrow(wide, narrow, pair_blocks(K), sms / 2))
     return launch_pair_grouped<PairNarrow>(Xq, sx, M_total, count, Wq, sw, r0, rows, N, K, Y, s, sms);
   return launch_pair_grouped<PairWide>(Xq, sx, M_total, count, Wq, sw, r0, rows, N, K, Y, s, sms);
 }
@@ -540,9 +543,7 @@ sq_status_t launch_w4a4_gemm_pair(const void* Xq, const void* sx, const void* Wq
                                   int K, void* Y, int32_t* accdbg, cudaStream_t s) {
   const int sms = sm_count();
   if (sms <= 0) return SQ_ERR_CUDA;
-  const int sb = pair_blocks(K);
-  if (pair_estimate_us(pair_tiles<PairNarrow>(M, N), sb, sms / 2, true) <
-      pair_estimate_us(pair_tiles<PairWide>(M, N), sb, sms / 2, false))
+  if (pair_prefers_narrow(pair_tiles<PairWide>(M, N), pair_tiles<PairNarrow>(M, N), pair_blocks(K), sms / 2))
     return launch_pair<PairNarrow>(Xq, sx, Wq, sw, M, N, K, Y, accdbg, s, sms);
   return launch_pair<PairWide>(Xq, sx, Wq, sw, M, N, K, Y, accdbg, s, sms);
 }

@@ -372,11 +372,11 @@ GEMM_SHAPES = [
 ]
 
 
-# The CTA-pair kernel's narrow form (two converter groups, two accumulators): one block, an odd k-block, fewer blocks than
-# groups and ring stages, ragged tokens and channels, several tiles per pair (both accumulators reused), both sides of the
-# line to the wide form; and the first batch size that goes to the pair kernel.
-PAIR_NARROW = [(65, 128, 128), (129, 136, 1152), (70, 264, 4096), (200, 1000, 1408), (512, 520, 4096), (333, 4096, 1024),
-               (257, 9480, 2560), (300, 9480, 2560), (130, 18952, 2304), (2048, 1280, 5120)]
+# The CTA-pair kernel's narrow form (two converter groups, two accumulators): the shortest K that takes it, an odd k-block,
+# ragged tokens and channels, several tiles per pair (both accumulators reused); the first batch size that goes to the pair
+# kernel, in either form; shapes beside the line that stay wide.
+PAIR_NARROW = [(65, 128, 1408), (129, 136, 1664), (70, 264, 4096), (200, 1000, 1408), (512, 520, 4096), (257, 9480, 2560),
+               (300, 9480, 2560), (130, 18952, 2304), (65, 128, 128), (129, 136, 1152), (333, 4096, 1024), (2048, 1280, 5120)]
 
 
 @pytest.mark.parametrize("M,N,K", GEMM_SHAPES + PAIR_NARROW)
