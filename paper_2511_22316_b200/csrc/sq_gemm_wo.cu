@@ -318,7 +318,8 @@ wo_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_const
 // channels.
 constexpr int WOD_CONV_GROUPS = 2;
 constexpr int WOD_CONV_WARPS = 4 * WOD_CONV_GROUPS;
-constexpr int WOD_THREADS = (2 + WOD_CONV_WARPS + WO_EPI_WARPS) * 32;
+constexpr int WOD_T_WARP = 2 + WOD_CONV_WARPS + WO_EPI_WARPS;      // the token loads have a warp of their own
+constexpr int WOD_THREADS = (WOD_T_WARP + 1) * 32;
 constexpr int WOD_A_STAGES = 2;           // tensor-memory operand stages of 128 columns (256 fp16 channels)
 // accumulators: columns [0, 2 NT); operand ring: two stages of 128 columns from column max(128, 2 NT) on
 
@@ -424,35 +425,40 @@ wo_gemm_tmem_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  griddep_wait();                                     // Z16 may come from the kernel launched before this one
 
   if (warp == 0) {
-    // ------------------------------ TMA producer ------------------------------------------
+    // ------------------------------ weight loads ------------------------------------------
     if (lane == 0) {
       uint32_t sit = 0;
       bool ok = true;
       for (int tile = cid; tile < num_tiles && ok; tile += ncl) {
-        for (int sb = sb0; sb < sb1 && ok; ++sb) {
-          for (int half = 0; half < CT && ok; ++half, ++sit) {
-            if (sit >= static_cast<uint32_t>(pre)) {        // the first `pre` blocks are on their way already
-              const int ss = sit % SS;
-              ok = mbar_wait(&st_empty[ss], ((sit / SS) & 1) ^ 1, WO_ST_EMPTY, limit);
-              if (!ok) break;
-              mbar_arrive_expect_tx(&st_full[ss], L::W_ST);
-              tma_load_2d(smem + L::OFF_W_ST + ss * L::W_ST, &tmap_w, &st_full[ss], sb * 128,
-                          ((tile % tiles_n) * CT + half) * 128);
-            }
-            if (half != 0) continue;                        // the token block serves both channel tiles
-            const uint32_t tit = sit / CT;
-            const int st = tit % ST;
-            const int nk = (num_kb - 4 * sb) < 4 ? (num_kb - 4 * sb) : 4;
-            ok = mbar_wait(&t_empty[st], ((tit / ST) & 1) ^ 1, WO_A_EMPTY, limit);
-            if (!ok) break;
-            mbar_arrive_expect_tx(&t_full[st], static_cast<uint32_t>(nk * L::T_KB));
-            for (int h = 0; h < nk; ++h)
-              tma_load_2d(smem + L::OFF_T + st * L::T_TILE + h * L::T_KB, &tmap_z, &t_full[st], (4 * sb + h) * 64,
-                          (tile / tiles_n) * NT);
-          }
+        for (int sbh = sb0 * CT; sbh < sb1 * CT; ++sbh, ++sit) {
+          if (sit < static_cast<uint32_t>(pre)) continue;   // on its way already
+          const int ss = sit % SS;
+          ok = mbar_wait(&st_empty[ss], ((sit / SS) & 1) ^ 1, WO_ST_EMPTY, limit);
+          if (!ok) break;
+          mbar_arrive_expect_tx(&st_full[ss], L::W_ST);
+          tma_load_2d(smem + L::OFF_W_ST + ss * L::W_ST, &tmap_w, &st_full[ss], (sbh / CT) * 128,
+                      ((tile % tiles_n) * CT + sbh % CT) * 128);
+        }
+      }
+    }
+  } else if (warp == WOD_T_WARP) {
+    // ------------------------------ token loads: a block serves all channel tiles of its token tile -------
+    griddep_wait();                                     // Z16 may come from the kernel launched before this one
+    if (lane == 0) {
+      uint32_t tit = 0;
+      bool ok = true;
+      for (int tile = cid; tile < num_tiles && ok; tile += ncl) {
+        for (int sb = sb0; sb < sb1; ++sb, ++tit) {
+          const int st = tit % ST;
+          const int nk = (num_kb - 4 * sb) < 4 ? (num_kb - 4 * sb) : 4;
+          ok = mbar_wait(&t_empty[st], ((tit / ST) & 1) ^ 1, WO_A_EMPTY, limit);
+          if (!ok) break;
+          mbar_arrive_expect_tx(&t_full[st], static_cast<uint32_t>(nk * L::T_KB));
+          for (int h = 0; h < nk; ++h)
+            tma_load_2d(smem + L::OFF_T + st * L::T_TILE + h * L::T_KB, &tmap_z, &t_full[st], (4 * sb + h) * 64,
+                        (tile / tiles_n) * NT);
         }
       }
     }
@@ -554,6 +560,7 @@ wo_gemm_tmem_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
     }
   } else {
     // ------------------------------ epilogue warps ------------------------------------------
+    griddep_wait();                                     // the kernel before this one may still read Y
     const int quarter = warp & 3;
     uint32_t tcount = 0;
     bool ok = true;
@@ -616,7 +623,7 @@ wo_gemm_tmem_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
     // Every thread of every CTA of the cluster comes through here, whatever happened above: the two
     // barriers are hardware barriers, not polled waits.
     cluster_sync_all();                                 // the partial tiles are in place
-    if (crank == 0 && warp >= 2 + WOD_CONV_WARPS && cid < num_tiles) {
+    if (crank == 0 && warp >= 2 + WOD_CONV_WARPS && warp < WOD_T_WARP && cid < num_tiles) {
       tc_fence_after_sync();
       const int quarter = warp & 3;
       const int ch = (cid % tiles_n) * 128 + quarter * 32 + lane;                          // CT = 1 here
@@ -670,15 +677,16 @@ wo_gemm_tmem_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
 // operand ring needs the other 256 columns; eight epilogue warps (two per lane quarter, 128 columns
 // each) hand it back after their last read.  The tile's token width is the host's choice (wo_pair_tile_m); 256 above
 // stands for the widest.
-//   warp 0        TMA: packed weights of this CTA's channels (staging ring), this CTA's tokens (ring
-//                 stage s = four 64-channel k-blocks)
+//   warp 0        TMA: packed weights of this CTA's channels (staging ring)
+//   warp 18       TMA: this CTA's tokens (ring stage s = four 64-channel k-blocks)
 //   warps 2..9    two converter groups, alternating stages: staging -> registers -> tensor-memory ring
 //                 stage s; a warp reports the stage to the leader once its part is stored AND this
 //                 CTA's tokens of the stage have landed
 //   warp 1        (leader CTA) sixteen MMAs per stage; the commit frees stage s in both CTAs
 //   warps 10..17  epilogue: tensor memory -> scale -> fp16 stores
 constexpr int WP_EPI_WARPS = 8;
-constexpr int WP_THREADS = (2 + WOD_CONV_WARPS + WP_EPI_WARPS) * 32;
+constexpr int WP_T_WARP = 2 + WOD_CONV_WARPS + WP_EPI_WARPS;       // the token loads have a warp of their own
+constexpr int WP_THREADS = (WP_T_WARP + 1) * 32;
 constexpr int WP_S = 2;                  // ring stages: 256 channels of K (tokens in shared, weights in tensor memory)
 constexpr int WP_A_COL0 = 256;           // first column of the operand ring (0..255: accumulator)
 static_assert(WP_S == WOD_CONV_GROUPS, "a converter group owns one ring stage");
@@ -769,24 +777,33 @@ wo_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
   cluster_sync_all();                                 // both CTAs' barriers exist before any remote arrival
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  griddep_wait();                                     // Z16 may come from the kernel launched before this one
 
   if (warp == 0) {
-    // ------------------------------ TMA producer ------------------------------------------
+    // ------------------------------ weight loads ------------------------------------------
     if (lane == 0) {                                  // thread 0: it knows how many blocks are on their way
       uint32_t it = 0;
       bool ok = true;
       for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
         const int ch0 = (tile % tiles_n) * 256 + static_cast<int>(rank) * 128;
+        for (int sb = 0; sb < num_sb; ++sb, ++it) {
+          if (it < static_cast<uint32_t>(pre)) continue;
+          const int ss = it % SS;
+          ok = mbar_wait(&st_empty[ss], ((it / SS) & 1) ^ 1, WP_ST_EMPTY, limit);
+          if (!ok) break;
+          mbar_arrive_expect_tx(&st_full[ss], L::W_ST);
+          tma_load_2d(smem + L::OFF_W_ST + ss * L::W_ST, &tmap_w, &st_full[ss], sb * 128, ch0);
+        }
+      }
+    }
+  } else if (warp == WP_T_WARP) {
+    // ------------------------------ token loads -------------------------------------------
+    griddep_wait();                                   // Z16 may come from the kernel launched before this one
+    if (lane == 0) {
+      uint32_t it = 0;
+      bool ok = true;
+      for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
         const int tok0 = (tile / tiles_n) * tile_m + static_cast<int>(rank) * (tile_m / 2);
-        for (int sb = 0; sb < num_sb && ok; ++sb, ++it) {
-          if (it >= static_cast<uint32_t>(pre)) {
-            const int ss = it % SS;
-            ok = mbar_wait(&st_empty[ss], ((it / SS) & 1) ^ 1, WP_ST_EMPTY, limit);
-            if (!ok) break;
-            mbar_arrive_expect_tx(&st_full[ss], L::W_ST);
-            tma_load_2d(smem + L::OFF_W_ST + ss * L::W_ST, &tmap_w, &st_full[ss], sb * 128, ch0);
-          }
+        for (int sb = 0; sb < num_sb; ++sb, ++it) {
           const int s = it % WP_S;
           const int nk = (num_kb - 4 * sb) < 4 ? (num_kb - 4 * sb) : 4;
           ok = mbar_wait(&empty[s], ((it / WP_S) & 1) ^ 1, WP_EMPTY_T, limit);
@@ -886,6 +903,7 @@ wo_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
     }
   } else {
     // ------------------------------ epilogue warps ------------------------------------------
+    griddep_wait();                                     // the kernel before this one may still read Y
     const int q = warp & 3;                             // TMEM lane quarter this warp may read
     // its part of the token columns, in chunks of 16: the first half (rounded up) or the rest
     const int half = (warp - (2 + WOD_CONV_WARPS)) >> 2;
