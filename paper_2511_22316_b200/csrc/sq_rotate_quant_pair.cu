@@ -230,201 +230,38 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
         }
       }
     }
-  } else if (CW == 2) {
-    // ------------------------------ compute groups, two warps per lane quarter ---------------------
-    // Eight warps per accumulator slot: warp (quarter, cp) owns columns [cp * N2/2, (cp+1) * N2/2) of its
-    // lane quarter, 16 at a time; the lane's scale is the larger of the two halves' (swapped through
-    // shared memory behind the group barrier, which also orders the reads of D1 before its overwrite).
-    constexpr int HC = N2 / 2;
-    const int gi = (warp - 2) >> 2;
-    const int w = gi >> 1, cp = gi & 1;
-    const int quarter = warp & 3;
-    const int lane_g = quarter * 32 + lane;
-    const int pp = static_cast<int>(rank) * 128 + lane_g;
-    const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
-    const uint32_t d1 = tmem_base + w * SLOT_COLS + lane_addr + cp * HC, d2 = d1 + N2;
-    const bool live = pp < n1;
-    float* lane_m = reinterpret_cast<float*>(smem + L.off_misc + 1024);       // [S][2][128 lanes]
-    bool ok = true;
-    for (long long i = w; i < my_tokens && ok; i += S) {
-      const long long token = pair + i * npairs;
-      const uint32_t ph = (i / S) & 1;
-      ok = mbar_wait(&d1_full[w], ph, RQP_D1_FULL, limit);
-      if (!ok) break;
-      tc_fence_after_sync();
-      float m = 0.0f;
-#pragma unroll
-      for (int c = 0; c < HC / 16; ++c) {
-        uint32_t r[16];
-        tmem_ld_32x32b_x16(d1 + 16 * c, r);
-        tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 16; e += 2)
-          m = fmaxf(m, fmaxf(fabsf(__uint_as_float(r[e])), fabsf(__uint_as_float(r[e + 1]))));
-      }
-      lane_m[(w * 2 + cp) * 128 + lane_g] = m;
-      named_barrier(1 + w, 256);
-      m = fmaxf(m, lane_m[(w * 2 + (cp ^ 1)) * 128 + lane_g]);
-      int ebits = static_cast<int>((__float_as_uint(m) >> 23) & 0xFF);
-      int k = 13 - (ebits - 127);
-      if (m == 0.0f) k = 0;
-      k = max(-126, min(127, k));
-      const float sc = __uint_as_float(static_cast<uint32_t>(k + 127) << 23);
-      const int uexp = -(k + 2 * kFactorScaleLog2) + 127;
-      const float un = (uexp >= 1) ? __uint_as_float(static_cast<uint32_t>(min(uexp, 254)) << 23) : 0.0f;
-#pragma unroll
-      for (int c = 0; c < HC / 16; ++c) {
-        uint32_t r[16], o[16];
-        tmem_ld_32x32b_x16(d1 + 16 * c, r);
-        tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float v0 = __uint_as_float(r[2 * e]), v1 = __uint_as_float(r[2 * e + 1]);
-          const __half2 hh = __floats2half2_rn(v0 * sc, v1 * sc);
-          const float2 hf = __half22float2(hh);
-          o[e] = *reinterpret_cast<const uint32_t*>(&hh);
-          o[8 + e] = pack_half2(fmaf(v0, sc, -hf.x), fmaf(v1, sc, -hf.y));
-        }
-        tmem_st_32x32b_x16(d1 + 16 * c, o);
-      }
-      tmem_wait_st();
-      tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(&a2_ready[w], 0);
-
-      ok = mbar_wait(&d2_full[w], ph, RQP_D2_FULL, limit);
-      if (!ok) break;
-      tc_fence_after_sync();
-      if constexpr (F16OUT) {
-        // rotation only: the rotated row leaves as fp16 (weight-only variant), nothing is quantised
-        __half* zrow16 = reinterpret_cast<__half*>(Xq) + token * n + static_cast<long long>(pp) * N2 + cp * HC;
-#pragma unroll
-        for (int c = 0; c < HC / 16; ++c) {
-          uint32_t r[16];
-          tmem_ld_32x32b_x16(d2 + 16 * c, r);
-          tmem_wait_ld();
-          uint4 lo, hi;
-          lo.x = pack_half2(__uint_as_float(r[0]) * un, __uint_as_float(r[1]) * un);
-          lo.y = pack_half2(__uint_as_float(r[2]) * un, __uint_as_float(r[3]) * un);
-          lo.z = pack_half2(__uint_as_float(r[4]) * un, __uint_as_float(r[5]) * un);
-          lo.w = pack_half2(__uint_as_float(r[6]) * un, __uint_as_float(r[7]) * un);
-          hi.x = pack_half2(__uint_as_float(r[8]) * un, __uint_as_float(r[9]) * un);
-          hi.y = pack_half2(__uint_as_float(r[10]) * un, __uint_as_float(r[11]) * un);
-          hi.z = pack_half2(__uint_as_float(r[12]) * un, __uint_as_float(r[13]) * un);
-          hi.w = pack_half2(__uint_as_float(r[14]) * un, __uint_as_float(r[15]) * un);
-          if (live) {
-            *reinterpret_cast<uint4*>(zrow16 + 16 * c) = lo;
-            *reinterpret_cast<uint4*>(zrow16 + 16 * c + 8) = hi;
-          }
-        }
-        continue;
-      }
-      float zm = 0.0f;
-#pragma unroll
-      for (int c = 0; c < HC / 16; ++c) {
-        uint32_t r[16];
-        tmem_ld_32x32b_x16(d2 + 16 * c, r);
-        tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 16; e += 2)
-          zm = fmaxf(zm, fmaxf(fabsf(__uint_as_float(r[e])), fabsf(__uint_as_float(r[e + 1]))));
-      }
-      zm *= un;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
-      float* amax_w = amax_x + (w * 2 + ph) * 8;
-      if (lane == 0) amax_w[quarter * 2 + cp] = zm;
-      named_barrier(1 + w, 256);
-      float amax = fmaxf(fmaxf(fmaxf(amax_w[0], amax_w[1]), fmaxf(amax_w[2], amax_w[3])),
-                         fmaxf(fmaxf(amax_w[4], amax_w[5]), fmaxf(amax_w[6], amax_w[7])));
-      if (lane_g == 0 && cp == 0) st_f32_peer_and_arrive(&amax_peer[w * 2 + ph], amax, &amax_bar[w], rank ^ 1u);
-      ok = mbar_wait_acq_cluster(&amax_bar[w], ph, RQP_AMAX, limit);
-      if (!ok) break;
-      amax = fmaxf(amax, amax_peer[w * 2 + ph]);
-      __half delta;
-      float inv;
-      row_scale(amax, delta, inv);
-      const float inv_un = inv * un;
-      const bool clamp = __half2float(delta) < 6.103515625e-05f;
-      uint8_t* orow = Xq + token * (n / 2) + static_cast<long long>(pp) * (N2 / 2) + cp * (HC / 2);
-      float* zrow = (Zdbg != nullptr && live) ? Zdbg + token * n + static_cast<long long>(pp) * N2 + cp * HC : nullptr;
-#pragma unroll
-      for (int c = 0; c < HC / 16; ++c) {
-        uint32_t r[16];
-        tmem_ld_32x32b_x16(d2 + 16 * c, r);
-        tmem_wait_ld();
-        float t[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          t[e] = __fadd_rn(__fmul_rn(__uint_as_float(r[e]), inv_un), 0.5f);
-          if (clamp) t[e] = fminf(fmaxf(t[e], -8.0f), 7.5f);
-        }
-        uint2 pk;
-        pk.x = pack8_codes(t);
-        pk.y = pack8_codes(t + 8);
-        if (live) {
-          *reinterpret_cast<uint2*>(orow + 8 * c) = pk;
-          if (zrow) {
-#pragma unroll
-            for (int e = 0; e < 16; e += 4)
-              *reinterpret_cast<float4*>(zrow + 16 * c + e) =
-                  make_float4(__uint_as_float(r[e]) * un, __uint_as_float(r[e + 1]) * un,
-                              __uint_as_float(r[e + 2]) * un, __uint_as_float(r[e + 3]) * un);
-          }
-        }
-      }
-      if (pp == 0 && cp == 0) scales[token] = delta;
-    }
   } else {
     // ------------------------------ compute groups ------------------------------------------------
-    const int w = (warp - 2) >> 2;                 // accumulator slot of this group
+    // CW warps per lane quarter, as in sq_rotate_quant_tc.cu.
+    constexpr int HC = N2 / CW;
+    const int gi = (warp - 2) >> 2;
+    const int w = gi / CW, cp = gi % CW;           // accumulator slot of this group
     const int quarter = warp & 3;
     const int lane_g = quarter * 32 + lane;        // TMEM lane
     const int pp = static_cast<int>(rank) * 128 + lane_g;    // row p' of the reshaped token
     const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
-    const uint32_t d1 = tmem_base + w * SLOT_COLS + lane_addr, d2 = d1 + N2;
+    const uint32_t d1 = tmem_base + w * SLOT_COLS + lane_addr + cp * HC, d2 = d1 + N2;
     const bool live = pp < n1;
+    float* lane_m = reinterpret_cast<float*>(smem + L.off_misc + 1024);       // CW == 2: [S][2][128 lanes]
     bool ok = true;
     for (long long i = w; i < my_tokens && ok; i += S) {
       const long long token = pair + i * npairs;
       const uint32_t ph = (i / S) & 1;
+      uint32_t r[32];
 
       // ---- D1 -> fp16 hi/lo in place, with a per-lane power-of-two scale --------------------------
       ok = mbar_wait(&d1_full[w], ph, RQP_D1_FULL, limit);
       if (!ok) break;
       tc_fence_after_sync();
-      float m = 0.0f;
-#pragma unroll
-      for (int c = 0; c < N2 / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(d1 + 32 * c, r);
-        tmem_wait_ld();
-        m = fmaxf(m, absmax32(r));
+      float m = lane_absmax<HC>(d1, r);
+      if constexpr (CW == 2) {
+        lane_m[(w * 2 + cp) * 128 + lane_g] = m;
+        named_barrier(1 + w, 256);
+        m = fmaxf(m, lane_m[(w * 2 + (cp ^ 1)) * 128 + lane_g]);
       }
-      int ebits = static_cast<int>((__float_as_uint(m) >> 23) & 0xFF);
-      int k = 13 - (ebits - 127);                  // the lane's largest entry lands in [2^13, 2^14)
-      if (m == 0.0f) k = 0;
-      k = max(-126, min(127, k));
-      const float sc = __uint_as_float(static_cast<uint32_t>(k + 127) << 23);
-      const int uexp = -(k + 2 * kFactorScaleLog2) + 127;
-      const float un = (uexp >= 1) ? __uint_as_float(static_cast<uint32_t>(min(uexp, 254)) << 23) : 0.0f;
-#pragma unroll
-      for (int c = 0; c < N2 / 32; ++c) {
-        uint32_t r[32], o[32];
-        tmem_ld_32x32b_x32(d1 + 32 * c, r);
-        tmem_wait_ld();
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float v0 = __uint_as_float(r[16 * h + 2 * e]), v1 = __uint_as_float(r[16 * h + 2 * e + 1]);
-            const __half2 hh = __floats2half2_rn(v0 * sc, v1 * sc);
-            const float2 hf = __half22float2(hh);
-            o[16 * h + e] = *reinterpret_cast<const uint32_t*>(&hh);
-            o[16 * h + 8 + e] = pack_half2(fmaf(v0, sc, -hf.x), fmaf(v1, sc, -hf.y));
-          }
-        tmem_st_32x32b_x32(d1 + 32 * c, o);
-      }
+      float sc, un;
+      lane_scale(m, sc, un);
+      split_in_place<HC>(d1, r, sc);
       tmem_wait_st();
       tc_fence_before_sync();
       __syncwarp();
@@ -434,80 +271,29 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
       ok = mbar_wait(&d2_full[w], ph, RQP_D2_FULL, limit);
       if (!ok) break;
       tc_fence_after_sync();
+      const long long row0 = token * n + static_cast<long long>(pp) * N2 + cp * HC;    // this lane's first channel
       if constexpr (F16OUT) {
-        // rotation only: the rotated row leaves as fp16 (weight-only variant), nothing is quantised
-        __half* zrow16 = reinterpret_cast<__half*>(Xq) + token * n + static_cast<long long>(pp) * N2;
-#pragma unroll
-        for (int c = 0; c < N2 / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld_32x32b_x32(d2 + 32 * c, r);
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 32; e += 8) {
-            uint4 v;
-            v.x = pack_half2(__uint_as_float(r[e]) * un, __uint_as_float(r[e + 1]) * un);
-            v.y = pack_half2(__uint_as_float(r[e + 2]) * un, __uint_as_float(r[e + 3]) * un);
-            v.z = pack_half2(__uint_as_float(r[e + 4]) * un, __uint_as_float(r[e + 5]) * un);
-            v.w = pack_half2(__uint_as_float(r[e + 6]) * un, __uint_as_float(r[e + 7]) * un);
-            if (live) *reinterpret_cast<uint4*>(zrow16 + 32 * c + e) = v;
-          }
-        }
+        store_rotated_f16<HC>(d2, un, reinterpret_cast<__half*>(Xq) + row0, live);
         continue;
       }
-      float zm = 0.0f;
-#pragma unroll
-      for (int c = 0; c < N2 / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(d2 + 32 * c, r);
-        tmem_wait_ld();
-        zm = fmaxf(zm, absmax32(r));
-      }
-      zm *= un;                                      // lanes of padding rows hold exact zeros
+      float zm = lane_absmax<HC>(d2, r) * un;        // lanes of padding rows hold exact zeros
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
-      float* amax_w = amax_x + (w * 2 + ph) * 4;
-      if (lane == 0) amax_w[quarter] = zm;
-      named_barrier(1 + w, 128);
-      float amax = fmaxf(fmaxf(amax_w[0], amax_w[1]), fmaxf(amax_w[2], amax_w[3]));
-      if (lane_g == 0) st_f32_peer_and_arrive(&amax_peer[w * 2 + ph], amax, &amax_bar[w], rank ^ 1u);
+      float* amax_w = amax_x + (w * 2 + ph) * 4 * CW;
+      if (lane == 0) amax_w[quarter * CW + cp] = zm;
+      named_barrier(1 + w, 128 * CW);
+      float amax = amax_w[0];
+#pragma unroll
+      for (int x = 1; x < 4 * CW; ++x) amax = fmaxf(amax, amax_w[x]);
+      if (lane_g == 0 && cp == 0) st_f32_peer_and_arrive(&amax_peer[w * 2 + ph], amax, &amax_bar[w], rank ^ 1u);
       ok = mbar_wait_acq_cluster(&amax_bar[w], ph, RQP_AMAX, limit);
       if (!ok) break;
       amax = fmaxf(amax, amax_peer[w * 2 + ph]);
       __half delta;
       float inv;
       row_scale(amax, delta, inv);
-      const float inv_un = inv * un;
-      const bool clamp = __half2float(delta) < 6.103515625e-05f;   // see sq_rotate_quant_tc.cu
-      uint8_t* orow = Xq + token * (n / 2) + static_cast<long long>(pp) * (N2 / 2);
-      float* zrow = (Zdbg != nullptr && live) ? Zdbg + token * n + static_cast<long long>(pp) * N2 : nullptr;
-#pragma unroll
-      for (int c = 0; c < N2 / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(d2 + 32 * c, r);
-        tmem_wait_ld();
-        float t[32];
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          t[e] = __fadd_rn(__fmul_rn(__uint_as_float(r[e]), inv_un), 0.5f);
-          if (clamp) t[e] = fminf(fmaxf(t[e], -8.0f), 7.5f);
-        }
-        uint4 pk;
-        pk.x = pack8_codes(t);
-        pk.y = pack8_codes(t + 8);
-        pk.z = pack8_codes(t + 16);
-        pk.w = pack8_codes(t + 24);
-        if (live) {
-          *reinterpret_cast<uint4*>(orow + 16 * c) = pk;
-          if (zrow) {
-#pragma unroll
-            for (int e = 0; e < 32; e += 4)
-              *reinterpret_cast<float4*>(zrow + 32 * c + e) =
-                  make_float4(__uint_as_float(r[e]) * un, __uint_as_float(r[e + 1]) * un,
-                              __uint_as_float(r[e + 2]) * un, __uint_as_float(r[e + 3]) * un);
-          }
-        }
-      }
-      if (pp == 0) scales[token] = delta;
+      store_codes<HC>(d2, r, delta, inv * un, un, live, Xq + row0 / 2, (Zdbg != nullptr && live) ? Zdbg + row0 : nullptr);
+      if (pp == 0 && cp == 0) scales[token] = delta;
     }
   }
 

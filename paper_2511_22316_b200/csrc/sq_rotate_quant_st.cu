@@ -339,20 +339,13 @@ rotate_quant_st_kernel(const __grid_constant__ StLayout L, int n1, int rows, con
 #pragma unroll
         for (int e = 0; e < N2; e += 4) *reinterpret_cast<float4*>(zrow + e) = make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);
       }
+      const F2 inv2 = f2_pack(inv, inv);
 #pragma unroll
       for (int b = 0; b < N2 / 32; ++b) {
-        float t[32];
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          t[e] = __fadd_rn(__fmul_rn(x[32 * b + e], inv), 0.5f);
-          if (clamp) t[e] = fminf(fmaxf(t[e], -8.0f), 7.5f);
-        }
-        uint4 pk;
-        pk.x = pack8_codes(t);
-        pk.y = pack8_codes(t + 8);
-        pk.z = pack8_codes(t + 16);
-        pk.w = pack8_codes(t + 24);
-        if (live) *reinterpret_cast<uint4*>(orow + 16 * b) = pk;
+        uint32_t pk[4];
+        if (clamp) codes32<true>(x + 32 * b, inv2, pk);
+        else codes32<false>(x + 32 * b, inv2, pk);
+        if (live) *reinterpret_cast<uint4*>(orow + 16 * b) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
       }
       if (live && pp == 0) scales[token] = delta;
     }

@@ -110,23 +110,210 @@ __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
 // Eight consecutive codes -> one packed word.  u_i = floor(t_i) + 8 is taken from the low bits of
 // t_i + (2^23 + 8) rounded towards -inf (no conversion instruction); the words' common high bits
 // cancel in `kBias`; flipping bit 3 of every nibble turns the offset code into two's complement.
-__device__ __forceinline__ uint32_t pack8_codes(const float* t) {
+__device__ __forceinline__ uint32_t join8_codes(const float* u) {
   constexpr uint32_t kBias = 0x4B000000u * 0x11111111u;
-  uint32_t w = __float_as_uint(__fadd_rd(t[7], 8388616.0f));
+  uint32_t w = __float_as_uint(u[7]);
 #pragma unroll
-  for (int i = 6; i >= 0; --i) w = w * 16u + __float_as_uint(__fadd_rd(t[i], 8388616.0f));
+  for (int i = 6; i >= 0; --i) w = w * 16u + __float_as_uint(u[i]);
   return (w - kBias) ^ 0x88888888u;
 }
+__device__ __forceinline__ uint32_t pack8_codes(const float* t) {
+  float u[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) u[i] = __fadd_rd(t[i], 8388616.0f);
+  return join8_codes(u);
+}
 
-// max |r[e]| over 32 fp32 bit patterns, as a tree (four independent chains).
-__device__ __forceinline__ float absmax32(const uint32_t (&r)[32]) {
+// Two fp32 numbers in a register pair: one instruction works on both, each rounded as the scalar form rounds it.  The warps
+// of these kernels issue on 64 % of the cycles (11008 x 4096), so instructions are what the element-wise steps cost.
+using F2 = unsigned long long;
+
+__device__ __forceinline__ F2 f2_pack(float a, float b) {
+  F2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ void f2_unpack(F2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  F2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  F2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ F2 f2_add_rd(F2 a, F2 b) {
+  F2 d;
+  asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ F2 f2_sub(F2 a, F2 b) {
+  F2 d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float absmax3(float a, float b, float c) {
+  float d;
+  asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
+// One whole 32-byte sector per lane: the lanes of a warp write rows that are 32 bytes (packed codes) to 256 bytes (fp16)
+// apart, and sectors written in two halves cost twice.  The buffers are only promised to be 16-byte aligned.
+__device__ __forceinline__ void store_sector(void* p, const uint32_t* v, bool aligned32) {
+  if (aligned32) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+                 "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+  } else {
+    static_cast<uint4*>(p)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    static_cast<uint4*>(p)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+  }
+}
+
+// Eight rotated values -> one packed word: code = floor(z / Delta + 1/2), product and sum rounded on their own.
+template <bool CLAMP>
+__device__ __forceinline__ uint32_t codes8(const float* z, F2 inv2) {
+  const F2 half2 = f2_pack(0.5f, 0.5f), magic2 = f2_pack(8388616.0f, 8388616.0f);
+  float u[8];
+#pragma unroll
+  for (int e = 0; e < 8; e += 2) {
+    F2 t = f2_add(f2_mul(f2_pack(z[e], z[e + 1]), inv2), half2);
+    if (CLAMP) {
+      float a, b;
+      f2_unpack(t, a, b);
+      t = f2_pack(fminf(fmaxf(a, -8.0f), 7.5f), fminf(fmaxf(b, -8.0f), 7.5f));
+    }
+    f2_unpack(f2_add_rd(t, magic2), u[e], u[e + 1]);
+  }
+  return join8_codes(u);
+}
+
+// 32 rotated values -> 16 packed bytes.
+template <bool CLAMP>
+__device__ __forceinline__ void codes32(const float* z, F2 inv2, uint32_t* pk) {
+#pragma unroll
+  for (int e = 0; e < 4; ++e) pk[e] = codes8<CLAMP>(z + 8 * e, inv2);
+}
+
+// max |D| over the HC columns of a lane from TMEM column `d` on (four independent chains).  `r` keeps the last 32 columns:
+// the pass that follows starts with those and reads the others once more.
+template <int HC>
+__device__ __forceinline__ float lane_absmax(uint32_t d, uint32_t (&r)[32]) {
   float m[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-  for (int e = 0; e < 32; e += 8)
+  for (int c = 0; c < HC / 32; ++c) {
+    tmem_ld_32x32b_x32(d + 32 * c, r);
+    tmem_wait_ld();
 #pragma unroll
-    for (int x = 0; x < 4; ++x)
-      m[x] = fmaxf(m[x], fmaxf(fabsf(__uint_as_float(r[e + 2 * x])), fabsf(__uint_as_float(r[e + 2 * x + 1]))));
+    for (int e = 0; e < 32; e += 8)
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+        m[x] = absmax3(m[x], __uint_as_float(r[e + 2 * x]), __uint_as_float(r[e + 2 * x + 1]));
+  }
   return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+}
+
+// The lane's power-of-two scale `sc`, chosen so that its largest entry lands in [2^13, 2^14), and `un`, which divides it
+// and the two factor scales out again exactly: z = D2 * 2^-(k + 20).
+__device__ __forceinline__ void lane_scale(float m, float& sc, float& un) {
+  const int ebits = static_cast<int>((__float_as_uint(m) >> 23) & 0xFF);
+  int k = 13 - (ebits - 127);
+  if (m == 0.0f) k = 0;
+  k = max(-126, min(127, k));
+  sc = __uint_as_float(static_cast<uint32_t>(k + 127) << 23);
+  const int uexp = -(k + 2 * kFactorScaleLog2) + 127;
+  un = (uexp >= 1) ? __uint_as_float(static_cast<uint32_t>(min(uexp, 254)) << 23) : 0.0f;
+}
+
+// D1 -> fp16 hi + lo of D1 * sc in place: 16 fp32 columns become 8 columns of hi and 8 of lo.  `r` holds the last 32
+// columns.  (v sc is exact unless it underflows, and then hi is 0: the difference is what the fused form would give.)
+template <int HC>
+__device__ __forceinline__ void split_in_place(uint32_t d1, uint32_t (&r)[32], float sc) {
+  const F2 sc2 = f2_pack(sc, sc);
+#pragma unroll
+  for (int c = HC / 32 - 1; c >= 0; --c) {
+    uint32_t o[32];
+    if (c < HC / 32 - 1) {
+      tmem_ld_32x32b_x32(d1 + 32 * c, r);
+      tmem_wait_ld();
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const F2 v = f2_mul(f2_pack(__uint_as_float(r[16 * h + 2 * e]), __uint_as_float(r[16 * h + 2 * e + 1])), sc2);
+        float a, b;
+        f2_unpack(v, a, b);
+        const __half2 hh = __floats2half2_rn(a, b);
+        const float2 hf = __half22float2(hh);
+        f2_unpack(f2_sub(v, f2_pack(hf.x, hf.y)), a, b);
+        o[16 * h + e] = *reinterpret_cast<const uint32_t*>(&hh);
+        o[16 * h + 8 + e] = pack_half2(a, b);
+      }
+    tmem_st_32x32b_x32(d1 + 32 * c, o);
+  }
+}
+
+// The lane's HC columns of D2, times `un`, as fp16 (the weight-only variant: nothing is quantised).
+template <int HC>
+__device__ __forceinline__ void store_rotated_f16(uint32_t d2, float un, __half* __restrict__ zrow, bool live) {
+  const F2 un2 = f2_pack(un, un);
+  const bool aligned32 = (reinterpret_cast<uintptr_t>(zrow) & 31) == 0;
+#pragma unroll
+  for (int c = 0; c < HC / 32; ++c) {
+    uint32_t r[32], o[16];
+    tmem_ld_32x32b_x32(d2 + 32 * c, r);
+    tmem_wait_ld();
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      float a, b;
+      f2_unpack(f2_mul(f2_pack(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])), un2), a, b);
+      o[e] = pack_half2(a, b);
+    }
+    if (live) {
+      store_sector(zrow + 32 * c, o, aligned32);
+      store_sector(zrow + 32 * c + 16, o + 8, aligned32);
+    }
+  }
+}
+
+// Quantises, packs and stores the lane's HC columns of D2.  `r` holds the last 32 columns; `inv_un` = un / Delta (exact, a
+// power of two times 1 / Delta).  Delta >= 2^-14 (a normal fp16) bounds |z / Delta| by 7 (1 + 2^-11): no clamp is needed then.
+template <int HC>
+__device__ __forceinline__ void store_codes(uint32_t d2, uint32_t (&r)[32], __half delta, float inv_un, float un, bool live,
+                                            uint8_t* __restrict__ orow, float* __restrict__ zrow) {
+  const F2 inv2 = f2_pack(inv_un, inv_un);
+  const bool aligned32 = (reinterpret_cast<uintptr_t>(orow) & 31) == 0;
+  uint32_t pk[HC / 8];
+  const bool clamp = __half2float(delta) < 6.103515625e-05f;
+#pragma unroll
+  for (int c = HC / 32 - 1; c >= 0; --c) {
+    if (c < HC / 32 - 1) {
+      tmem_ld_32x32b_x32(d2 + 32 * c, r);
+      tmem_wait_ld();
+    }
+    const float* z = reinterpret_cast<const float*>(r);
+    if (clamp) codes32<true>(z, inv2, pk + 4 * c);
+    else codes32<false>(z, inv2, pk + 4 * c);
+    if (live) {
+      if (zrow) {
+#pragma unroll
+        for (int e = 0; e < 32; e += 4)
+          *reinterpret_cast<float4*>(zrow + 32 * c + e) = make_float4(z[e] * un, z[e + 1] * un, z[e + 2] * un, z[e + 3] * un);
+      }
+    }
+  }
+  if (live) {
+    if constexpr (HC == 32) {
+      *reinterpret_cast<uint4*>(orow) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    } else {
+#pragma unroll
+      for (int c = 0; c < HC / 64; ++c) store_sector(orow + 32 * c, pk + 8 * c, aligned32);
+    }
+  }
 }
 
 // The kernel's body, for CTA `cta` of `ncta` that share the token groups (the fused decode kernel of
@@ -292,208 +479,42 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
         }
       }
     }
-  } else if (CW == 2 && warp < 2 + 4 * S * CW) {
-    // ------------------------------ compute groups, two warps per lane quarter ---------------------
-    // Eight warps per accumulator slot: warp (quarter, cp) owns columns [cp * N2/2, (cp+1) * N2/2) of
-    // its lane quarter and works through them 16 at a time (the register budget of 18 warps per CTA).
-    // Twice as many warps are there to issue while others wait for tensor memory or a barrier.
-    constexpr int HC = N2 / 2;                     // columns per warp
-    const int gi = (warp - 2) >> 2;
-    const int w = gi >> 1, cp = gi & 1;
-    const int quarter = warp & 3;
-    const int lane_g = quarter * 32 + lane;
-    const int tk = lane_g / LS, pp = lane_g % LS;
-    const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
-    const uint32_t d1 = tmem_base + w * SLOT_COLS + lane_addr + cp * HC, d2 = d1 + N2;
-    const int wpt = LS / 32;
-    const int q0 = (quarter / wpt) * wpt;
-    float* lane_m = reinterpret_cast<float*>(smem + L.off_misc + 512);       // [S][2][128 lanes]
-    bool ok = true;
-    for (int i = w; i < my_groups && ok; i += S) {
-      const int g = cta + i * ncta;
-      const long long token = static_cast<long long>(g) * G + tk;
-      const uint32_t ph = (i / S) & 1;
-      ok = mbar_wait(&d1_full[w], ph, RQ_D1_FULL, limit);
-      if (!ok) break;
-      tc_fence_after_sync();
-      // The lane's scale must be the same in the two warps that share the lane: each takes the absmax of
-      // its own columns and they swap through shared memory.  The barrier also keeps either from
-      // overwriting a column of D1 that the other has yet to read (it reads only its own: nothing to keep).
-      float m = 0.0f;
-#pragma unroll
-      for (int c = 0; c < HC / 16; ++c) {
-        uint32_t r[16];
-        tmem_ld_32x32b_x16(d1 + 16 * c, r);
-        tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 16; e += 2)
-          m = fmaxf(m, fmaxf(fabsf(__uint_as_float(r[e])), fabsf(__uint_as_float(r[e + 1]))));
-      }
-      lane_m[(w * 2 + cp) * 128 + lane_g] = m;
-      named_barrier(1 + w, 256);
-      m = fmaxf(m, lane_m[(w * 2 + (cp ^ 1)) * 128 + lane_g]);
-      int ebits = static_cast<int>((__float_as_uint(m) >> 23) & 0xFF);
-      int k = 13 - (ebits - 127);
-      if (m == 0.0f) k = 0;
-      k = max(-126, min(127, k));
-      const float sc = __uint_as_float(static_cast<uint32_t>(k + 127) << 23);
-      const int uexp = -(k + 2 * kFactorScaleLog2) + 127;
-      const float un = (uexp >= 1) ? __uint_as_float(static_cast<uint32_t>(min(uexp, 254)) << 23) : 0.0f;
-#pragma unroll
-      for (int c = 0; c < HC / 16; ++c) {
-        uint32_t r[16], o[16];
-        tmem_ld_32x32b_x16(d1 + 16 * c, r);
-        tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float v0 = __uint_as_float(r[2 * e]), v1 = __uint_as_float(r[2 * e + 1]);
-          const __half2 hh = __floats2half2_rn(v0 * sc, v1 * sc);
-          const float2 hf = __half22float2(hh);
-          o[e] = *reinterpret_cast<const uint32_t*>(&hh);
-          o[8 + e] = pack_half2(fmaf(v0, sc, -hf.x), fmaf(v1, sc, -hf.y));
-        }
-        tmem_st_32x32b_x16(d1 + 16 * c, o);
-      }
-      tmem_wait_st();
-      tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&a2_ready[w]);
-
-      ok = mbar_wait(&d2_full[w], ph, RQ_D2_FULL, limit);
-      if (!ok) break;
-      tc_fence_after_sync();
-      if constexpr (F16OUT) {
-        // rotation only: the rotated row leaves as fp16 (weight-only variant), nothing is quantised
-        const bool live16 = (pp < n1) && (tk < G) && (token < rows);
-        __half* zrow16 = reinterpret_cast<__half*>(Xq) + token * n + pp * N2 + cp * HC;
-#pragma unroll
-        for (int c = 0; c < HC / 16; ++c) {
-          uint32_t r[16];
-          tmem_ld_32x32b_x16(d2 + 16 * c, r);
-          tmem_wait_ld();
-          uint4 lo, hi;
-          lo.x = pack_half2(__uint_as_float(r[0]) * un, __uint_as_float(r[1]) * un);
-          lo.y = pack_half2(__uint_as_float(r[2]) * un, __uint_as_float(r[3]) * un);
-          lo.z = pack_half2(__uint_as_float(r[4]) * un, __uint_as_float(r[5]) * un);
-          lo.w = pack_half2(__uint_as_float(r[6]) * un, __uint_as_float(r[7]) * un);
-          hi.x = pack_half2(__uint_as_float(r[8]) * un, __uint_as_float(r[9]) * un);
-          hi.y = pack_half2(__uint_as_float(r[10]) * un, __uint_as_float(r[11]) * un);
-          hi.z = pack_half2(__uint_as_float(r[12]) * un, __uint_as_float(r[13]) * un);
-          hi.w = pack_half2(__uint_as_float(r[14]) * un, __uint_as_float(r[15]) * un);
-          if (live16) {
-            *reinterpret_cast<uint4*>(zrow16 + 16 * c) = lo;
-            *reinterpret_cast<uint4*>(zrow16 + 16 * c + 8) = hi;
-          }
-        }
-        continue;
-      }
-      float zm = 0.0f;
-#pragma unroll
-      for (int c = 0; c < HC / 16; ++c) {
-        uint32_t r[16];
-        tmem_ld_32x32b_x16(d2 + 16 * c, r);
-        tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 16; e += 2)
-          zm = fmaxf(zm, fmaxf(fabsf(__uint_as_float(r[e])), fabsf(__uint_as_float(r[e + 1]))));
-      }
-      zm *= un;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
-      float* amax_w = amax_x + (w * 2 + ph) * 8;
-      if (lane == 0) amax_w[quarter * 2 + cp] = zm;
-      named_barrier(1 + w, 256);
-      float amax = fmaxf(amax_w[q0 * 2], amax_w[q0 * 2 + 1]);
-      for (int x = 1; x < wpt; ++x) amax = fmaxf(amax, fmaxf(amax_w[(q0 + x) * 2], amax_w[(q0 + x) * 2 + 1]));
-      __half delta;
-      float inv;
-      row_scale(amax, delta, inv);
-      const float inv_un = inv * un;
-      const bool live = (pp < n1) && (tk < G) && (token < rows);
-      const bool clamp = __half2float(delta) < 6.103515625e-05f;
-      uint8_t* orow = Xq + token * (n / 2) + pp * (N2 / 2) + cp * (HC / 2);
-      float* zrow = (Zdbg != nullptr && live) ? Zdbg + token * n + pp * N2 + cp * HC : nullptr;
-#pragma unroll
-      for (int c = 0; c < HC / 16; ++c) {
-        uint32_t r[16];
-        tmem_ld_32x32b_x16(d2 + 16 * c, r);
-        tmem_wait_ld();
-        float t[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          t[e] = __fadd_rn(__fmul_rn(__uint_as_float(r[e]), inv_un), 0.5f);
-          if (clamp) t[e] = fminf(fmaxf(t[e], -8.0f), 7.5f);
-        }
-        uint2 pk;
-        pk.x = pack8_codes(t);
-        pk.y = pack8_codes(t + 8);
-        if (live) {
-          *reinterpret_cast<uint2*>(orow + 8 * c) = pk;
-          if (zrow) {
-#pragma unroll
-            for (int e = 0; e < 16; e += 4)
-              *reinterpret_cast<float4*>(zrow + 16 * c + e) =
-                  make_float4(__uint_as_float(r[e]) * un, __uint_as_float(r[e + 1]) * un,
-                              __uint_as_float(r[e + 2]) * un, __uint_as_float(r[e + 3]) * un);
-          }
-        }
-      }
-      if (live && pp == 0 && cp == 0) scales[token] = delta;
-    }
-  } else if (CW == 1 && warp < 2 + 4 * S) {
+  } else if (warp < 2 + 4 * S * CW) {
     // ------------------------------ compute groups ------------------------------------------------
-    const int w = (warp - 2) >> 2;                 // accumulator slot of this group
+    // CW warps per lane quarter: warp (quarter, cp) owns columns [cp * HC, (cp + 1) * HC) of it.
+    constexpr int HC = N2 / CW;                    // columns per warp
+    const int gi = (warp - 2) >> 2;
+    const int w = gi / CW, cp = gi % CW;           // accumulator slot of this group
     const int quarter = warp & 3;                  // TMEM lane quarter this warp may touch
     const int lane_g = quarter * 32 + lane;        // accumulator lane = token-in-group * LS + p'
     const int tk = lane_g / LS, pp = lane_g % LS;
     const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
-    const uint32_t d1 = tmem_base + w * SLOT_COLS + lane_addr, d2 = d1 + N2;
-    const int wpt = LS / 32;                       // warps that share a token
+    const uint32_t d1 = tmem_base + w * SLOT_COLS + lane_addr + cp * HC, d2 = d1 + N2;
+    const int wpt = LS / 32;                       // lane quarters that share a token
     const int q0 = (quarter / wpt) * wpt;
+    float* lane_m = reinterpret_cast<float*>(smem + L.off_misc + 512);       // CW == 2: [S][2][128 lanes]
     bool ok = true;
     for (int i = w; i < my_groups && ok; i += S) {
       const int g = cta + i * ncta;
       const long long token = static_cast<long long>(g) * G + tk;
       const uint32_t ph = (i / S) & 1;
+      const bool live = (pp < n1) && (tk < G) && (token < rows);
+      uint32_t r[32];
 
       // ---- D1 -> fp16 hi/lo in place, with a per-lane power-of-two scale --------------------------
       ok = mbar_wait(&d1_full[w], ph, RQ_D1_FULL, limit);
       if (!ok) break;
       tc_fence_after_sync();
-      float m = 0.0f;
-#pragma unroll
-      for (int c = 0; c < N2 / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(d1 + 32 * c, r);
-        tmem_wait_ld();
-        m = fmaxf(m, absmax32(r));
+      float m = lane_absmax<HC>(d1, r);
+      if constexpr (CW == 2) {
+        // The lane's scale must be the same in the two warps that share the lane.
+        lane_m[(w * 2 + cp) * 128 + lane_g] = m;
+        named_barrier(1 + w, 256);
+        m = fmaxf(m, lane_m[(w * 2 + (cp ^ 1)) * 128 + lane_g]);
       }
-      // scale so that the lane's largest entry lands in [2^13, 2^14)
-      int ebits = static_cast<int>((__float_as_uint(m) >> 23) & 0xFF);
-      int k = 13 - (ebits - 127);
-      if (m == 0.0f) k = 0;
-      k = max(-126, min(127, k));
-      const float sc = __uint_as_float(static_cast<uint32_t>(k + 127) << 23);
-      // z = D2 * 2^-(k + 20): the two factor scales and the lane scale, divided out exactly
-      const int uexp = -(k + 2 * kFactorScaleLog2) + 127;
-      const float un = (uexp >= 1) ? __uint_as_float(static_cast<uint32_t>(min(uexp, 254)) << 23) : 0.0f;
-#pragma unroll
-      for (int c = 0; c < N2 / 32; ++c) {
-        uint32_t r[32], o[32];
-        tmem_ld_32x32b_x32(d1 + 32 * c, r);
-        tmem_wait_ld();
-#pragma unroll
-        for (int h = 0; h < 2; ++h)                  // 16 fp32 columns -> 8 columns of hi + 8 of lo
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float v0 = __uint_as_float(r[16 * h + 2 * e]), v1 = __uint_as_float(r[16 * h + 2 * e + 1]);
-            const __half2 hh = __floats2half2_rn(v0 * sc, v1 * sc);
-            const float2 hf = __half22float2(hh);
-            o[16 * h + e] = *reinterpret_cast<const uint32_t*>(&hh);
-            o[16 * h + 8 + e] = pack_half2(fmaf(v0, sc, -hf.x), fmaf(v1, sc, -hf.y));
-          }
-        tmem_st_32x32b_x32(d1 + 32 * c, o);
-      }
+      float sc, un;
+      lane_scale(m, sc, un);
+      split_in_place<HC>(d1, r, sc);
       tmem_wait_st();
       tc_fence_before_sync();
       __syncwarp();
@@ -504,79 +525,23 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       if (!ok) break;
       tc_fence_after_sync();
       if constexpr (F16OUT) {
-        // rotation only: the rotated row leaves as fp16 (weight-only variant), nothing is quantised
-        const bool live16 = (pp < n1) && (tk < G) && (token < rows);
-        __half* zrow16 = reinterpret_cast<__half*>(Xq) + token * n + pp * N2;
-#pragma unroll
-        for (int c = 0; c < N2 / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld_32x32b_x32(d2 + 32 * c, r);
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 32; e += 8) {
-            uint4 v;
-            v.x = pack_half2(__uint_as_float(r[e]) * un, __uint_as_float(r[e + 1]) * un);
-            v.y = pack_half2(__uint_as_float(r[e + 2]) * un, __uint_as_float(r[e + 3]) * un);
-            v.z = pack_half2(__uint_as_float(r[e + 4]) * un, __uint_as_float(r[e + 5]) * un);
-            v.w = pack_half2(__uint_as_float(r[e + 6]) * un, __uint_as_float(r[e + 7]) * un);
-            if (live16) *reinterpret_cast<uint4*>(zrow16 + 32 * c + e) = v;
-          }
-        }
+        store_rotated_f16<HC>(d2, un, reinterpret_cast<__half*>(Xq) + token * n + pp * N2 + cp * HC, live);
         continue;
       }
-      float zm = 0.0f;
-#pragma unroll
-      for (int c = 0; c < N2 / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(d2 + 32 * c, r);
-        tmem_wait_ld();
-        zm = fmaxf(zm, absmax32(r));
-      }
-      zm *= un;                                      // lanes of padding rows hold exact zeros
+      float zm = lane_absmax<HC>(d2, r) * un;        // lanes of padding rows hold exact zeros
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
-      float* amax_w = amax_x + (w * 2 + ph) * 4;
-      if (lane == 0) amax_w[quarter] = zm;
-      named_barrier(1 + w, 128);
-      float amax = amax_w[q0];
-      for (int x = 1; x < wpt; ++x) amax = fmaxf(amax, amax_w[q0 + x]);
+      float* amax_w = amax_x + (w * 2 + ph) * 4 * CW;
+      if (lane == 0) amax_w[quarter * CW + cp] = zm;
+      named_barrier(1 + w, 128 * CW);
+      float amax = amax_w[q0 * CW];
+      for (int x = 1; x < wpt * CW; ++x) amax = fmaxf(amax, amax_w[q0 * CW + x]);
       __half delta;
       float inv;
       row_scale(amax, delta, inv);
-      const float inv_un = inv * un;                 // exact: un is a power of two
-      const bool live = (pp < n1) && (tk < G) && (token < rows);
-      // Delta >= 2^-14 (a normal fp16) bounds |z / Delta| by 7 (1 + 2^-11): no clamp is needed then.
-      const bool clamp = __half2float(delta) < 6.103515625e-05f;
-      uint8_t* orow = Xq + token * (n / 2) + pp * (N2 / 2);
-      float* zrow = (Zdbg != nullptr && live) ? Zdbg + token * n + pp * N2 : nullptr;
-#pragma unroll
-      for (int c = 0; c < N2 / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld_32x32b_x32(d2 + 32 * c, r);
-        tmem_wait_ld();
-        float t[32];
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          t[e] = __fadd_rn(__fmul_rn(__uint_as_float(r[e]), inv_un), 0.5f);
-          if (clamp) t[e] = fminf(fmaxf(t[e], -8.0f), 7.5f);
-        }
-        uint4 pk;
-        pk.x = pack8_codes(t);
-        pk.y = pack8_codes(t + 8);
-        pk.z = pack8_codes(t + 16);
-        pk.w = pack8_codes(t + 24);
-        if (live) {
-          *reinterpret_cast<uint4*>(orow + 16 * c) = pk;
-          if (zrow) {
-#pragma unroll
-            for (int e = 0; e < 32; e += 4)
-              *reinterpret_cast<float4*>(zrow + 32 * c + e) =
-                  make_float4(__uint_as_float(r[e]) * un, __uint_as_float(r[e + 1]) * un,
-                              __uint_as_float(r[e + 2]) * un, __uint_as_float(r[e + 3]) * un);
-          }
-        }
-      }
-      if (live && pp == 0) scales[token] = delta;
+      store_codes<HC>(d2, r, delta, inv * un, un, live, Xq + token * (n / 2) + pp * (N2 / 2) + cp * (HC / 2),
+                      (Zdbg != nullptr && live) ? Zdbg + token * n + pp * N2 + cp * HC : nullptr);
+      if (live && pp == 0 && cp == 0) scales[token] = delta;
     }
   }
 

@@ -158,6 +158,23 @@ def test_rotate_quant_warp_level(sq, n1, n2, M):
     check_rotate_quant(sq, X, R1, R2)
 
 
+# Whole 32-byte sectors are stored at once where the buffers allow it; 16 bytes is what callers have to promise.
+@pytest.mark.parametrize("n1,n2,M", [(64, 64, 35), (48, 128, 33), (172, 64, 5), (136, 128, 3), (64, 64, 3)])
+def test_rotate_outputs_16_byte_aligned_only(sq, n1, n2, M):
+    K = n1 * n2
+    X = wl.make_activations(wl.small(f"al{n1}x{n2}", M, n1, n2, 8, seed=n1 + n2))
+    R1, R2 = ora.build_rotation(X.astype(np.float32), n1, n2, seed=2)
+    rot, Xd, got = sq.sq_rotation_from_factors(R1, R2), dev(X), []
+    for skew in (0, 16):
+        q, sx, z = Guarded(M * K // 2 + 16), Guarded(M * 2), Guarded(M * K * 2 + 16)
+        sq.sq_rotate_quant_act(rot, Xd, M, q.data_ptr() + skew, sx)
+        sq.sq_rotate_act_f16(rot, Xd, M, z.data_ptr() + skew)
+        torch_mod().cuda.synchronize()
+        q.check(), z.check()
+        got.append((q.view[skew:skew + M * K // 2].cpu().numpy(), z.view[skew:skew + M * K * 2].cpu().numpy()))
+    assert all(np.array_equal(a, b) for a, b in zip(*got))
+
+
 def test_rotate_quant_tiny_config(sq):
     w = wl.TINY
     X = wl.make_activations(w)
