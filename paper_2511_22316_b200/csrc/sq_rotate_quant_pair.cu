@@ -74,7 +74,7 @@ __device__ __forceinline__ uint64_t umma_desc_mn(uint32_t smem_addr, uint32_t sb
 template <int N2, int CW, bool F16OUT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((2 + 4 * CW * (256 / N2)) * 32, 1)
 rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsigned char* __restrict__ a1_img,
-                         const unsigned char* __restrict__ b2_img, int n1, long long rows,
+                         const unsigned char* __restrict__ b2_img, int n1, int rows,
                          uint8_t* __restrict__ Xq, __half* __restrict__ scales, float* __restrict__ Zdbg) {
   constexpr int S = 256 / N2;
   constexpr int SLOT_COLS = 2 * N2;
@@ -102,17 +102,16 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
-  const long long pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
-  const long long my_tokens = (rows > pair) ? (rows - pair + npairs - 1) / npairs : 0;
+  const int pair = static_cast<int>(blockIdx.x >> 1), npairs = static_cast<int>(gridDim.x >> 1);
+  const int my_tokens = (rows > pair) ? (rows - pair + npairs - 1) / npairs : 0;
   const uint32_t limit = wait_limit();
 
-  auto load_token = [&](long long i) {
-    const long long t = pair + i * npairs;
-    const int s = static_cast<int>(i % L.XS);
+  auto load_token = [&](int i, int s) {                  // token i -> ring stage s
+    const int t = pair + i * npairs;
     mbar_arrive_expect_tx(&x_full[s], static_cast<uint32_t>(L.x_tile));
-    tma_load_3d(xs + s * L.x_tile, &tmap_x, &x_full[s], static_cast<int32_t>(rank) * L.HQ, 0, static_cast<int32_t>(t));
+    tma_load_3d(xs + s * L.x_tile, &tmap_x, &x_full[s], static_cast<int32_t>(rank) * L.HQ, 0, t);
   };
-  const long long preload = my_tokens < L.XS ? my_tokens : L.XS;
+  const int preload = my_tokens < L.XS ? my_tokens : L.XS;
 
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmap_x);
@@ -142,7 +141,7 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
     // only now may a GEMM launched behind this kernel start (it requests its weights before it waits for
     // this kernel, and this kernel's predecessor may have been writing them)
     griddep_launch_dependents();
-    for (long long i = 0; i < preload; ++i) load_token(i);
+    for (int i = 0; i < preload; ++i) load_token(i, i);
   }
   if (warp == 1) {
     tmem_alloc_pair(tmem_slot, 512);
@@ -157,9 +156,15 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
   if (warp == 0) {
     // ------------------------------ producer: keeps this CTA's half of the X ring full --------------
     if (lane == 0) {
-      for (long long i = preload; i < my_tokens; ++i) {
-        if (!mbar_wait(&x_empty[i % L.XS], ((i / L.XS) & 1) ^ 1, RQP_X_EMPTY, limit)) break;
-        load_token(i);
+      int s = 0;                                       // preload == XS here
+      uint32_t ph = 0;
+      for (int i = preload; i < my_tokens; ++i) {
+        if (!mbar_wait(&x_empty[s], ph, RQP_X_EMPTY, limit)) break;
+        load_token(i, s);
+        if (++s == L.XS) {
+          s = 0;
+          ph ^= 1;
+        }
       }
     }
   } else if (warp == 1) {
@@ -168,9 +173,15 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
       if (lane == 0) {
         bool ok = mbar_wait(img_full, 0, RQP_IMG, limit);
         if (ok) mbar_arrive_cluster(peer_img, 0);
-        for (long long i = 0; i < my_tokens && ok; ++i) {
-          ok = mbar_wait(&x_full[i % L.XS], (i / L.XS) & 1, RQP_X_FULL, limit);
-          if (ok) mbar_arrive_cluster(&xp_full[i % L.XS], 0);
+        int s = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < my_tokens && ok; ++i) {
+          ok = mbar_wait(&x_full[s], ph, RQP_X_FULL, limit);
+          if (ok) mbar_arrive_cluster(&xp_full[s], 0);
+          if (++s == L.XS) {
+            s = 0;
+            ph ^= 1;
+          }
         }
       }
     } else if (elect_one()) {
@@ -181,8 +192,8 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
       const uint64_t x_desc0 = umma_desc_mn(smem_u32(xs), 8u * L.x_row, N2 == 128 ? 2u : 4u);
       const int ksteps1 = L.N1 / 16;
       bool ok = mbar_wait(img_full, 0, RQP_IMG, limit) && mbar_wait(peer_img, 0, RQP_IMG, limit);
-      auto stage1 = [&](long long i) {
-        const int slot = static_cast<int>(i % S), xs_i = static_cast<int>(i % L.XS);
+      auto stage1 = [&](int i, int xs_i) {
+        const int slot = i % S;
         tc_fence_after_sync();
         const uint32_t d1 = tmem_base + slot * SLOT_COLS;
         uint64_t bd = x_desc0 + ((xs_i * L.x_tile) >> 4);
@@ -194,8 +205,8 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
         umma_commit_pair_mc(&x_empty[xs_i], 3);
         umma_commit_pair_mc(&d1_full[slot], 3);
       };
-      auto stage2 = [&](long long i) {
-        const int slot = static_cast<int>(i % S);
+      auto stage2 = [&](int i) {
+        const int slot = i % S;
         tc_fence_after_sync();
         const uint32_t d1 = tmem_base + slot * SLOT_COLS, d2 = d1 + N2;
 #pragma unroll
@@ -207,15 +218,22 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
         }
         umma_commit_pair_mc(&d2_full[slot], 3);
       };
-      long long i1 = 0, i2 = 0;
+      // Ring stage and phase of X are counted along: with a 64-bit division by XS in each of them, a round of polls had taken
+      // 800 cycles.
+      int i1 = 0, i2 = 0, xr = 0;
+      uint32_t xph = 0;
       uint32_t idle = 0;
       while (ok && i2 < my_tokens) {
         bool did = false;
         if (i1 < my_tokens && i1 < i2 + S &&
-            mbar_test_wait(&x_full[i1 % L.XS], (i1 / L.XS) & 1) &&
-            mbar_test_wait(&xp_full[i1 % L.XS], (i1 / L.XS) & 1) &&
+            mbar_test_wait(&x_full[xr], xph) &&
+            mbar_test_wait(&xp_full[xr], xph) &&
             mbar_test_wait(&d2_full[i1 % S], ((i1 / S) & 1) ^ 1)) {   // D1 free: the slot's previous stage 2 is done
-          stage1(i1++);
+          stage1(i1++, xr);
+          if (++xr == L.XS) {
+            xr = 0;
+            xph ^= 1;
+          }
           did = true;
         }
         if (i2 < i1 && mbar_test_wait(&a2_ready[i2 % S], (i2 / S) & 1)) {
@@ -244,8 +262,8 @@ rotate_quant_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const unsig
     const bool live = pp < n1;
     float* lane_m = reinterpret_cast<float*>(smem + L.off_misc + 1024);       // CW == 2: [S][2][128 lanes]
     bool ok = true;
-    for (long long i = w; i < my_tokens && ok; i += S) {
-      const long long token = pair + i * npairs;
+    for (int i = w; i < my_tokens && ok; i += S) {
+      const long long token = pair + static_cast<long long>(i) * npairs;
       const uint32_t ph = (i / S) & 1;
       uint32_t r[32];
 
@@ -353,6 +371,7 @@ bool rotate_quant_pair_prepare(sq_rotation* h) {
 sq_status_t launch_rotate_quant_pair(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
                                      float* Zdbg, cudaStream_t s, bool f16out) {
   const int n1 = h->n1, n2 = h->n2;
+  if (rows > 0x7FFFFFFF) return SQ_ERR_UNSUPPORTED;   // the kernel counts tokens in 32 bits
   const RqPairLayout L = rq_pair_layout(n1, n2);
   EncodeTiledFn enc = get_encode_fn();
   if (!enc) return SQ_ERR_CUDA;
@@ -375,14 +394,14 @@ sq_status_t launch_rotate_quant_pair(const sq_rotation* h, const void* X, int64_
   if (n2 == 64) {
     auto kern = f16out ? rotate_quant_pair_kernel<64, 1, true> : rotate_quant_pair_kernel<64, 1, false>;
     if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem)) return SQ_ERR_CUDA;
-    if (launch_dependent(kern, dim3(grid), dim3((2 + 4 * 4) * 32), static_cast<size_t>(smem), s, mx, a1, b2, n1, rows,
+    if (launch_dependent(kern, dim3(grid), dim3((2 + 4 * 4) * 32), static_cast<size_t>(smem), s, mx, a1, b2, n1, static_cast<int>(rows),
                          static_cast<uint8_t*>(Xq), static_cast<__half*>(scales), Zdbg) != cudaSuccess)
       return SQ_ERR_CUDA;
   } else {
     // two slots of eight warps (18 warps in the CTA instead of 10)
     auto kern = f16out ? rotate_quant_pair_kernel<128, 2, true> : rotate_quant_pair_kernel<128, 2, false>;
     if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem)) return SQ_ERR_CUDA;
-    if (launch_dependent(kern, dim3(grid), dim3((2 + 4 * 2 * 2) * 32), static_cast<size_t>(smem), s, mx, a1, b2, n1, rows,
+    if (launch_dependent(kern, dim3(grid), dim3((2 + 4 * 2 * 2) * 32), static_cast<size_t>(smem), s, mx, a1, b2, n1, static_cast<int>(rows),
                          static_cast<uint8_t*>(Xq), static_cast<__half*>(scales), Zdbg) != cudaSuccess)
       return SQ_ERR_CUDA;
   }

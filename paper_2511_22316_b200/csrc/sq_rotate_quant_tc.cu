@@ -353,9 +353,8 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
   const uint32_t limit = wait_limit();
 
   // One X tile set per token group: G tokens, XQ 64-column blocks each.
-  auto load_group = [&](int i) {
+  auto load_group = [&](int i, int s) {                  // group i -> ring stage s
     const int g = cta + i * ncta;
-    const int s = i % L.XS;
     mbar_arrive_expect_tx(&x_full[s], static_cast<uint32_t>(L.x_bytes));
     for (int tk = 0; tk < G; ++tk)
       for (int a = 0; a < XQ; ++a)
@@ -383,7 +382,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
     // Only now may a GEMM launched behind this kernel start: it requests its weights before it waits for
     // this kernel, and whatever precedes this kernel (sq_pack_weight, say) may have been writing them.
     griddep_launch_dependents();
-    for (int i = 0; i < preload; ++i) load_group(i);
+    for (int i = 0; i < preload; ++i) load_group(i, i);
     for (int b = 0; b < 4; ++b) {
       mbar_init(&x_empty[b], 1);
       mbar_init(&d1_full[b], 1);
@@ -404,9 +403,15 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
   if (warp == 0) {
     // ------------------------------ producer: keeps the X ring full -------------------------------------
     if (lane == 0) {
+      int s = 0;                                       // preload == XS here: ring stage and phase are counted along
+      uint32_t ph = 0;
       for (int i = preload; i < my_groups; ++i) {
-        if (!mbar_wait(&x_empty[i % L.XS], ((i / L.XS) & 1) ^ 1, RQ_X_EMPTY, limit)) break;
-        load_group(i);
+        if (!mbar_wait(&x_empty[s], ph, RQ_X_EMPTY, limit)) break;
+        load_group(i, s);
+        if (++s == L.XS) {
+          s = 0;
+          ph ^= 1;
+        }
       }
     }
   } else if (warp == 1) {
@@ -419,8 +424,8 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       const uint64_t x_desc0 = umma_desc_sw128_mn(smem_u32(xs), static_cast<uint32_t>(L.x_tile));
       const int ksteps1 = L.N1 / 16;                 // K = p, 16 per MMA
       bool ok = mbar_wait(img_full, 0, RQ_IMG, limit);
-      auto stage1 = [&](int i) {
-        const int slot = i % S, xs_i = i % L.XS;
+      auto stage1 = [&](int i, int xs_i) {
+        const int slot = i % S;
         tc_fence_after_sync();
         const uint32_t d1 = tmem_base + slot * SLOT_COLS;
         uint32_t acc = 0;
@@ -457,14 +462,21 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       // so stage 1 of the next group runs while the previous one is still being quantised out of the D2
       // columns; D2 is not written again before the group's warps have finished reading it, because
       // they convert the next group (which is what lets its stage 2 go) only after that.
-      int i1 = 0, i2 = 0;
+      // (Ring stage and phase of X are counted along: XS is a run-time number, and a division per poll cost more than what
+      // it polled for.)
+      int i1 = 0, i2 = 0, xr = 0;
+      uint32_t xph = 0;
       uint32_t idle = 0;
       while (ok && i2 < my_groups) {
         bool did = false;
         if (i1 < my_groups && i1 < i2 + S &&
-            mbar_test_wait(&x_full[i1 % L.XS], (i1 / L.XS) & 1) &&
+            mbar_test_wait(&x_full[xr], xph) &&
             mbar_test_wait(&d2_full[i1 % S], ((i1 / S) & 1) ^ 1)) {
-          stage1(i1++);
+          stage1(i1++, xr);
+          if (++xr == L.XS) {
+            xr = 0;
+            xph ^= 1;
+          }
           did = true;
         }
         if (i2 < i1 && mbar_test_wait(&a2_ready[i2 % S], (i2 / S) & 1)) {
