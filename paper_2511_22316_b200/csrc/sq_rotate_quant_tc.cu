@@ -139,11 +139,6 @@ __device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
-  F2 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
 __device__ __forceinline__ F2 f2_add_rd(F2 a, F2 b) {
   F2 d;
   asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -173,20 +168,24 @@ __device__ __forceinline__ void store_sector(void* p, const uint32_t* v, bool al
   }
 }
 
-// Eight rotated values -> one packed word: code = floor(z / Delta + 1/2), product and sum rounded on their own.
+// Eight rotated values -> one packed word: code = floor(z / Delta + 1/2), product and sum rounded on their own.  The sum is
+// taken one by one: as a pair behind the pair product it was contracted into a fused multiply-add for all its ".rn", and
+// one code in some 5e7 came out one lower.
 template <bool CLAMP>
 __device__ __forceinline__ uint32_t codes8(const float* z, F2 inv2) {
-  const F2 half2 = f2_pack(0.5f, 0.5f), magic2 = f2_pack(8388616.0f, 8388616.0f);
+  const F2 magic2 = f2_pack(8388616.0f, 8388616.0f);
   float u[8];
 #pragma unroll
   for (int e = 0; e < 8; e += 2) {
-    F2 t = f2_add(f2_mul(f2_pack(z[e], z[e + 1]), inv2), half2);
+    float a, b;
+    f2_unpack(f2_mul(f2_pack(z[e], z[e + 1]), inv2), a, b);
+    a = __fadd_rn(a, 0.5f);
+    b = __fadd_rn(b, 0.5f);
     if (CLAMP) {
-      float a, b;
-      f2_unpack(t, a, b);
-      t = f2_pack(fminf(fmaxf(a, -8.0f), 7.5f), fminf(fmaxf(b, -8.0f), 7.5f));
+      a = fminf(fmaxf(a, -8.0f), 7.5f);
+      b = fminf(fmaxf(b, -8.0f), 7.5f);
     }
-    f2_unpack(f2_add_rd(t, magic2), u[e], u[e + 1]);
+    f2_unpack(f2_add_rd(f2_pack(a, b), magic2), u[e], u[e + 1]);
   }
   return join8_codes(u);
 }

@@ -175,6 +175,26 @@ def test_rotate_outputs_16_byte_aligned_only(sq, n1, n2, M):
     assert all(np.array_equal(a, b) for a, b in zip(*got))
 
 
+# The decision itself, on enough codes to meet its ties: code = floor(fl(fl(z * inv) + 0.5)) of the z that the kernel
+# reports, no code excepted.  (A product and sum rounded together differ in one of some 5e7.)
+@pytest.mark.parametrize("n1,n2,M", [(64, 64, 32768), (172, 64, 8192), (112, 128, 8192), (64, 64, 32)])
+def test_quantiser_rounds_product_and_sum_on_their_own(sq, n1, n2, M):
+    torch, K = torch_mod(), n1 * n2
+    rng = np.random.default_rng(n1 + M)
+    X0 = rng.standard_normal((8, K)).astype(np.float32)
+    rot = sq.sq_build_rotation(X0, n1, n2, seed=3)
+    X = torch.randn(M, K, device="cuda", generator=torch.Generator(device="cuda").manual_seed(M)).mul_(0.02).half()
+    Xq = torch.empty(M, K // 2, dtype=torch.uint8, device="cuda")
+    sx, z = torch.empty(M, dtype=torch.float16, device="cuda"), torch.empty(M, K, dtype=torch.float32, device="cuda")
+    sq.sq_rotate_quant_act(rot, X, M, Xq, sx, z)
+    z.mul_((1.0 / sx.float()).unsqueeze(1))
+    z.add_(0.5)
+    z.floor_().clamp_(-8, 7)
+    want = z.view(M, K // 2, 2).to(torch.int8)
+    got_lo, got_hi = (Xq & 15).to(torch.int8), (Xq >> 4).to(torch.int8)
+    assert bool(torch.all(got_lo == (want[..., 0] & 15))) and bool(torch.all(got_hi == (want[..., 1] & 15)))
+
+
 def test_rotate_quant_tiny_config(sq):
     w = wl.TINY
     X = wl.make_activations(w)
