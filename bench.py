@@ -93,7 +93,7 @@ def gemm_kernel_name(w):
         return "w4a4_gemv_kernel"
     if decode:
         return "w4a4_gemm_decode_kernel"
-    if fast and w.M > 128 and w.N >= 128:
+    if fast and w.M > 64 and w.N >= 128:
         return "w4a4_gemm_pair_kernel"
     return "w4a4_gemm_tc_kernel" if fast else "w4a4_gemm_simple_kernel"
 
@@ -101,6 +101,8 @@ def gemm_kernel_name(w):
 def rotate_kernel_name(w, structured=False):
     if structured:
         return "rotate_quant_st_kernel"
+    if w.n2 == 32 and w.n1 <= 128:
+        return "rotate_quant_mma_kernel"
     if w.n2 in (64, 128) and w.n1 <= 128:
         return "rotate_quant_tc_kernel"
     if w.n2 in (64, 128) and w.n1 <= 256:

@@ -306,13 +306,13 @@ wo_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_const
 // MMA takes its A operand -- through shared memory the fp16 operand alone cost 128 KB of traffic per
 // 256 channels and bounded the kernel (20 us on 14336 x 4096 against 28.7 us with 64-channel stages,
 // whose hand-overs cost 920 cycles each).  A stage is a whole staging block: 256 channels, sixteen
-// MMAs.  Two converter groups alternate stages (a third group and a third operand stage changed
-// nothing).  What bounds a stage now, at about 1300 cycles: two things of about the same size -- the
-// sixteen MMAs of a stage take about 76 cycles each (with the converters idle a stage still takes 1220
-// cycles; a second issuing thread with an accumulator of its own, with or without a third converter
-// group, changed nothing, so it is the tensor pipe reading its 4 KB A operand out of tensor memory per
-// MMA, not the issue), and a converter group needs about as long to widen and move
-// the 64 KB fp16 operand of a stage into tensor memory.  Where the tiles alone leave most SMs idle
+// MMAs.  Two converter groups alternate stages.  A stage takes about 1050 cycles (clock stamps, 16 x 4096 ->
+// 14336): a converter group needs about 1020 for its 64 KB -- widening and the stores to tensor memory --
+// and can only start on a stage when the MMAs two stages back have retired; the issuing thread spends about
+// as long on the waits, the sixteen MMAs (18 cycles each with N = 16) and the commits of a stage.  Neither a
+// third operand stage (12.3 -> 12.8 us), nor fewer MMAs, nor weights that need no loading change the sum.
+// Weights and tokens have loading warps of their own: with one producer for both, the next weights were
+// not requested before a token stage had been freed (layer 19.4 -> 15.3 us).  Where the tiles alone leave most SMs idle
 // (4096 channels: 32 tiles) K is split over a cluster of 2 or 4 CTAs.  The accumulator holds one channel
 // per thread and the tokens along its registers; a warp's stores of one token cover 32 consecutive
 // channels.
