@@ -55,6 +55,10 @@ struct PairShape {
   static constexpr int THREADS = (WARP_EPI + EPI_WARPS) * 32;
   static_assert(TN == 128 || TN == 256, "whole accumulators in 256 columns; a chunk pair per epilogue warp");
   static_assert(S_OP >= 2 && S_OP <= 4, "the A ring has room for at most 4 blocks in TMEM");
+  // A group tells the phases of a stage apart by their parity, so it has to meet every one of them.  With five stages and
+  // two groups it met every other one, whose parities are the same: a group that ran ahead of a load still in flight took
+  // the stage's contents of ten blocks before for its own.
+  static_assert(S_OP % GROUPS == 0 && S_ST % GROUPS == 0, "a stage belongs to one group");
   static constexpr int B_ROWS = TN / 2;              // weight rows staged per CTA
   static constexpr int B_KB = B_ROWS * 128;          // int8 B half, one k-block
   static constexpr int B_OP = 2 * B_KB;
@@ -73,7 +77,7 @@ struct PairShape {
   static_assert(DYN_BYTES <= 227 * 1024, "shared memory of one SM");
 };
 using PairWide = PairShape<3, 3, 256, 1>;
-using PairNarrow = PairShape<4, 5, 128, 2>;
+using PairNarrow = PairShape<4, 6, 128, 2>;
 
 // 2-D fp16 map over Y [M x N]; box = 32 rows x 32 columns (64 bytes) with the 64-byte swizzle.
 bool make_out_map(CUtensorMap* map, void* Y, uint64_t M, uint64_t N) {

@@ -348,6 +348,7 @@ wo_gemm_tmem_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
   // reaches shared memory feeds two MMAs instead of one.
   static_assert(CT == 1 || CT == 2, "one or two channel tiles per token tile");
   static_assert(2 * NT + 128 * WOD_A_STAGES <= 512, "tensor-memory plan does not fit");
+  static_assert(SS % WOD_CONV_GROUPS == 0 && WOD_A_STAGES % WOD_CONV_GROUPS == 0, "a converter group meets every phase of its stages");
   constexpr int NBUF = 2 / CT;                           // accumulator sets that alternate between tiles
   constexpr int WOD_A_COL0 = 2 * NT > 128 ? 2 * NT : 128;
   griddep_launch_dependents();
@@ -714,6 +715,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(WP_THREADS, 1)
 wo_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_constant__ CUtensorMap tmap_w,
                     const __half* __restrict__ sw, int M, int N, int K, int tile_m, __half* __restrict__ Y) {
   using L = WoPairSmem<SS>;
+  static_assert(SS % WOD_CONV_GROUPS == 0, "a converter group meets every phase of its stages");
   griddep_launch_dependents();
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
