@@ -1170,19 +1170,22 @@ sq_status_t launch_wo_decode(const void* Z16, const void* Wq, const void* sw, in
   return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SQ_OK : SQ_ERR_CUDA;
 }
 
-// Token width of the CTA-pair kernel's tiles, a multiple of 16 from 64 to 256.  A tile of width w takes a time of about
-// w + 144 (fit of eleven widths on 777 x 11008 x 4096: 14.4 us at 96, 18.6 at 160, 24.4 at 256; the constant is the weights'
-// share of the operand supply and the hand-overs), and a batch that is no multiple of 256 tokens, or whose tiles do not
-// divide by the pairs, wastes part of the wide ones: 777 x 11008 x 4096 72 us in three waves of 256 (two thirds of the last
-// wave empty), 56 us in three full waves of 160.  The cost is waves x (w + 144), mixed with the same sum without rounding
-// up: what the chip as a whole has to move (2048 x 4096 x 4096: two waves of 240 measure 53.6 us, two of 256 50.9).
+// Token width of the CTA-pair kernel's tiles.  It is the N of a cta_group::2 MMA of M = 256 with A in tensor memory: a
+// multiple of 32 up to 256.  A tile of width w takes a time of about w + 70 (the constant is the weights' share of the
+// operand supply and the hand-overs), and a batch that is no multiple of 256 tokens, or whose tiles do not divide by the
+// pairs, wastes part of the wide ones: 777 x 11008 x 4096 72 us in three waves of 256 (two thirds of the last wave empty),
+// 54 us in three full waves of 160.  The cost is waves x (w + 70), mixed with the same sum without rounding up: what the
+// chip as a whole has to move.  Both constants from a fit to the seven widths on 199 shapes (70 to 2048 tokens, K 2048 to
+// 28672, 1024 to 32000 channels): the width taken is 0.1 % slower than the best on the geometric mean, more than 5 % on
+// two shapes (14 % at 2048 x 14336 x 4096, where 192 beats 256; a K-dependent term did not help).
+constexpr int WP_TILE_STEP = 32;
 int wo_pair_tile_m(int M, int N, int pairs) {
   const double ch_tiles = (N + 255) / 256;
   int best = 256;
   double best_cost = 0.0;
-  for (int w = 256; w >= 64; w -= 16) {
+  for (int w = 256; w >= 64; w -= WP_TILE_STEP) {
     const double load = ch_tiles * ((M + w - 1) / w) / pairs, waves = std::ceil(load);
-    const double cost = (0.6 * waves + 0.4 * load) * (w + 144);
+    const double cost = (0.8 * waves + 0.2 * load) * (w + 70);
     if (w == 256 || cost < best_cost) {
       best = w;
       best_cost = cost;

@@ -18,6 +18,7 @@ import pytest
 from oracle import singlequant_oracle as ora
 from paper_2511_22316_b200 import workloads as wl
 
+from csrc_util import wo_pair_widths
 from gpu_util import Guarded, dev, torch_mod
 
 pytestmark = pytest.mark.gpu
@@ -187,13 +188,21 @@ def test_wo_gemm_full_size_bit_exact_on_sampled_rows(sq, M, N, K):
         assert np.array_equal(Yg[rows, c0:c0 + 4096].view(np.uint16), Yo.view(np.uint16))
 
 
-# Token widths of the CTA-pair kernel's tiles from 64 up (one tile as wide as the batch, ragged last tiles, several waves),
-# and both sides of its line to the single-CTA form between 65 and 128 tokens.
-@pytest.mark.parametrize("M,N,K", [(65, 256, 64), (81, 264, 320), (97, 520, 256), (128, 4096, 128), (145, 256, 512),
-                                   (161, 264, 64), (177, 512, 192), (209, 256, 256), (241, 392, 128), (513, 4096, 128),
-                                   (777, 11008, 64), (100, 18944, 64), (100, 18952, 64)])
+# Every token width of the CTA-pair kernel's tiles (one tile as wide as the batch, ragged last tiles, several waves), and
+# both sides of its line to the single-CTA form between 65 and 128 tokens.
+WO_WIDTHS = [(65, 256, 64), (81, 264, 320), (97, 520, 256), (128, 4096, 128), (145, 256, 512),
+             (161, 264, 64), (177, 512, 192), (209, 256, 256), (241, 392, 128), (513, 4096, 128),
+             (777, 11008, 64), (100, 18944, 64), (65, 9480, 64), (97, 9480, 128), (129, 9480, 320), (161, 9480, 64),
+             (193, 9480, 192), (225, 9480, 128), (100, 18952, 64)]
+
+
+@pytest.mark.parametrize("M,N,K", WO_WIDTHS)
 def test_wo_gemm_tile_widths_bit_exact(sq, M, N, K):
     test_wo_gemm_is_bit_exact_on_small_integers(sq, M, N, K)
+
+
+def test_the_tile_width_shapes_reach_every_width():
+    assert set(wo_pair_widths([(M, N) for M, N, _ in WO_WIDTHS[:-1]])) == set(range(64, 257, 32))
 
 
 def test_wo_gemm_random_shapes_bit_exact(sq):

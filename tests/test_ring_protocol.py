@@ -5,13 +5,9 @@ Two groups of converter warps take the blocks of a ring in turn and tell the pha
 interleaving of loads, groups and MMAs for a ring of given depth and reports whether a group can be let through to a
 block whose load has not landed.  The depths are taken out of the sources by compiling the kernels' layout structs.
 """
-import os
-import re
-import subprocess
-
 import pytest
 
-CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2511_22316_b200", "csrc")
+from csrc_util import block, lines, run, source
 
 
 def let_through_too_early(stages, op_stages, groups, operand_first=False, blocks=None):
@@ -72,21 +68,11 @@ def test_the_model_tells_sound_rings_from_unsound_ones():
     assert let_through_too_early(3, 3, 1) is None
 
 
-def _block(text, head):
-    """The struct that `head` opens, to its closing brace."""
-    start = text.index(head)
-    end = text.index("\n};", start)
-    return text[start:end + 3]
-
-
 @pytest.fixture(scope="module")
-def rings(tmp_path_factory):
-    pair = open(os.path.join(CSRC, "sq_gemm_pair.cu")).read()
-    dec = open(os.path.join(CSRC, "sq_gemm_decode.cu")).read()
-    consts = "\n".join(re.findall(r"^constexpr int D_.*$", dec, re.M))
-    src = ("#include <cstdio>\n" + _block(pair, "template <int S_OP_, int S_ST_") + "\n"
-           + "\n".join(re.findall(r"^using Pair\w+ = .*$", pair, re.M)) + "\n" + consts + "\n"
-           + _block(dec, "template <int NT>\nstruct DecSmem") + """
+def rings():
+    pair, dec = source("sq_gemm_pair.cu"), source("sq_gemm_decode.cu")
+    rows = run(block(pair, "template <int S_OP_, int S_ST_") + lines(pair, r"^using Pair\w+ = .*$") + "\n"
+               + lines(dec, r"^constexpr int D_.*$") + "\n" + block(dec, "template <int NT>\nstruct DecSmem") + """
 template <class P> void pair(const char* n) { printf("%s %d %d %d 0\\n", n, P::S_ST, P::S_OP, P::GROUPS); }
 template <int NT> void dec() {
   using L = DecSmem<NT>;
@@ -95,11 +81,7 @@ template <int NT> void dec() {
 }
 int main() { pair<PairWide>("wide"); pair<PairNarrow>("narrow"); dec<16>(); dec<32>(); dec<64>(); }
 """)
-    d = tmp_path_factory.mktemp("rings")
-    (d / "rings.cpp").write_text(src)
-    subprocess.run(["g++", "-std=c++17", "-o", str(d / "rings"), str(d / "rings.cpp")], check=True)
-    out = subprocess.run([str(d / "rings")], check=True, capture_output=True, text=True).stdout
-    return {line.split()[0]: tuple(int(v) for v in line.split()[1:]) for line in out.splitlines()}
+    return {row[0]: tuple(int(v) for v in row[1:]) for row in rows}
 
 
 @pytest.mark.parametrize("name", ["wide", "narrow", "decode_w16", "decode_x16", "decode_w32", "decode_x32", "decode_w64",
