@@ -72,7 +72,8 @@ __host__ __device__ inline RqLayout rq_layout(int n1, int n2, int budget = kMaxD
   L.off_a1 = 0;
   L.off_b2 = L.off_a1 + L.a1_bytes;
   L.off_x = L.off_b2 + L.b2_bytes;
-  const int extra = (n2 == 128) ? 2048 : 0;       // per-lane absmax swap of the eight-warp slot form
+  // per-lane absmax swap of the forms with eight warps per slot: [slots][2][128 lanes] floats, behind the barriers
+  const int extra = one_token ? 1024 : (n2 == 128 ? 2048 : 0);
   const int room = budget - 1024 - 512 - extra - L.off_x;
   const int xs = room / L.x_bytes;
   L.XS = xs > 4 ? 4 : xs;                         // X ring depth

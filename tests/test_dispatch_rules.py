@@ -9,3 +9,24 @@ def test_weight_only_pair_widths_are_instruction_shapes():
     shapes = [(M, N) for M in range(65, 2100, 37) for N in (256, 264, 1024, 4096, 5120, 9480, 11008, 14336, 18944, 32000)]
     widths = csrc_util.wo_pair_widths(shapes)
     assert set(widths) == set(range(64, 257, 32))
+
+
+def test_rotate_layouts_hold_all_that_the_kernel_writes():
+    """The forms with eight warps per accumulator slot swap a maximum per lane, 1024 bytes a slot, 512 bytes behind the
+    start of the barrier area; 1024 bytes on top of the layout belong to its alignment."""
+    tc = csrc_util.source("sq_rotate_quant_tc.cu")
+    rows = csrc_util.run(
+        csrc_util.lines(tc, r"^constexpr int k(?:Max|Half)DynSmem.*$") + "\n" + csrc_util.block(tc, "struct RqLayout")
+        + csrc_util.block(tc, "__host__ __device__ inline RqLayout rq_layout(") + """
+int main() {
+  for (int n2 = 64; n2 <= 128; n2 *= 2)
+    for (int n1 = 1; n1 <= 128; ++n1)
+      for (int few = 0; few < 2; ++few) {
+        const RqLayout L = rq_layout(n1, n2, kMaxDynSmem, few);
+        const int swap_slots = few ? 1 : (n2 == 128 ? 2 : 0);          // slots of eight warps
+        printf("%d %d %d %d %d %d\\n", n1, n2, few, L.off_misc + 512 + 1024 * swap_slots, L.total, L.XS);
+      }
+}""")
+    assert len(rows) == 2 * 128 * 2
+    for n1, n2, few, end, total, stages in (map(int, r) for r in rows):
+        assert end <= total and total + 1024 <= 227 * 1024 and stages >= 2, (n1, n2, few)
