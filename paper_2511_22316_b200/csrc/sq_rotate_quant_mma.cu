@@ -82,6 +82,12 @@ constexpr int rm_smem(int NT, int PW) {
   return ntt / 2 * ntt * 512 + RM_SLICES * RM_A2_SLICE + (PW > 1 ? RM_SLICES * 2 * (ntt / 2) * 512 : 0) + 128;
 }
 
+// Tokens cta, cta + ncta, ... of `rows`: how many there are.  Unsigned, since rows goes up to 2^31 - 1 and the token behind
+// the last one may lie beyond that.
+__host__ __device__ inline int rm_tokens(int cta, int ncta, int rows) {
+  return rows > cta ? static_cast<int>((static_cast<unsigned>(rows - cta) + static_cast<unsigned>(ncta - 1)) / static_cast<unsigned>(ncta)) : 0;
+}
+
 template <int NT, int PW>
 __global__ void __launch_bounds__(RM_SLICES * PW * 32, 3)
 rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restrict__ b1_img, int n1, int rows,
@@ -119,8 +125,8 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
   griddep_launch_dependents();                         // not earlier: see the tcgen05 kernel
   __syncthreads();                                     // the barrier exists
   uint4 x[NT];
-  auto load_x = [&](int token) {
-    const __half* xt = X + static_cast<size_t>(token) * n + c * 8;
+  auto load_x = [&](long long token) {
+    const __half* xt = X + token * n + c * 8;
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
       const int p = (part * NT + t) * 8 + g;
@@ -131,7 +137,8 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
   int par = 0;
   load_x(blockIdx.x);
   const bool ok = mbar_wait(bar, 0, RM_B1, limit);
-  for (int token = blockIdx.x; token < rows; token += gridDim.x, par ^= 1) {
+  long long token = blockIdx.x;
+  for (int left = rm_tokens(blockIdx.x, gridDim.x, rows); left > 0; --left, token += gridDim.x, par ^= 1) {
     // ---- stage 1 ------------------------------------------------------------------------------------------
     float T[NT][4];
 #pragma unroll
@@ -147,7 +154,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
 #pragma unroll
       for (int t = 0; t < NT; ++t) mma_f16_16816(T[t], l, s ? x[t].z : x[t].x, s ? x[t].w : x[t].y);
     }
-    if (token + static_cast<int>(gridDim.x) < rows) load_x(token + gridDim.x);      // the next token's rows
+    if (left > 1) load_x(token + gridDim.x);      // the next token's rows
     // ---- T -> fp16 hi + lo, scaled so that the slice's largest entry lands in [2^13, 2^14) ----------------------
     float tm = 0.0f;
 #pragma unroll
@@ -217,7 +224,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
     }
     // z[t][e], z[t][2 + e]: channels q' = 16 m + 2 g, + 1 of row p' = 8 (part NT + t) + 2 c + e.
     if (qmax == 0) {                                   // rotation only: fp16 rows out
-      __half* zrow = reinterpret_cast<__half*>(Xq) + static_cast<size_t>(token) * n + m * 16 + 2 * g;
+      __half* zrow = reinterpret_cast<__half*>(Xq) + token * n + m * 16 + 2 * g;
 #pragma unroll
       for (int t = 0; t < NT; ++t)
 #pragma unroll
@@ -245,7 +252,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
     const float inv_un = inv * un;                     // exact: un is a power of two
     // Delta >= 2^-14 (a normal fp16) bounds |z / Delta| by qmax (1 + 2^-11): no clamp is needed then.
     const bool clamp = __half2float(delta) < 6.103515625e-05f;
-    uint8_t* orow = Xq + static_cast<size_t>(token) * (n / 2) + m * 8;
+    uint8_t* orow = Xq + token * (n / 2) + m * 8;
 #pragma unroll
     for (int gr = 0; gr < (NT + 3) / 4; ++gr) {
       uint32_t w[2];
@@ -269,7 +276,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
       if (t < NT && p < n1 && ok) *reinterpret_cast<uint2*>(orow + p * (N2 / 2)) = out;
     }
     if (Zdbg != nullptr) {
-      float* zrow = Zdbg + static_cast<size_t>(token) * n + m * 16 + 2 * g;
+      float* zrow = Zdbg + token * n + m * 16 + 2 * g;
 #pragma unroll
       for (int t = 0; t < NT; ++t)
 #pragma unroll

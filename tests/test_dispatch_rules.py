@@ -30,3 +30,14 @@ int main() {
     assert len(rows) == 2 * 128 * 2
     for n1, n2, few, end, total, stages in (map(int, r) for r in rows):
         assert end <= total and total + 1024 <= 227 * 1024 and stages >= 2, (n1, n2, few)
+
+
+@pytest.mark.parametrize("rows,ncta", [(1, 1), (5, 5), (1300, 1184), (2 ** 31 - 1, 1184), (2 ** 31 - 1, 444), (2 ** 31 - 100, 740)])
+def test_warp_level_rotation_counts_its_tokens_beyond_32_bits(rows, ncta):
+    """n = 32 fits 2^31 - 1 rows on one GPU; the counts of all blocks add up to the rows, and no block's is negative."""
+    code = csrc_util.block(csrc_util.source("sq_rotate_quant_mma.cu"), "__host__ __device__ inline int rm_tokens(")
+    got = csrc_util.run(code + """
+int main(int, char** v) { for (int c = 0; c < atoi(v[1]); ++c) printf("%d\\n", rm_tokens(c, atoi(v[1]), atoi(v[2]))); }
+""", ncta, rows)
+    counts = [int(r[0]) for r in got]
+    assert counts == [(rows - c + ncta - 1) // ncta for c in range(ncta)] and sum(counts) == rows
