@@ -92,7 +92,7 @@ sq_status_t rotate_quant_dispatch(const sq_rotation* h, const void* X, int64_t r
 }
 // Step 1 alone, fp16 rows out (weight-only variant): the same kernels in their rotation-only form.
 sq_status_t rotate_f16_dispatch(const sq_rotation* h, const void* X, int64_t rows, void* Z16, cudaStream_t s) {
-  if (h->dMmaImg) return launch_rotate_quant_mma(h, X, rows, Z16, nullptr, nullptr, s, 0);
+  if (h->dMmaImg) return launch_rotate_quant_mma(h, X, rows, Z16, nullptr, nullptr, s, true);
   if (h->tc_ready) return launch_rotate_quant_tc(h, X, rows, Z16, nullptr, nullptr, s, true);
   if (h->tc_pair) return launch_rotate_quant_pair(h, X, rows, Z16, nullptr, nullptr, s, true);
   return launch_rotate_quant(h->dR1, h->dR2, h->n1, h->n2, X, rows, Z16, nullptr, nullptr, s, 0);
@@ -489,9 +489,7 @@ sq_status_t sq_pack_weight_wo(const sq_rotation_t* rot_or_null, const void* W, i
     st = sq::launch_rotate_quant(nullptr, nullptr, 1, static_cast<int>(K), W, N, Wq, sw, nullptr, s, qmax);
   else if (bits == 4)
     st = sq::rotate_quant_dispatch(rot_or_null, W, N, Wq, sw, nullptr, s);
-  else if (rot_or_null->dMmaImg)      // other widths: the kernels that take the number of levels as an argument
-    st = sq::launch_rotate_quant_mma(rot_or_null, W, N, Wq, sw, nullptr, s, qmax);
-  else
+  else      // 3 bits: always the fp32 kernel.  Through another kernel a few codes in a million differ, and a step of 3 bits is large.
     st = sq::launch_rotate_quant(rot_or_null->dR1, rot_or_null->dR2, rot_or_null->n1, rot_or_null->n2, W, N, Wq, sw,
                                  nullptr, s, qmax);
   if (st != SQ_OK) return st;

@@ -138,11 +138,11 @@ bool rotate_quant_pair_supported(int n1, int n2);
 bool rotate_quant_pair_prepare(sq_rotation* h);
 sq_status_t launch_rotate_quant_pair(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales,
                                      float* Zdbg, cudaStream_t s, bool f16out = false);
-// Warp-level variant (sq_rotate_quant_mma.cu): n2 = 32.  qmax as in launch_rotate_quant.
+// Warp-level variant (sq_rotate_quant_mma.cu): n2 = 32.
 bool rotate_quant_mma_supported(int n1, int n2);
 bool rotate_quant_mma_prepare(sq_rotation* h);
 sq_status_t launch_rotate_quant_mma(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales, float* Zdbg,
-                                    cudaStream_t s, int qmax = 7);
+                                    cudaStream_t s, bool f16out = false);
 // Steps 1+2 with R2 applied through its structure (sq_rotate_quant_st.cu): R1^T on the tensor cores,
 // then the Hadamard butterflies and the two rotation chains of URT in registers.
 bool rotate_quant_st_prepare(sq_rotation* h);

@@ -92,7 +92,7 @@ template <int NT, int PW>
 __global__ void __launch_bounds__(RM_SLICES * PW * 32, 3)
 rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restrict__ b1_img, int n1, int rows,
                         const __half* __restrict__ X, uint8_t* __restrict__ Xq, __half* __restrict__ scales,
-                        float* __restrict__ Zdbg, int qmax) {
+                        float* __restrict__ Zdbg, bool f16out) {
   constexpr int N2 = RM_N2, WARPS = RM_SLICES * PW;
   constexpr int NTT = NT * PW, KJ = NTT / 2;           // p tiles, k-steps of stage 2
   static_assert(NTT % 2 == 0, "whole k-steps");
@@ -223,7 +223,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
       for (int t = 0; t < NT; ++t) mma_f16_16816(z[t], h, b[t].z, b[t].w);      // hi * lo
     }
     // z[t][e], z[t][2 + e]: channels q' = 16 m + 2 g, + 1 of row p' = 8 (part NT + t) + 2 c + e.
-    if (qmax == 0) {                                   // rotation only: fp16 rows out
+    if (f16out) {                                      // rotation only: fp16 rows out
       __half* zrow = reinterpret_cast<__half*>(Xq) + token * n + m * 16 + 2 * g;
 #pragma unroll
       for (int t = 0; t < NT; ++t)
@@ -248,9 +248,9 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
     for (int w = 1; w < WARPS; ++w) amax = fmaxf(amax, zp[w]);
     __half delta;
     float inv;
-    row_scale(amax, delta, inv, qmax);
+    row_scale(amax, delta, inv);
     const float inv_un = inv * un;                     // exact: un is a power of two
-    // Delta >= 2^-14 (a normal fp16) bounds |z / Delta| by qmax (1 + 2^-11): no clamp is needed then.
+    // Delta >= 2^-14 (a normal fp16) bounds |z / Delta| by 7 (1 + 2^-11): no clamp is needed then.
     const bool clamp = __half2float(delta) < 6.103515625e-05f;
     uint8_t* orow = Xq + token * (n / 2) + m * 8;
 #pragma unroll
@@ -265,7 +265,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
 #pragma unroll
           for (int o = 0; o < 2; ++o) {
             float v = t < NT ? __fadd_rn(__fmul_rn(z[t < NT ? t : 0][2 * o + e], inv_un), 0.5f) : 0.0f;
-            if (clamp) v = fminf(fmaxf(v, -1.0f - static_cast<float>(qmax)), static_cast<float>(qmax) + 0.5f);
+            if (clamp) v = fminf(fmaxf(v, -8.0f), 7.5f);
             tt[2 * i + o] = v;
           }
         }
@@ -290,7 +290,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
 }
 
 template <int NT, int PW>
-sq_status_t launch_rm(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales, float* Zdbg, int qmax,
+sq_status_t launch_rm(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales, float* Zdbg, bool f16out,
                       cudaStream_t s) {
   const int sms = sm_count();
   if (sms <= 0) return SQ_ERR_CUDA;
@@ -305,7 +305,7 @@ sq_status_t launch_rm(const sq_rotation* h, const void* X, int64_t rows, void* X
   const cudaError_t err = launch_dependent(kern, dim3(static_cast<unsigned>((rows + per - 1) / per)), dim3(RM_SLICES * PW * 32),
                                            static_cast<size_t>(smem), s, a2, b1, static_cast<int>(h->n1), static_cast<int>(rows),
                                            static_cast<const __half*>(X), static_cast<uint8_t*>(Xq),
-                                           static_cast<__half*>(scales), Zdbg, qmax);
+                                           static_cast<__half*>(scales), Zdbg, f16out);
   count_launch();
   return err == cudaSuccess ? SQ_OK : SQ_ERR_CUDA;
 }
@@ -358,19 +358,19 @@ bool rotate_quant_mma_prepare(sq_rotation* h) {
 }
 
 sq_status_t launch_rotate_quant_mma(const sq_rotation* h, const void* X, int64_t rows, void* Xq, void* scales, float* Zdbg,
-                                    cudaStream_t s, int qmax) {
+                                    cudaStream_t s, bool f16out) {
   if (rows > 0x7FFFFFFF) return SQ_ERR_UNSUPPORTED;
   const RmShape sh = rm_shape(h->n1);
   if (sh.PW == 1) {
-    if (sh.NT == 2) return launch_rm<2, 1>(h, X, rows, Xq, scales, Zdbg, qmax, s);
-    if (sh.NT == 4) return launch_rm<4, 1>(h, X, rows, Xq, scales, Zdbg, qmax, s);
-    if (sh.NT == 6) return launch_rm<6, 1>(h, X, rows, Xq, scales, Zdbg, qmax, s);
-    return launch_rm<8, 1>(h, X, rows, Xq, scales, Zdbg, qmax, s);
+    if (sh.NT == 2) return launch_rm<2, 1>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+    if (sh.NT == 4) return launch_rm<4, 1>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+    if (sh.NT == 6) return launch_rm<6, 1>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+    return launch_rm<8, 1>(h, X, rows, Xq, scales, Zdbg, f16out, s);
   }
-  if (sh.NT == 5) return launch_rm<5, 2>(h, X, rows, Xq, scales, Zdbg, qmax, s);
-  if (sh.NT == 6) return launch_rm<6, 2>(h, X, rows, Xq, scales, Zdbg, qmax, s);
-  if (sh.NT == 7) return launch_rm<7, 2>(h, X, rows, Xq, scales, Zdbg, qmax, s);
-  return launch_rm<8, 2>(h, X, rows, Xq, scales, Zdbg, qmax, s);
+  if (sh.NT == 5) return launch_rm<5, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+  if (sh.NT == 6) return launch_rm<6, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+  if (sh.NT == 7) return launch_rm<7, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+  return launch_rm<8, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
 }
 
 }  // namespace sq

@@ -80,6 +80,35 @@ def test_pack_weight_wo_identity_rotation_is_bit_exact(sq, bits):
     assert np.array_equal(s.numpy(np.float16, (N,)).view(np.uint16), sw_o.view(np.uint16))
 
 
+# 3-bit codes come from the fp32 kernel whatever n2 is: T[p][q'] = sum_q x R2 and z = sum_p R1 T as chains of fused
+# multiply-adds in rising q and p.  In float64 the products are exact and a sum rounds twice, which can move a value by one
+# ulp in some 2^29 of them: bytes are compared exactly all the same.
+@pytest.mark.parametrize("n1,n2,N", [(16, 32, 4096), (64, 32, 4096), (128, 32, 4096), (64, 64, 1024), (48, 128, 1024)])
+def test_three_bit_codes_are_those_of_the_fp32_kernel(sq, n1, n2, N):
+    torch, K = torch_mod(), n1 * n2
+    rng = np.random.default_rng(n1 + n2)
+    rot = sq.sq_build_rotation(rng.standard_normal((8, K)).astype(np.float32), n1, n2, seed=4)
+    R1, R2 = (torch.from_numpy(r).cuda().double() for r in rot.factors())
+    W = torch.randn(N, K, device="cuda", generator=torch.Generator(device="cuda").manual_seed(n1)).mul_(0.02).half()
+    x = W.double().view(N, n1, n2)
+    T, z = torch.zeros_like(x), torch.zeros_like(x)
+    for q in range(n2):
+        T = (x[:, :, q:q + 1] * R2[q] + T).float().double()
+    for p in range(n1):
+        z = (R1[p].view(1, n1, 1) * T[:, p:p + 1, :] + z).float().double()
+    z = z.float().view(N, K)
+    step = (z.abs().amax(1) / 3.0).half()
+    t = z * (1.0 / step.float()).view(N, 1)
+    codes = (t + 0.5).floor().clamp(-4, 3).to(torch.int8)
+    q, s = Guarded(N * K // 2), Guarded(N * 2)
+    sq.sq_pack_weight_wo(rot, W, N, K, 3, q, s)
+    _sync_ok(sq)
+    q.check(); s.check()
+    assert np.array_equal(s.numpy(np.uint16, (N,)), step.cpu().numpy().view(np.uint16))
+    assert np.array_equal(q.numpy(np.uint8, (N, K // 2)), ora.pack_int4_interleaved(codes.cpu().numpy()))
+    rot.close()
+
+
 def test_weight_only_argument_checks(sq):
     lib = sq.load()
     w = wl.small("woarg", 8, 8, 8, 16, 5)
