@@ -1,26 +1,28 @@
-// Steps 1+2 on warp-level tensor instructions: factor pairs with n2 = 32 (n1 <= 128), any number of rows.
+// Steps 1+2 on warp-level tensor instructions in float64: factor pairs with n2 = 32 (n1 <= 128), any number of rows.
 //
 // The tcgen05 kernels want n2 = 64 or 128; the narrow layers of small models (512, 1024, 2048 channels) went through the
 // fp32 kernel, which is bound by its multiply-adds.  Here a warp carries 16 columns q' of a token through both stages:
 //
-//   stage 1  T^T[q'][p]  = sum_q R2^T[q'][q] X^T[q][p]    A = R2^T (shared memory, fp16 hi + lo), B = X^T: the token's
-//                                                         rows as they lie in memory, 16 bytes per lane, exact fp16
+//   stage 1  T^T[q'][p]  = sum_q R2^T[q'][q] X^T[q][p]    A = R2^T (shared memory), B = X^T: the token's rows as they lie
+//                                                         in memory, 16 bytes per lane
 //   stage 2  Z^T[q'][p'] = sum_p T^T[q'][p] R1[p][p']     A = T^T: the accumulators of stage 1 are in the layout of
-//                                                         this operand (fp16 hi + lo, one power-of-two scale),
-//                                                         B = R1 (shared memory, fp16 hi + lo)
-// with the split, the passes (hi*hi + lo*hi + hi*lo) and the 2^10 pre-scale of the factors as in the tcgen05 kernel: the
-// result keeps fp32 accuracy.  For n1 > 64 the p axis is cut over two warps: each makes its part of T and of Z, and the
-// fp16 operand of stage 2 goes through shared memory once.  A CTA (two or four warps) owns a token at a time; its warps
-// meet for the absmax.
+//                                                         this operand, B = R1 (shared memory, as fp32)
+// Both are mma.sync m16n8k16 in float64, rounded once to fp32 at the end.  The unit runs at half the fp32 rate, which these
+// sizes do not feel, and it takes any fp32 factor and passes infinities and NaN on as the fp32 kernel does.  Operands split
+// into two fp16 numbers (the tcgen05 kernels' way) were faster on many rows, 2048 x 4096 in 26 us, but two to three times as
+// far from float64 as the fp32 kernel, NaN for factors beyond 64, and finite codes for tokens with infinities.
+// For n1 > 64 the p axis is cut over two warps: each makes its part of T and of Z, and the operand of stage 2 goes through
+// shared memory once.  A CTA (two or four warps) owns a token at a time; its warps meet for the absmax.
 //
 // Operand order.  k-slots may stand for any channel as long as A and B agree: lane (g, c) loads q = 8 c .. 8 c + 7 of row
 // p = 8 t + g, and the eight halves are the b registers of both k-steps; the image of R2^T is stored in that order.  Rows
 // g and g + 8 of the m16 tile stand for q' = 2 g and 2 g + 1, so that a thread holds the two codes of a byte; three
 // shuffles turn eight lanes' bytes into eight-byte pieces of the packed row.
 //
-// Bound by latency at these sizes (one token is 0.1 to 0.3 us of products).  Measured against the fp32 kernel, back-to-back
-// launches: 64 x 512 (16 x 32) 4.8 -> 1.7 us, 1024 x 2048 (64 x 32) 20.6 -> 5.9 us, 2048 x 4096 (128 x 32) 113 -> 26 us;
-// fp16 rows out 64 x 512 7.2 -> 1.5 us.
+// Few rows are bound by the latency of a token's products, many by the float64 unit: 8192 x 4096 (128 x 32) runs it at
+// 16.2 TFMA/s, 87 % of its 64 per cycle and SM.  Measured against the fp32 kernel, back-to-back launches: 64 x 512
+// (16 x 32) 5.0 -> 1.9 us, 300 x 2048 (64 x 32) 11.3 -> 7.0 us, 2048 x 4096 (128 x 32) 111 -> 84 us; fp16 rows out 64 x 512
+// 7.4 -> 1.7 us.  Distance of z from float64: 2.5e-8 of it (the one rounding), the fp32 kernel's 1.0e-7 to 2.6e-7.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -34,10 +36,18 @@ namespace {
 
 enum RmSite : uint32_t { RM_B1 = 112 };
 
-__device__ __forceinline__ void mma_f16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+// Fragments: a[2 i], a[2 i + 1] rows g and g + 8 of k = c + 4 i; b[i] column g of k = c + 4 i; d rows g, g + 8 (d[2], d[3]),
+// columns 2 c, 2 c + 1.
+__device__ __forceinline__ void mma_f64_16816(double (&d)[4], const double (&a)[8], const double (&b)[4]) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5, %6, %7, %8, %9, %10, %11}, "
+      "{%12, %13, %14, %15}, {%0, %1, %2, %3};"
+      : "+d"(d[0]), "+d"(d[1]), "+d"(d[2]), "+d"(d[3])
+      : "d"(a[0]), "d"(a[1]), "d"(a[2]), "d"(a[3]), "d"(a[4]), "d"(a[5]), "d"(a[6]), "d"(a[7]), "d"(b[0]), "d"(b[1]), "d"(b[2]),
+        "d"(b[3]));
+}
+__device__ __forceinline__ void halves_to_f64(uint32_t w0, uint32_t w1, double (&b)[4]) {
+  const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&w0)), f1 = __half22float2(*reinterpret_cast<const __half2*>(&w1));
+  b[0] = f0.x; b[1] = f0.y; b[2] = f1.x; b[3] = f1.y;
 }
 
 // Token bytes the kernel before this one may just have written: past the L1 cache.
@@ -60,26 +70,30 @@ __device__ __forceinline__ uint2 transpose_bytes_8(uint32_t w0, uint32_t w1, int
   return make_uint2(__byte_perm(s0, s1, 0x5140), __byte_perm(s0, s1, 0x7362));
 }
 
-// Tiles of eight p per warp (NT) and warps per q' slice (PW) for n1; the padded n1 is 8 * NT * PW.
+// Tiles of eight p per warp (NT) and warps per q' slice (PW) for n1; the padded n1 is 8 * NT * PW.  Few tiles per warp and
+// more warps, as far as the padding stays small: with few rows a token's chain of products is all there is (one token of
+// 64 x 32: 5.8 us with eight tiles and one warp, 3.4 with two and four).
 struct RmShape { int NT, PW; };
 inline RmShape rm_shape(int n1) {
-  if (n1 <= 16) return {2, 1};
-  if (n1 <= 32) return {4, 1};
-  if (n1 <= 48) return {6, 1};
-  if (n1 <= 64) return {8, 1};
+  if (n1 <= 16) return {1, 2};
+  if (n1 <= 32) return {2, 2};
+  if (n1 <= 48) return {3, 2};
+  if (n1 <= 64) return {2, 4};
   if (n1 <= 80) return {5, 2};
-  if (n1 <= 96) return {6, 2};
+  if (n1 <= 96) return {3, 4};
   if (n1 <= 112) return {7, 2};
-  return {8, 2};
+  return {4, 4};
 }
+// Blocks that share an SM: what the registers allow, or fewer where that measured faster.
+constexpr int rm_ctas(int NT, int PW) { return PW == 4 ? (NT == 4 ? 2 : 3) : (NT == 1 ? 8 : (NT <= 3 ? 4 : 3)); }
 
 constexpr int RM_N2 = 32, RM_SLICES = RM_N2 / 16;      // q' slices of a token, PW warps each
 
-// Shared memory: [R1 operand][R2^T operand][T operand, PW > 1: slice x (hi, lo) x k-step x half x lane x 8 B][maxima, barrier].
-constexpr int RM_A2_SLICE = RM_N2 / 16 * 1024;
+// Shared memory: [R1 operand, fp32][R2^T operand][T operand, PW > 1: slice x tile x half x lane x 16 B][maxima, barrier].
+constexpr int RM_A2_SLICE = RM_N2 * 32 / 4 * 16;
 constexpr int rm_smem(int NT, int PW) {
   const int ntt = NT * PW;
-  return ntt / 2 * ntt * 512 + RM_SLICES * RM_A2_SLICE + (PW > 1 ? RM_SLICES * 2 * (ntt / 2) * 512 : 0) + 128;
+  return ntt / 2 * ntt * 512 + RM_SLICES * RM_A2_SLICE + (PW > 1 ? RM_SLICES * ntt * 1024 : 0) + 128;
 }
 
 // Tokens cta, cta + ncta, ... of `rows`: how many there are.  Unsigned, since rows goes up to 2^31 - 1 and the token behind
@@ -89,21 +103,20 @@ __host__ __device__ inline int rm_tokens(int cta, int ncta, int rows) {
 }
 
 template <int NT, int PW>
-__global__ void __launch_bounds__(RM_SLICES * PW * 32, 3)
-rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restrict__ b1_img, int n1, int rows,
+__global__ void __launch_bounds__(RM_SLICES * PW * 32, rm_ctas(NT, PW))
+rotate_quant_mma_kernel(const double2* __restrict__ a2_img, const float4* __restrict__ b1_img, int n1, int rows,
                         const __half* __restrict__ X, uint8_t* __restrict__ Xq, __half* __restrict__ scales,
                         float* __restrict__ Zdbg, bool f16out) {
   constexpr int N2 = RM_N2, WARPS = RM_SLICES * PW;
   constexpr int NTT = NT * PW, KJ = NTT / 2;           // p tiles, k-steps of stage 2
   static_assert(NTT % 2 == 0, "whole k-steps");
   constexpr int B1_BYTES = KJ * NTT * 512, A2_BYTES = RM_SLICES * RM_A2_SLICE;
-  constexpr int T_BYTES = PW > 1 ? RM_SLICES * 2 * KJ * 512 : 0;
+  constexpr int T_BYTES = PW > 1 ? RM_SLICES * NTT * 1024 : 0;
   extern __shared__ __align__(128) unsigned char rm_smem_raw[];
-  uint4* b1s = reinterpret_cast<uint4*>(rm_smem_raw);
+  const float4* b1s = reinterpret_cast<const float4*>(rm_smem_raw);
   unsigned char* a2s = rm_smem_raw + B1_BYTES;
-  uint2* ts = reinterpret_cast<uint2*>(a2s + A2_BYTES);                    // [slice][hi, lo][k-step][half][lane]
+  double2* ts = reinterpret_cast<double2*>(a2s + A2_BYTES);                // [slice][tile][even, odd p][lane]
   float* zmax = reinterpret_cast<float*>(a2s + A2_BYTES + T_BYTES);        // [2][WARPS]: of the token
-  float* tmax = zmax + 16;                                                 // [WARPS]: of T (PW > 1)
   uint64_t* bar = reinterpret_cast<uint64_t*>(zmax + 28);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
@@ -133,95 +146,77 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
       x[t] = p < n1 ? ld_token16(xt + p * N2) : make_uint4(0u, 0u, 0u, 0u);
     }
   };
-  const uint4* a2 = reinterpret_cast<const uint4*>(a2s + m * RM_A2_SLICE) + lane;
+  const double2* a2 = reinterpret_cast<const double2*>(a2s + m * RM_A2_SLICE) + lane;
   int par = 0;
   load_x(blockIdx.x);
   const bool ok = mbar_wait(bar, 0, RM_B1, limit);
   long long token = blockIdx.x;
   for (int left = rm_tokens(blockIdx.x, gridDim.x, rows); left > 0; --left, token += gridDim.x, par ^= 1) {
     // ---- stage 1 ------------------------------------------------------------------------------------------
-    float T[NT][4];
+    double T[NT][4];
 #pragma unroll
     for (int t = 0; t < NT; ++t)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) T[t][e] = 0.0f;
+      for (int e = 0; e < 4; ++e) T[t][e] = 0.0;
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-      const uint4 h4 = a2[(s * 2 + 0) * 32], l4 = a2[(s * 2 + 1) * 32];
-      const uint32_t h[4] = {h4.x, h4.y, h4.z, h4.w}, l[4] = {l4.x, l4.y, l4.z, l4.w};
+      double a[8];
 #pragma unroll
-      for (int t = 0; t < NT; ++t) mma_f16_16816(T[t], h, s ? x[t].z : x[t].x, s ? x[t].w : x[t].y);
+      for (int i = 0; i < 4; ++i) {
+        const double2 v = a2[(4 * s + i) * 32];
+        a[2 * i] = v.x;
+        a[2 * i + 1] = v.y;
+      }
 #pragma unroll
-      for (int t = 0; t < NT; ++t) mma_f16_16816(T[t], l, s ? x[t].z : x[t].x, s ? x[t].w : x[t].y);
+      for (int t = 0; t < NT; ++t) {
+        double b[4];
+        halves_to_f64(s ? x[t].z : x[t].x, s ? x[t].w : x[t].y, b);
+        mma_f64_16816(T[t], a, b);
+      }
     }
     if (left > 1) load_x(token + gridDim.x);      // the next token's rows
-    // ---- T -> fp16 hi + lo, scaled so that the slice's largest entry lands in [2^13, 2^14) ----------------------
-    float tm = 0.0f;
-#pragma unroll
-    for (int t = 0; t < NT; ++t)
-      tm = fmaxf(tm, fmaxf(fmaxf(fabsf(T[t][0]), fabsf(T[t][1])), fmaxf(fabsf(T[t][2]), fabsf(T[t][3]))));
-    tm = warp_max(tm);
-    if constexpr (PW > 1) {
-      if (lane == 0) tmax[warp] = tm;
-      named_barrier(1 + m, PW * 32);
-#pragma unroll
-      for (int w = 0; w < PW; ++w) tm = fmaxf(tm, tmax[m * PW + w]);
-    }
-    int k = 13 - (static_cast<int>((__float_as_uint(tm) >> 23) & 0xFF) - 127);
-    if (tm == 0.0f) k = 0;
-    k = max(-126, min(127, k));
-    const float sc = __uint_as_float(static_cast<uint32_t>(k + 127) << 23);
-    const int uexp = -(k + 2 * kFactorScaleLog2) + 127;        // z = result * 2^-(k + 20), exactly
-    const float un = (uexp >= 1) ? __uint_as_float(static_cast<uint32_t>(min(uexp, 254)) << 23) : 0.0f;
-    uint32_t th[NT][2], tl[NT][2];
-#pragma unroll
-    for (int t = 0; t < NT; ++t)
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const float v0 = T[t][2 * r], v1 = T[t][2 * r + 1];
-        const __half2 hh = __floats2half2_rn(v0 * sc, v1 * sc);
-        const float2 hf = __half22float2(hh);
-        th[t][r] = *reinterpret_cast<const uint32_t*>(&hh);
-        tl[t][r] = pack_half2(fmaf(v0, sc, -hf.x), fmaf(v1, sc, -hf.y));
-      }
     if constexpr (PW > 1) {
 #pragma unroll
       for (int t = 0; t < NT; ++t) {
-        const int tg = part * NT + t;                  // k-step tg / 2, half tg % 2 of it
-        ts[((m * 2 + 0) * KJ * 2 + tg) * 32 + lane] = make_uint2(th[t][0], th[t][1]);
-        ts[((m * 2 + 1) * KJ * 2 + tg) * 32 + lane] = make_uint2(tl[t][0], tl[t][1]);
+        double2* o = ts + ((m * NTT + part * NT + t) * 2) * 32 + lane;
+        o[0] = make_double2(T[t][0], T[t][2]);
+        o[32] = make_double2(T[t][1], T[t][3]);
       }
       named_barrier(1 + m, PW * 32);
     }
     // ---- stage 2 ------------------------------------------------------------------------------------------
+    double zd[NT][4];
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) zd[t][e] = 0.0;
+    const float4* bj = b1s + part * NT * 32 + lane;
+#pragma unroll(KJ > 4 ? 1 : KJ)
+    for (int j = 0; j < KJ; ++j) {
+      double a[8];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {                    // tile 2 j + h: even rows p, odd rows p
+        if constexpr (PW > 1) {
+          const double2* o = ts + ((m * NTT + 2 * j + h) * 2) * 32 + lane;
+          const double2 v0 = o[0], v1 = o[32];
+          a[4 * h + 0] = v0.x; a[4 * h + 1] = v0.y; a[4 * h + 2] = v1.x; a[4 * h + 3] = v1.y;
+        } else {
+          a[4 * h + 0] = T[2 * j + h][0]; a[4 * h + 1] = T[2 * j + h][2];
+          a[4 * h + 2] = T[2 * j + h][1]; a[4 * h + 3] = T[2 * j + h][3];
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < NT; ++t) {
+        const float4 v = bj[(j * NTT + t) * 32];
+        const double b[4] = {v.x, v.y, v.z, v.w};
+        mma_f64_16816(zd[t], a, b);
+      }
+    }
     float z[NT][4];
 #pragma unroll
     for (int t = 0; t < NT; ++t)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) z[t][e] = 0.0f;
-    const uint4* bj = b1s + part * NT * 32 + lane;
-#pragma unroll(PW > 1 ? 1 : KJ)
-    for (int j = 0; j < KJ; ++j) {
-      uint32_t h[4], l[4];
-      if constexpr (PW > 1) {
-        const uint2 h01 = ts[((m * 2 + 0) * KJ * 2 + 2 * j) * 32 + lane], h23 = ts[((m * 2 + 0) * KJ * 2 + 2 * j + 1) * 32 + lane];
-        const uint2 l01 = ts[((m * 2 + 1) * KJ * 2 + 2 * j) * 32 + lane], l23 = ts[((m * 2 + 1) * KJ * 2 + 2 * j + 1) * 32 + lane];
-        h[0] = h01.x; h[1] = h01.y; h[2] = h23.x; h[3] = h23.y;
-        l[0] = l01.x; l[1] = l01.y; l[2] = l23.x; l[3] = l23.y;
-      } else {
-        h[0] = th[2 * j][0]; h[1] = th[2 * j][1]; h[2] = th[2 * j + 1][0]; h[3] = th[2 * j + 1][1];
-        l[0] = tl[2 * j][0]; l[1] = tl[2 * j][1]; l[2] = tl[2 * j + 1][0]; l[3] = tl[2 * j + 1][1];
-      }
-      uint4 b[NT];
-#pragma unroll
-      for (int t = 0; t < NT; ++t) b[t] = bj[(j * NTT + t) * 32];
-#pragma unroll
-      for (int t = 0; t < NT; ++t) mma_f16_16816(z[t], h, b[t].x, b[t].y);      // hi * hi
-#pragma unroll
-      for (int t = 0; t < NT; ++t) mma_f16_16816(z[t], l, b[t].x, b[t].y);      // lo * hi
-#pragma unroll
-      for (int t = 0; t < NT; ++t) mma_f16_16816(z[t], h, b[t].z, b[t].w);      // hi * lo
-    }
+      for (int e = 0; e < 4; ++e) z[t][e] = static_cast<float>(zd[t][e]);
     // z[t][e], z[t][2 + e]: channels q' = 16 m + 2 g, + 1 of row p' = 8 (part NT + t) + 2 c + e.
     if (f16out) {                                      // rotation only: fp16 rows out
       __half* zrow = reinterpret_cast<__half*>(Xq) + token * n + m * 16 + 2 * g;
@@ -230,7 +225,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int p = (part * NT + t) * 8 + 2 * c + e;
-          if (p < n1 && ok) *reinterpret_cast<uint32_t*>(zrow + p * N2) = pack_half2(z[t][e] * un, z[t][2 + e] * un);
+          if (p < n1 && ok) *reinterpret_cast<uint32_t*>(zrow + p * N2) = pack_half2(z[t][e], z[t][2 + e]);
         }
       if constexpr (PW > 1) __syncthreads();           // the T operand has been read
       continue;
@@ -239,7 +234,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
 #pragma unroll
     for (int t = 0; t < NT; ++t)
       zm = fmaxf(zm, fmaxf(fmaxf(fabsf(z[t][0]), fabsf(z[t][1])), fmaxf(fabsf(z[t][2]), fabsf(z[t][3]))));
-    zm = warp_max(zm * un);                            // padding rows hold exact zeros
+    zm = warp_max(zm);                                 // padding rows hold zeros, or NaN, which a maximum passes over
     float* zp = zmax + par * WARPS;                    // two sets in turn: one barrier per token is enough
     if (lane == 0) zp[warp] = zm;
     __syncthreads();
@@ -249,9 +244,9 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
     __half delta;
     float inv;
     row_scale(amax, delta, inv);
-    const float inv_un = inv * un;                     // exact: un is a power of two
-    // Delta >= 2^-14 (a normal fp16) bounds |z / Delta| by 7 (1 + 2^-11): no clamp is needed then.
-    const bool clamp = __half2float(delta) < 6.103515625e-05f;
+    // A finite Delta >= 2^-14 (a normal fp16) bounds |z / Delta| by 7 (1 + 2^-11): no clamp is needed then.  A token with an
+    // infinity has an infinite Delta, one with a NaN has 0; its codes are 0.
+    const bool clamp = !(__half2float(delta) >= 6.103515625e-05f && __half2float(delta) <= 65504.0f);
     uint8_t* orow = Xq + token * (n / 2) + m * 8;
 #pragma unroll
     for (int gr = 0; gr < (NT + 3) / 4; ++gr) {
@@ -264,8 +259,8 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
           const int t = 4 * gr + 2 * h + (i >> 1), e = i & 1;
 #pragma unroll
           for (int o = 0; o < 2; ++o) {
-            float v = t < NT ? __fadd_rn(__fmul_rn(z[t < NT ? t : 0][2 * o + e], inv_un), 0.5f) : 0.0f;
-            if (clamp) v = fminf(fmaxf(v, -8.0f), 7.5f);
+            float v = t < NT ? __fadd_rn(__fmul_rn(z[t < NT ? t : 0][2 * o + e], inv), 0.5f) : 0.0f;
+            if (clamp) v = v == v ? fminf(fmaxf(v, -8.0f), 7.5f) : 0.5f;
             tt[2 * i + o] = v;
           }
         }
@@ -282,7 +277,7 @@ rotate_quant_mma_kernel(const uint4* __restrict__ a2_img, const uint4* __restric
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int p = (part * NT + t) * 8 + 2 * c + e;
-          if (p < n1) *reinterpret_cast<float2*>(zrow + p * N2) = make_float2(z[t][e] * un, z[t][2 + e] * un);
+          if (p < n1) *reinterpret_cast<float2*>(zrow + p * N2) = make_float2(z[t][e], z[t][2 + e]);
         }
     }
     if (threadIdx.x == 0 && ok) scales[token] = delta;
@@ -297,12 +292,11 @@ sq_status_t launch_rm(const sq_rotation* h, const void* X, int64_t rows, void* X
   auto kern = rotate_quant_mma_kernel<NT, PW>;
   constexpr int smem = rm_smem(NT, PW);
   if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem)) return SQ_ERR_CUDA;
-  // Tokens in equal runs over the CTAs that are resident at once.
-  const long long cap = static_cast<long long>(sms) * std::min(PW == 2 ? 3 : (NT <= 4 ? 8 : 5), 220 * 1024 / (smem + 1024));
-  const long long per = (rows + cap - 1) / cap;
-  const uint4* b1 = static_cast<const uint4*>(h->dMmaImg);
-  const uint4* a2 = b1 + static_cast<size_t>(NT * PW / 2) * (NT * PW) * 32;
-  const cudaError_t err = launch_dependent(kern, dim3(static_cast<unsigned>((rows + per - 1) / per)), dim3(RM_SLICES * PW * 32),
+  const int resident = std::min(rm_ctas(NT, PW), 220 * 1024 / (smem + 1024));
+  const long long grid = std::min<long long>(rows, static_cast<long long>(sms) * resident);
+  const float4* b1 = static_cast<const float4*>(h->dMmaImg);
+  const double2* a2 = reinterpret_cast<const double2*>(b1 + static_cast<size_t>(NT * PW / 2) * (NT * PW) * 32);
+  const cudaError_t err = launch_dependent(kern, dim3(static_cast<unsigned>(grid)), dim3(RM_SLICES * PW * 32),
                                            static_cast<size_t>(smem), s, a2, b1, static_cast<int>(h->n1), static_cast<int>(rows),
                                            static_cast<const __half*>(X), static_cast<uint8_t*>(Xq),
                                            static_cast<__half*>(scales), Zdbg, f16out);
@@ -314,43 +308,30 @@ sq_status_t launch_rm(const sq_rotation* h, const void* X, int64_t rows, void* X
 
 bool rotate_quant_mma_supported(int n1, int n2) { return n1 >= 1 && n1 <= 128 && n2 == RM_N2; }
 
-// Uploads the two operand images in fragment order: R1 as [k-step][tile][lane] {b0 hi, b1 hi, b0 lo, b1 lo}, then R2^T as
-// [q' slice][k-step][hi, lo][lane] {a0 .. a3}.
+// Uploads the two operand images in fragment order: R1 in fp32 as [k-step][tile][lane] {b0 .. b3}, then R2^T in float64 as
+// [q' slice][k-slot of a lane][lane] {rows g, g + 8}.
 bool rotate_quant_mma_prepare(sq_rotation* h) {
   const int n1 = h->n1, n2 = h->n2;
   const RmShape sh = rm_shape(n1);
   const int ntt = sh.NT * sh.PW, kj = ntt / 2;
-  const size_t b1_words = static_cast<size_t>(kj) * ntt * 128, a2_words = static_cast<size_t>(n2 / 16) * (n2 / 16) * 256;
-  std::vector<uint32_t> img(b1_words + a2_words, 0u);
-  auto split_word = [](float v0, float v1, uint32_t& hi, uint32_t& lo) {
-    __half h0, l0, h1, l1;
-    split_half(v0, h0, l0);
-    split_half(v1, h1, l1);
-    hi = __half_as_ushort(h0) | static_cast<uint32_t>(__half_as_ushort(h1)) << 16;
-    lo = __half_as_ushort(l0) | static_cast<uint32_t>(__half_as_ushort(l1)) << 16;
-  };
-  auto r1 = [&](int p, int pp) { return p < n1 && pp < n1 ? kFactorScale * h->R1[static_cast<size_t>(p) * n1 + pp] : 0.0f; };
-  auto r2 = [&](int q, int qp) { return kFactorScale * h->R2[static_cast<size_t>(q) * n2 + qp]; };
+  const size_t b1_bytes = static_cast<size_t>(kj) * ntt * 512;
+  std::vector<unsigned char> img(b1_bytes + static_cast<size_t>(RM_SLICES) * RM_A2_SLICE, 0);
+  float* b1 = reinterpret_cast<float*>(img.data());
+  double* a2 = reinterpret_cast<double*>(img.data() + b1_bytes);
   for (int j = 0; j < kj; ++j)
     for (int t = 0; t < ntt; ++t)
-      for (int lane = 0; lane < 32; ++lane) {
-        const int g = lane >> 2, c = lane & 3;
-        uint32_t* w = img.data() + (static_cast<size_t>(j * ntt + t) * 32 + lane) * 4;
-        for (int r = 0; r < 2; ++r)
-          split_word(r1(16 * j + 8 * r + 2 * c, 8 * t + g), r1(16 * j + 8 * r + 2 * c + 1, 8 * t + g), w[r], w[2 + r]);
-      }
-  for (int m = 0; m < n2 / 16; ++m)
-    for (int s = 0; s < n2 / 16; ++s)
-      for (int lane = 0; lane < 32; ++lane) {
-        const int g = lane >> 2, c = lane & 3;
-        uint32_t* w = img.data() + b1_words + (static_cast<size_t>((m * (n2 / 16) + s) * 2) * 32 + lane) * 4;
-        for (int r = 0; r < 4; ++r) {
-          const int q = 32 * (s >> 1) + 8 * c + 4 * (s & 1) + 2 * (r >> 1), qp = 16 * m + 2 * g + (r & 1);
-          split_word(r2(q, qp), r2(q + 1, qp), w[r], w[128 + r]);
+      for (int lane = 0; lane < 32; ++lane)
+        for (int i = 0; i < 4; ++i) {
+          const int p = 16 * j + 8 * (i >> 1) + 2 * (lane & 3) + (i & 1), pp = 8 * t + (lane >> 2);
+          if (p < n1 && pp < n1) b1[(static_cast<size_t>(j * ntt + t) * 32 + lane) * 4 + i] = h->R1[static_cast<size_t>(p) * n1 + pp];
         }
-      }
-  if (cudaMalloc(&h->dMmaImg, img.size() * 4) != cudaSuccess ||
-      cudaMemcpy(h->dMmaImg, img.data(), img.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+  for (int m = 0; m < RM_SLICES; ++m)
+    for (int k = 0; k < 8; ++k)
+      for (int lane = 0; lane < 32; ++lane)
+        for (int r = 0; r < 2; ++r)
+          a2[((m * 8 + k) * 32 + lane) * 2 + r] = h->R2[static_cast<size_t>(8 * (lane & 3) + k) * n2 + 16 * m + 2 * (lane >> 2) + r];
+  if (cudaMalloc(&h->dMmaImg, img.size()) != cudaSuccess ||
+      cudaMemcpy(h->dMmaImg, img.data(), img.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -361,16 +342,16 @@ sq_status_t launch_rotate_quant_mma(const sq_rotation* h, const void* X, int64_t
                                     cudaStream_t s, bool f16out) {
   if (rows > 0x7FFFFFFF) return SQ_ERR_UNSUPPORTED;
   const RmShape sh = rm_shape(h->n1);
-  if (sh.PW == 1) {
-    if (sh.NT == 2) return launch_rm<2, 1>(h, X, rows, Xq, scales, Zdbg, f16out, s);
-    if (sh.NT == 4) return launch_rm<4, 1>(h, X, rows, Xq, scales, Zdbg, f16out, s);
-    if (sh.NT == 6) return launch_rm<6, 1>(h, X, rows, Xq, scales, Zdbg, f16out, s);
-    return launch_rm<8, 1>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+  if (sh.PW == 4) {
+    if (sh.NT == 2) return launch_rm<2, 4>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+    if (sh.NT == 3) return launch_rm<3, 4>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+    return launch_rm<4, 4>(h, X, rows, Xq, scales, Zdbg, f16out, s);
   }
+  if (sh.NT == 1) return launch_rm<1, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+  if (sh.NT == 2) return launch_rm<2, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+  if (sh.NT == 3) return launch_rm<3, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
   if (sh.NT == 5) return launch_rm<5, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
-  if (sh.NT == 6) return launch_rm<6, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
-  if (sh.NT == 7) return launch_rm<7, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
-  return launch_rm<8, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
+  return launch_rm<7, 2>(h, X, rows, Xq, scales, Zdbg, f16out, s);
 }
 
 }  // namespace sq

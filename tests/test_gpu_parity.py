@@ -158,6 +158,54 @@ def test_rotate_quant_warp_level(sq, n1, n2, M):
     check_rotate_quant(sq, X, R1, R2)
 
 
+# Its sums are float64, rounded once: every rotated value is within half an ulp (2^-24 of it) of the exact one, up to float64's
+# own rounding (1e-12 of the row's largest).  Any fp32 factor is taken, also far from a rotation's.
+@pytest.mark.parametrize("n1", [1, 16, 32, 48, 64, 80, 96, 112, 128])
+@pytest.mark.parametrize("scale", [1.0, 100.0, 1e-6])
+def test_warp_level_rotation_is_rounded_once(sq, n1, scale):
+    M = 300
+    X = wl.make_activations(wl.small(f"r64{n1}", M, n1, 32, 8, seed=n1))
+    R1, R2 = ora.build_rotation(X.astype(np.float32), n1, 32, seed=2)
+    R1, R2 = (R1 * scale).astype(np.float32), (R2 / scale).astype(np.float32)
+    rot = sq.sq_rotation_from_factors(R1, R2)
+    _, _, Z = run_rotate_quant(sq, rot, X)
+    want = np.einsum("pa,mpq,qb->mab", R1.astype(np.float64), X.astype(np.float64).reshape(M, n1, 32), R2.astype(np.float64),
+                     optimize=True).reshape(M, -1)
+    assert np.all(np.abs(Z - want) <= 2.0 ** -24 * np.abs(want) + 1e-12 * np.abs(want).max(axis=1, keepdims=True))
+    rot.close()
+
+
+@pytest.mark.parametrize("n1", [16, 64, 128, 130])
+def test_tokens_with_infinities_or_nan_stay_marked(sq, n1):
+    """n2 = 32, through the warp-level kernel and (n1 = 130) the fp32 kernel: a token with an infinity gets an infinite step and
+    codes 0, so that its outputs are NaN; one with a NaN gets step 0 and codes 0; its neighbours are what they are alone."""
+    K, M = n1 * 32, 9
+    rng = np.random.default_rng(n1)
+    X = rng.standard_normal((M, K)).astype(np.float16)
+    R1, R2 = ora.build_rotation(X.astype(np.float32), n1, 32, seed=2)
+    rot = sq.sq_rotation_from_factors(R1, R2)
+    clean = run_rotate_quant(sq, rot, X)
+    bad = X.copy()
+    bad[1, 77] = np.inf
+    bad[3, 5] = np.nan
+    bad[4, 40] = -np.inf
+    bad[7, 9], bad[7, 300] = np.inf, -np.inf
+    Xq, sx, Z = run_rotate_quant(sq, rot, bad)
+    ok = [0, 2, 5, 6, 8]
+    for got, want in zip((Xq, sx, Z), clean):
+        assert np.array_equal(got[ok], want[ok])
+    assert not np.any(Xq[[1, 3, 4, 7]]) and np.all(np.isposinf(sx[[1, 4, 7]])) and sx[3] == 0
+    assert not np.any(np.isfinite(Z[[1, 3, 4, 7]]))
+    z16 = Guarded(M * K * 2)
+    sq.sq_rotate_act_f16(rot, dev(bad), M, z16)
+    torch_mod().cuda.synchronize()
+    z16.check()
+    Z16 = z16.numpy(np.float16, (M, K))
+    assert np.all(np.isfinite(Z16[ok])) and not np.any(np.isfinite(Z16[[1, 3, 4, 7]]))
+    assert np.all(np.isnan(Z16[3])) and np.all(np.isinf(Z16[[1, 4]]))
+    rot.close()
+
+
 # Whole 32-byte sectors are stored at once where the buffers allow it; 16 bytes is what callers have to promise.
 @pytest.mark.parametrize("n1,n2,M", [(64, 64, 35), (48, 128, 33), (172, 64, 5), (136, 128, 3), (64, 64, 3)])
 def test_rotate_outputs_16_byte_aligned_only(sq, n1, n2, M):
