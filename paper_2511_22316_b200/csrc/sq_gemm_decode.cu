@@ -652,6 +652,23 @@ int choose_splits(int tiles, int blocks, int sms) {
   return best;
 }
 
+// Time of one launch in microseconds, back to back with others: fits to 62 shapes per token class (K 1024 to 28672, 128 to
+// 14336 channels), within a fifth.  `fixed`, then per wave of tiles the 256-channel blocks and the exchange of a split tile,
+// then the weights' megabytes.
+template <int NT>
+double decode_estimate_us(int N, int K) {
+  const int sms = sm_count();
+  if (sms <= 0 || !ensure_dyn_smem(reinterpret_cast<const void*>(w4a4_gemm_decode_kernel<NT>), DecSmem<NT>::DYN_BYTES)) return 1e30;
+  const int tiles = (N + 127) / 128, blocks = (K / 128 + 1) / 2;
+  const int splits = choose_splits<NT>(tiles, blocks, sms);
+  const int ncl = max_clusters<NT>(splits, sms);
+  if (ncl <= 0) return 1e30;
+  constexpr double fixed = NT == 64 ? 3.8 : (NT == 32 ? 2.7 : 2.2), block = NT == 64 ? 0.24 : (NT == 32 ? 0.18 : 0.16);
+  constexpr double split = NT == 64 ? 2.0 : (NT == 32 ? 1.4 : 1.1), mbyte = NT == 64 ? 0.083 : (NT == 32 ? 0.119 : 0.126);
+  const int waves = (tiles + ncl - 1) / ncl;
+  return fixed + waves * ((blocks + splits - 1) / splits * block + (splits > 1 ? split : 0.0)) + 0.5e-6 * N * K * mbyte;
+}
+
 template <int NT>
 sq_status_t launch_decode(const void* Xq, const void* sx, const void* Wq, const void* sw, int M, int N, int K, void* Y,
                           int32_t* accdbg, cudaStream_t s) {
@@ -724,6 +741,11 @@ sq_status_t launch_w4a4_gemm_decode_grouped(const void* Xq, const void* sx, int6
 
 bool gemm_decode_supported(int64_t M, int64_t N, int64_t K) {
   return M >= 1 && M <= 64 && N >= 128 && (K % 128 == 0) && K >= 256 && (N % 8 == 0);
+}
+
+double gemm_decode_estimate_us(int64_t M, int64_t N, int64_t K) {
+  const int n = static_cast<int>(N), k = static_cast<int>(K);
+  return M <= 16 ? decode_estimate_us<16>(n, k) : (M <= 32 ? decode_estimate_us<32>(n, k) : decode_estimate_us<64>(n, k));
 }
 
 sq_status_t launch_w4a4_gemm_decode(const void* Xq, const void* sx, const void* Wq, const void* sw, int M, int N, int K,

@@ -537,8 +537,18 @@ sq_status_t launch_w4a4_gemm_pair_grouped(const void* Xq, const void* sx, int64_
   return launch_pair_grouped<PairWide>(Xq, sx, M_total, count, Wq, sw, r0, rows, N, K, Y, s, sms);
 }
 
-// From 65 tokens on: with the narrow form even a tile that is three quarters empty beats two passes of the decode kernel
-// (100 x 4096 x 4096: 10.0 us against 16.1; 100 x 14336 x 4096, where that kernel splits K: 24.5 against 23.8).
+// Time of one launch in microseconds, back to back with others, for one token tile (at most 256 tokens): both forms' waves as
+// in pair_prefers_narrow, with the fixed cost that such a run of launches shows (28672 -> 512 43.1 us, 4096 -> 1024 9.5).
+double gemm_pair_estimate_us(int64_t M, int64_t N, int64_t K) {
+  const int pairs = sm_count() / 2;
+  if (pairs <= 0) return 1e30;
+  const long long wide = pair_tiles<PairWide>(M, N), narrow = pair_tiles<PairNarrow>(M, N);
+  const int num_sb = pair_blocks(K);
+  if (pair_prefers_narrow(wide, narrow, num_sb, pairs)) return static_cast<double>((narrow + pairs - 1) / pairs) * (0.345 * num_sb + 0.6) + 3.6;
+  return static_cast<double>((wide + pairs - 1) / pairs) * (0.57 * num_sb + 1.8) + 3.5;
+}
+
+// From 65 tokens on (launch_w4a4_gemm weighs it against two passes of the decode kernel up to 128).
 bool gemm_pair_supported(int64_t M, int64_t N, int64_t K) {
   return M > 64 && N >= 128 && (K % 128 == 0) && K >= 128 && (N % 8 == 0);
 }

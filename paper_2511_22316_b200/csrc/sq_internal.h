@@ -167,12 +167,14 @@ sq_status_t launch_w4a4_gemm(const void* Xq, const void* sx, const void* Wq, con
 
 // Step 3 on CTA pairs (sq_gemm_pair.cu): prefill-sized problems.
 bool gemm_pair_supported(int64_t M, int64_t N, int64_t K);
+double gemm_pair_estimate_us(int64_t M, int64_t N, int64_t K);
 sq_status_t launch_w4a4_gemm_pair(const void* Xq, const void* sx, const void* Wq, const void* sw, int M, int N,
                                   int K, void* Y, int32_t* accdbg, cudaStream_t s);
 
 // Step 3 for decode-sized problems (sq_gemm_decode.cu): weights as the A operand, K split over a
 // thread-block cluster with the partial tiles exchanged on chip (no scratch in global memory).
 bool gemm_decode_supported(int64_t M, int64_t N, int64_t K);
+double gemm_decode_estimate_us(int64_t M, int64_t N, int64_t K);
 // The CTA-pair kernel over the experts of a grouped layer in one launch (any number of rows per expert).
 int gemm_pair_max_groups();
 sq_status_t launch_w4a4_gemm_pair_grouped(const void* Xq, const void* sx, int64_t M_total, int count,

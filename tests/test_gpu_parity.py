@@ -464,7 +464,23 @@ PAIR_NARROW = [(65, 128, 1408), (129, 136, 1664), (70, 264, 4096), (200, 1000, 1
                (300, 9480, 2560), (130, 18952, 2304), (65, 128, 128), (129, 136, 1152), (333, 4096, 1024), (2048, 1280, 5120)]
 
 
-@pytest.mark.parametrize("M,N,K", GEMM_SHAPES + PAIR_NARROW)
+# 65 to 128 tokens: long K with few channels takes two passes (64 tokens, then 1, 2, 16, 32 or 64 more: dot products and every
+# class of the decode kernel, with K split over clusters), the others one.
+TWO_PASSES = [(65, 128, 14336), (66, 136, 11008), (80, 512, 8192), (96, 1024, 14336), (128, 264, 28672), (100, 2304, 14336)]
+ONE_PASS = [(65, 4096, 1024), (128, 4096, 4096), (100, 14336, 1024), (129, 128, 14336)]
+
+
+@pytest.mark.parametrize("M,N,K,passes", [s + (2,) for s in TWO_PASSES] + [s + (1,) for s in ONE_PASS])
+def test_gemm_65_to_128_tokens_takes_the_cheaper_route(sq, M, N, K, passes):
+    torch = torch_mod()
+    X, W = (torch.zeros(r, K // 2, dtype=torch.uint8, device="cuda") for r in (M, N))
+    sx, sw, Y = (torch.zeros(n, dtype=torch.float16, device="cuda") for n in (M, N, M * N))
+    before = sq.sq_kernel_launch_count()
+    sq.sq_w4a4_gemm(X, sx, W, sw, M, N, K, Y)
+    assert sq.sq_kernel_launch_count() - before == passes
+
+
+@pytest.mark.parametrize("M,N,K", GEMM_SHAPES + PAIR_NARROW + TWO_PASSES + ONE_PASS)
 def test_gemm_accumulators_bit_exact(sq, M, N, K):
     rng = np.random.default_rng(M * 1000003 + N * 101 + K)
     Xc, Wc = random_codes(rng, M, K), random_codes(rng, N, K)
