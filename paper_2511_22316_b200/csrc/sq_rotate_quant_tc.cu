@@ -641,11 +641,14 @@ sq_status_t launch_rotate_quant_tc(const sq_rotation* h, const void* X, int64_t 
   const RqLayout Lh = rq_layout(n1, n2, kHalfDynSmem);
   const bool dual = (n2 == 64) && Lh.XS >= 2;
   // A handful of tokens: latency is all there is.  One token per accumulator (a group's stage 1 is half or a quarter as
-  // long) and eight warps on it also with n2 = 64; the sums are the same, in the same order.  Not beyond 32 tokens: every
-  // CTA here keeps one of the product's off its SM.  16 x 4096 (64 x 64): 4.57 -> 3.86 us, layer to 14336 11.5 -> 10.7.
-  // The quantising form asks for an SM of its own (120 KB: the layer for one token 11.1 us without, 9.9 with), the fp16
-  // form does not (18.4 without, 25 with: the dot-product kernel behind it then doubles up on another SM).
-  const bool few = rows <= 32;
+  // long) and eight warps on it also with n2 = 64; the sums are the same, in the same order.  16 x 4096 (64 x 64): 4.57 ->
+  // 3.86 us, layer to 14336 11.5 -> 10.7.
+  // The quantising form asks for an SM of its own (120 KB: the layer for one token 11.1 us without, 9.9 with) and keeps the
+  // product's CTA off it.  Hence no more than 16 tokens: many layers have 128 such CTAs in clusters, and beyond 20 tokens the
+  // last of them wait for the rotation to end (32 x 4096 -> 4096 10.2 us, 9.1 in the other form; 32 x 8192 -> 4096 12.9 and
+  // 11.8; against that 24 x 8192 -> 1024 9.9 and 10.2).  The fp16 form shares its SM (18.4 us, alone on it 25: the
+  // dot-product kernel behind it then doubles up on another SM) and goes up to 32.
+  const bool few = rows <= (f16out ? 32 : 16);
   const RqLayout L = few ? rq_layout(n1, n2, kMaxDynSmem, true) : (dual ? Lh : rq_layout(n1, n2));
   EncodeTiledFn enc = get_encode_fn();
   if (!enc) return SQ_ERR_CUDA;
