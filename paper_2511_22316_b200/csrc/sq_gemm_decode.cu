@@ -211,11 +211,16 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
     return true;
   };
 
+  // Two of the eight stages are requested when the first has landed: with all of them in flight at once the loads of the
+  // rotate kernel, which this kernel overtakes, come late.  Layers: 4 x 8192 -> 4096 10.1 -> 9.6 us, 16 x 8192 -> 8192 13.4 ->
+  // 12.6, 16 x 4096 -> 32000 16.4 -> 16.0.  (Rings of six gain the same there and lose where much is streamed, 4 x 28672 ->
+  // 8192 26.1 -> 27.0; so did waiting for the rotate kernel itself.)
+  const bool hold_back = NT < 64 && tokens_ready == nullptr;
   if (threadIdx.x == 0) {
-    // First of all the weights of the whole staging ring: nothing else is on the critical path.
+    // First of all the weights of the staging ring: nothing else is on the critical path.
     for (int s = 0; s < S_W; ++s) mbar_init(&w_full[s], 1);
     mbar_fence_init();
-    produce_w(S_W);
+    produce_w(hold_back ? S_W - 2 : S_W);
     tma_prefetch_desc(&tmap_x);
     for (int s = 0; s < S_W; ++s) mbar_init(&w_empty[s], 4);     // one converter group
     for (int s = 0; s < S_X; ++s) {
@@ -254,7 +259,7 @@ __device__ __forceinline__ void w4a4_gemm_decode_body(const CUtensorMap& tmap_w,
 
   if (warp == 0) {
     // ------------------------------ weight loads ------------------------------------------------
-    if (lane == 0) produce_w(0xFFFFFFFFu);
+    if (lane == 0 && (!hold_back || cid >= tiles || mbar_wait(&w_full[0], 0, DSITE_W_FULL, limit))) produce_w(0xFFFFFFFFu);
   } else if (warp == D_X_WARP) {
     // ------------------------------ token loads -------------------------------------------------
     // The tokens come from the kernel before this one; in the fused form this one thread polls the counter of the CTAs
