@@ -224,23 +224,58 @@ def test_rotate_outputs_16_byte_aligned_only(sq, n1, n2, M):
 
 
 # The decision itself, on enough codes to meet its ties: code = floor(fl(fl(z * inv) + 0.5)) of the z that the kernel
-# reports, no code excepted.  (A product and sum rounded together differ in one of some 5e7.)
-@pytest.mark.parametrize("n1,n2,M", [(64, 64, 32768), (172, 64, 8192), (112, 128, 8192), (64, 64, 32)])
-def test_quantiser_rounds_product_and_sum_on_their_own(sq, n1, n2, M):
+# reports, no code excepted.  (A product and sum rounded together differ in one of some 5e7.)  What the compiler makes of the
+# two is decided for every instantiation, so each is here: the dense kernels with one and two warps per lane quarter, one, two
+# and four slots, CTA pairs, up to 16 tokens a call (`chunk`), R2 through its structure, n2 = 32.
+ROUNDING = [(64, 64, 32768, 0, False), (172, 64, 8192, 0, False), (112, 128, 8192, 0, False), (64, 64, 32, 0, False),
+            (128, 64, 16384, 0, False), (224, 128, 4096, 0, False), (64, 64, 16384, 16, False), (112, 128, 4096, 16, False),
+            (64, 64, 32768, 0, True), (64, 128, 16384, 0, True), (16, 32, 131072, 0, False), (64, 32, 65536, 0, False),
+            (128, 32, 32768, 0, False)]
+
+
+@pytest.mark.parametrize("n1,n2,M,chunk,structured", ROUNDING)
+def test_quantiser_rounds_product_and_sum_on_their_own(sq, n1, n2, M, chunk, structured):
     torch, K = torch_mod(), n1 * n2
     rng = np.random.default_rng(n1 + M)
     X0 = rng.standard_normal((8, K)).astype(np.float32)
-    rot = sq.sq_build_rotation(X0, n1, n2, seed=3)
+    rot = sq.sq_build_rotation(X0, n1, n2, seed=3, flags=ora.ROT_DEFAULT | (sq.SQ_ROT_APPLY_STRUCTURED if structured else 0))
+    assert rot.structured == structured
     X = torch.randn(M, K, device="cuda", generator=torch.Generator(device="cuda").manual_seed(M)).mul_(0.02).half()
     Xq = torch.empty(M, K // 2, dtype=torch.uint8, device="cuda")
     sx, z = torch.empty(M, dtype=torch.float16, device="cuda"), torch.empty(M, K, dtype=torch.float32, device="cuda")
-    sq.sq_rotate_quant_act(rot, X, M, Xq, sx, z)
+    step = chunk or M
+    for r in range(0, M, step):
+        sx_r = torch.empty(step, dtype=torch.float16, device="cuda")        # a slice of sx need not be 16-byte aligned
+        sq.sq_rotate_quant_act(rot, X[r:r + step], step, Xq[r:r + step], sx_r, z[r:r + step])
+        sx[r:r + step] = sx_r
     z.mul_((1.0 / sx.float()).unsqueeze(1))
     z.add_(0.5)
     z.floor_().clamp_(-8, 7)
     want = z.view(M, K // 2, 2).to(torch.int8)
     got_lo, got_hi = (Xq & 15).to(torch.int8), (Xq >> 4).to(torch.int8)
     assert bool(torch.all(got_lo == (want[..., 0] & 15))) and bool(torch.all(got_hi == (want[..., 1] & 15)))
+
+
+@pytest.mark.parametrize("n1,n2,m", [(64, 64, 16), (64, 64, 64), (64, 128, 32)])
+def test_one_launch_layer_takes_the_same_codes(sq, n1, n2, m):
+    """The rotating blocks of the one-launch layer are compiled into its kernels: their codes and steps, read out of the
+    workspace, are those of the kernel by itself, over 1e8 codes."""
+    torch, K, N = torch_mod(), n1 * n2, 256
+    calls = 100_000_000 // (m * K)
+    X0 = np.random.default_rng(5).standard_normal((8, K)).astype(np.float32)
+    rots = [sq.sq_build_rotation(X0, n1, n2, seed=3, flags=ora.ROT_DEFAULT | f) for f in (0, sq.SQ_ROT_FUSE_DECODE)]
+    X = torch.randn(calls * m, K, device="cuda", generator=torch.Generator(device="cuda").manual_seed(m)).mul_(0.02).half()
+    Wq, sw = torch.zeros(N, K // 2, dtype=torch.uint8, device="cuda"), torch.zeros(N, dtype=torch.float16, device="cuda")
+    nb = sq.sq_linear_workspace_bytes(m, K)
+    ws, Y = torch.zeros(2, nb, dtype=torch.uint8, device="cuda"), torch.empty(m, N, dtype=torch.float16, device="cuda")
+    same = torch.ones((), dtype=torch.bool, device="cuda")
+    before = sq.sq_kernel_launch_count()
+    for r in range(0, calls * m, m):
+        for rot, w in zip(rots, ws):
+            sq.sq_linear(rot, X[r:r + m], m, Wq, sw, N, K, w, nb, Y)
+        same &= torch.all(ws[0] == ws[1])
+    assert bool(same) and sq.sq_last_device_status() == sq.SQ_OK
+    assert sq.sq_kernel_launch_count() - before == 3 * calls                 # two launches and one
 
 
 def test_rotate_quant_tiny_config(sq):

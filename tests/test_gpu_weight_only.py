@@ -43,7 +43,8 @@ def _sync_ok(sq):
 
 # ------------------------------------------------------------------ offline weight path
 @pytest.mark.parametrize("bits", [4, 3])
-@pytest.mark.parametrize("n1,n2,N", [(16, 32, 40), (64, 64, 130), (172, 64, 24), (112, 128, 17), (12, 8, 9), (7, 8, 5)])
+@pytest.mark.parametrize("n1,n2,N", [(16, 32, 40), (64, 64, 130), (172, 64, 24), (112, 128, 17), (12, 8, 9), (7, 8, 5),
+                                     (128, 32, 40), (64, 32, 700)])
 def test_pack_weight_wo_matches_oracle(sq, bits, n1, n2, N):
     w = wl.small(f"wo{n1}x{n2}", 16, n1, n2, N, seed=n1 + 3 * n2 + bits)
     X, W = wl.make_layer(w)
@@ -136,7 +137,9 @@ def test_weight_only_argument_checks(sq):
 
 # ------------------------------------------------------------------ step 1 alone, fp16 rows
 ROT_SHAPES = [(16, 32, 64), (64, 64, 37), (64, 64, 301), (8, 64, 9), (100, 128, 3), (112, 128, 4), (64, 128, 70),
-              (129, 64, 3), (172, 64, 9), (224, 128, 5), (144, 128, 150), (12, 8, 5), (7, 6, 3)]
+              (129, 64, 3), (172, 64, 9), (224, 128, 5), (144, 128, 150), (12, 8, 5), (7, 6, 3),
+              # warp-level kernel, several warps per slice and several tokens per block
+              (65, 32, 5), (100, 32, 700), (128, 32, 700), (48, 32, 1300), (16, 32, 2500)]
 
 
 @pytest.mark.parametrize("n1,n2,M", ROT_SHAPES)
