@@ -867,15 +867,39 @@ def run_ours(args, w):
             line["sustained"] = sustained
         if cpu is not None:
             line["cpu_baseline"] = cpu
-        if per_workload is not None:
-            line["per_workload"] = per_workload
-        if variants is not None:
-            line["variants"] = variants
-        print(json.dumps(line))
+        tables = {k: v for k, v in (("per_workload", per_workload), ("variants", variants)) if v is not None}
+        print_line(line, tables)
     if dist is not None:
         dist.barrier()
         dist.destroy_process_group()
     return 0
+
+
+def rounded(v):
+    """Floats to six significant digits, in nested lists and dicts."""
+    if isinstance(v, dict):
+        return {k: rounded(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [rounded(x) for x in v]
+    return float(f"{v:.6g}") if isinstance(v, float) else v
+
+
+LINE_LIMIT = 2400       # bytes of the result line: whoever keeps only the end of the output still has all of it
+
+
+def print_line(line, tables):
+    """The result as one line on stdout, the tables of the other workloads on stderr.  Explanations leave the line, longest
+    first, where it would be longer than LINE_LIMIT; the whole of it is then on stderr too."""
+    line, full = rounded(line), rounded(line)
+    texts = sorted(((len(x), k, t) for k, d in line.items() if isinstance(d, dict) and k != "config"
+                    for t, x in d.items() if isinstance(x, str) and len(x) > 24), reverse=True)
+    for _, k, t in texts:
+        if len(json.dumps(line)) <= LINE_LIMIT:
+            break
+        del line[k][t]
+    if tables or line != full:
+        print(json.dumps(dict(full if line != full else {}, **rounded(tables))), file=sys.stderr)
+    print(json.dumps(line))
 
 
 def main():
