@@ -67,8 +67,8 @@ struct DecSmem {
   // Stages of 256 channels: packed weights, packed tokens, int8 operands (weights in TMEM, tokens in shared memory).
   // Weights and tokens have rings of their own: the weights come in, and are converted as far as the operand ring goes,
   // before the tokens exist.  Deeper is not better: the weights that stream in meanwhile hold up the rotate kernel's own
-  // loads.  Layer 16 x 4096 -> 14336 with 5 / 6 / 8 / 10 stages: 10.9 / 10.7 / 10.7 / 11.2 us (12.2 with one ring of six
-  // for both); 16 x 8192 -> 28672: 29.3 / 28.4 / 27.3 / 27.7 (31.0).
+  // loads.  Layer 16 x 4096 -> 14336 with 5 / 6 / 8 / 10 stages, all requested at once: 10.9 / 10.7 / 10.7 / 11.2 us (12.2
+  // with one ring of six for both); 16 x 8192 -> 28672: 29.3 / 28.4 / 27.3 / 27.7 (31.0).
   static constexpr int S_W = NT == 64 ? 5 : 8;
   static constexpr int S_X = NT == 64 ? 5 : 8;
   static constexpr int S_OP = 4;
