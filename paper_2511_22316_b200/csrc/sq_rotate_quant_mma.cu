@@ -5,14 +5,14 @@
 //
 //   stage 1  T^T[q'][p]  = sum_q R2^T[q'][q] X^T[q][p]    A = R2^T (shared memory), B = X^T: the token's rows as they lie
 //                                                         in memory, 16 bytes per lane
-//   stage 2  Z^T[q'][p'] = sum_p T^T[q'][p] R1[p][p']     A = T^T: the accumulators of stage 1 are in the layout of
-//                                                         this operand, B = R1 (shared memory, as fp32)
+//   stage 2  Z^T[q'][p'] = sum_p T^T[q'][p] R1[p][p']     A = T^T: the accumulators of stage 1 as they are (through
+//                                                         shared memory), B = R1 (shared memory, as fp32)
 // Both are mma.sync m16n8k16 in float64, rounded once to fp32 at the end.  The unit runs at half the fp32 rate, which these
 // sizes do not feel, and it takes any fp32 factor and passes infinities and NaN on as the fp32 kernel does.  Operands split
 // into two fp16 numbers (the tcgen05 kernels' way) were faster on many rows, 2048 x 4096 in 26 us, but two to three times as
 // far from float64 as the fp32 kernel, NaN for factors beyond 64, and finite codes for tokens with infinities.
-// For n1 > 64 the p axis is cut over two warps: each makes its part of T and of Z, and the operand of stage 2 goes through
-// shared memory once.  A CTA (two or four warps) owns a token at a time; its warps meet for the absmax.
+// The p axis is cut over two or four warps: each makes its part of T and of Z, and the operand of stage 2 goes through
+// shared memory once.  A CTA (four or eight warps) owns a token at a time; its warps meet for the absmax.
 //
 // Operand order.  k-slots may stand for any channel as long as A and B agree: lane (g, c) loads q = 8 c .. 8 c + 7 of row
 // p = 8 t + g, and the eight halves are the b registers of both k-steps; the image of R2^T is stored in that order.  Rows
@@ -89,11 +89,11 @@ constexpr int rm_ctas(int NT, int PW) { return PW == 4 ? (NT == 4 ? 2 : 3) : (NT
 
 constexpr int RM_N2 = 32, RM_SLICES = RM_N2 / 16;      // q' slices of a token, PW warps each
 
-// Shared memory: [R1 operand, fp32][R2^T operand][T operand, PW > 1: slice x tile x half x lane x 16 B][maxima, barrier].
+// Shared memory: [R1 operand, fp32][R2^T operand][T operand: slice x tile x half x lane x 16 B][maxima, barrier].
 constexpr int RM_A2_SLICE = RM_N2 * 32 / 4 * 16;
 constexpr int rm_smem(int NT, int PW) {
   const int ntt = NT * PW;
-  return ntt / 2 * ntt * 512 + RM_SLICES * RM_A2_SLICE + (PW > 1 ? RM_SLICES * ntt * 1024 : 0) + 128;
+  return ntt / 2 * ntt * 512 + RM_SLICES * RM_A2_SLICE + RM_SLICES * ntt * 1024 + 128;
 }
 
 // Tokens cta, cta + ncta, ... of `rows`: how many there are.  Unsigned, since rows goes up to 2^31 - 1 and the token behind
@@ -111,7 +111,7 @@ rotate_quant_mma_kernel(const double2* __restrict__ a2_img, const float4* __rest
   constexpr int NTT = NT * PW, KJ = NTT / 2;           // p tiles, k-steps of stage 2
   static_assert(NTT % 2 == 0, "whole k-steps");
   constexpr int B1_BYTES = KJ * NTT * 512, A2_BYTES = RM_SLICES * RM_A2_SLICE;
-  constexpr int T_BYTES = PW > 1 ? RM_SLICES * NTT * 1024 : 0;
+  constexpr int T_BYTES = RM_SLICES * NTT * 1024;
   extern __shared__ __align__(128) unsigned char rm_smem_raw[];
   const float4* b1s = reinterpret_cast<const float4*>(rm_smem_raw);
   unsigned char* a2s = rm_smem_raw + B1_BYTES;
@@ -175,15 +175,13 @@ rotate_quant_mma_kernel(const double2* __restrict__ a2_img, const float4* __rest
       }
     }
     if (left > 1) load_x(token + gridDim.x);      // the next token's rows
-    if constexpr (PW > 1) {
 #pragma unroll
-      for (int t = 0; t < NT; ++t) {
-        double2* o = ts + ((m * NTT + part * NT + t) * 2) * 32 + lane;
-        o[0] = make_double2(T[t][0], T[t][2]);
-        o[32] = make_double2(T[t][1], T[t][3]);
-      }
-      named_barrier(1 + m, PW * 32);
+    for (int t = 0; t < NT; ++t) {
+      double2* o = ts + ((m * NTT + part * NT + t) * 2) * 32 + lane;
+      o[0] = make_double2(T[t][0], T[t][2]);
+      o[32] = make_double2(T[t][1], T[t][3]);
     }
+    named_barrier(1 + m, PW * 32);
     // ---- stage 2 ------------------------------------------------------------------------------------------
     double zd[NT][4];
 #pragma unroll
@@ -196,14 +194,9 @@ rotate_quant_mma_kernel(const double2* __restrict__ a2_img, const float4* __rest
       double a[8];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {                    // tile 2 j + h: even rows p, odd rows p
-        if constexpr (PW > 1) {
-          const double2* o = ts + ((m * NTT + 2 * j + h) * 2) * 32 + lane;
-          const double2 v0 = o[0], v1 = o[32];
-          a[4 * h + 0] = v0.x; a[4 * h + 1] = v0.y; a[4 * h + 2] = v1.x; a[4 * h + 3] = v1.y;
-        } else {
-          a[4 * h + 0] = T[2 * j + h][0]; a[4 * h + 1] = T[2 * j + h][2];
-          a[4 * h + 2] = T[2 * j + h][1]; a[4 * h + 3] = T[2 * j + h][3];
-        }
+        const double2* o = ts + ((m * NTT + 2 * j + h) * 2) * 32 + lane;
+        const double2 v0 = o[0], v1 = o[32];
+        a[4 * h + 0] = v0.x; a[4 * h + 1] = v0.y; a[4 * h + 2] = v1.x; a[4 * h + 3] = v1.y;
       }
 #pragma unroll
       for (int t = 0; t < NT; ++t) {
@@ -227,7 +220,7 @@ rotate_quant_mma_kernel(const double2* __restrict__ a2_img, const float4* __rest
           const int p = (part * NT + t) * 8 + 2 * c + e;
           if (p < n1 && ok) *reinterpret_cast<uint32_t*>(zrow + p * N2) = pack_half2(z[t][e], z[t][2 + e]);
         }
-      if constexpr (PW > 1) __syncthreads();           // the T operand has been read
+      __syncthreads();                                 // the T operand has been read
       continue;
     }
     float zm = 0.0f;
