@@ -320,6 +320,12 @@ __device__ __forceinline__ void store_codes(uint32_t d2, uint32_t (&r)[32], __ha
   }
 }
 
+// Shared memory that a launch asks for.  Forms that want an SM of their own ask for more than half of it.  No form asks for so
+// little that a CTA-pair rotation (142 KB and more) fits beside it: dependents may start before a CTA has allocated its tensor
+// memory, one that took all 512 columns first would leave it waiting, and then wait for it.
+constexpr int kAloneSmem = 120 * 1024, kLeastSmem = 88 * 1024;
+inline int rq_smem(const RqLayout& L, int ctas_per_sm) { return std::max(L.total + 1024, ctas_per_sm == 1 ? kAloneSmem : kLeastSmem); }
+
 // The kernel's body, for CTA `cta` of `ncta` that share the token groups (the fused decode kernel of
 // sq_linear_fused.cu runs it in its first CTAs, with more warps in the block than the roles below use).
 template <int N2, int S, int CW = 1, bool F16OUT = false>
@@ -385,6 +391,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
     griddep_wait();
     // Only now may a GEMM launched behind this kernel start: it requests its weights before it waits for
     // this kernel, and whatever precedes this kernel (sq_pack_weight, say) may have been writing them.
+    // (Not later either: behind the tensor memory's allocation, 4 x 11008 -> 4096 took 11.3 us instead of 10.8.)
     griddep_launch_dependents();
     for (int i = 0; i < preload; ++i) load_group(i, i);
     for (int b = 0; b < 4; ++b) {
@@ -671,8 +678,7 @@ sq_status_t launch_rotate_quant_tc(const sq_rotation* h, const void* X, int64_t 
   const unsigned char* a1 = static_cast<const unsigned char*>(h->dA1img);
   const unsigned char* b2 = static_cast<const unsigned char*>(h->dB2img);
   auto launch = [&](auto kern, int slots, int ctas_per_sm, int cw = 1) -> bool {
-    // A CTA that wants all of TMEM asks for more than half of the shared memory, so that it is alone.
-    const int smem = ctas_per_sm == 1 ? std::max(L.total + 1024, 120 * 1024) : L.total + 1024;
+    const int smem = rq_smem(L, ctas_per_sm);
     if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem)) return false;
     const unsigned grid = static_cast<unsigned>(std::min<long long>(ngroups, static_cast<long long>(sms) * ctas_per_sm));
     return launch_dependent(kern, dim3(grid), dim3((2 + 4 * slots * cw) * 32), static_cast<size_t>(smem), s, mx, L, a1, b2, n1,
