@@ -90,6 +90,8 @@ def gemm_kernel_name(w):
     """The kernel sq_w4a4_gemm picks for this shape (mirrors the library's dispatch)."""
     fast = w.K % 128 == 0 and w.N % 8 == 0
     decode = fast and w.M <= 64 and w.N >= 128 and w.K >= 256
+    if w.M <= 8 and w.N >= 128 and w.N % 2 == 0 and w.K % 32 == 0 and w.K >= 256 and (w.M > 1 or not 8e6 <= w.N * w.K / 2 <= 16e6):
+        return "w4a4_gemm_stream_kernel"
     if w.M <= 4 and w.K % 32 == 0 and w.K <= 32768 and (w.M <= 2 or not decode):
         return "w4a4_gemv_kernel"
     if decode:
@@ -549,7 +551,7 @@ def weight_only_entry(sq, torch, w, bits, pk, l2, quick=False):
     rot_bytes = 4.0 * M * K
     if M <= 64:
         gbs = gemm_bytes_wo / (gemm_ms * 1e-3) / 1e9
-        roof = {"kernel": "wo_gemv_kernel" if M <= 2 else "wo_gemm_tmem_kernel", "bound": "hbm", "achieved": gbs, "peak": pk["hbm_gbs"], "unit": "GB/s",
+        roof = {"kernel": "wo_gemm_stream_kernel" if M <= 8 else "wo_gemm_tmem_kernel", "bound": "hbm", "achieved": gbs, "peak": pk["hbm_gbs"], "unit": "GB/s",
                 "frac": gbs / pk["hbm_gbs"], "traffic": NCU_TRAFFIC.get(("wo_gemm", w.name)) if bits == 4 else None,
                 "ms_per_launch": gemm_ms,
                 "algorithmic_bytes": gemm_bytes_wo}

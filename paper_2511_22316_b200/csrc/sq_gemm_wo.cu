@@ -1255,6 +1255,7 @@ sq_status_t launch_wo_gemm(const void* Z16, const void* Wq, const void* sw, int6
                            cudaStream_t s) {
   if (M == 0 || N == 0) return SQ_OK;
   const bool tc_ok = (K % 64 == 0) && (N % 8 == 0);
+  if (wo_stream_supported(M, N, K)) return launch_wo_gemm_stream(Z16, Wq, sw, (int)M, (int)N, (int)K, Y, s);
   if (M <= 2 && K % 32 == 0 && static_cast<int64_t>(M) * K * 4 <= 200 * 1024) {
     // one or two tokens: dot products on the CUDA cores
     if (M == 1) return launch_wo_gemv<1>(Z16, Wq, sw, (int)M, (int)N, (int)K, Y, s);

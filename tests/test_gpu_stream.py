@@ -1,0 +1,113 @@
+"""The products for up to 8 tokens as a stream of weights (sq_gemm_stream.cu): layouts on the CPU, edges of tiles and rings on the GPU."""
+import numpy as np
+import pytest
+
+import csrc_util
+from gpu_util import Guarded, dev, torch_mod
+from oracle import singlequant_oracle as ora
+
+
+def test_layouts_fit_and_their_rings_can_be_followed():
+    """Every warp meets every phase of its stages (the depth is a multiple of the stages worked on side by side), no more
+    stages are in flight than there are, and ring, sums and barriers lie apart inside the shared memory of a block."""
+    src = csrc_util.source("sq_gemm_stream.cu")
+    rows = csrc_util.run(
+        csrc_util.lines(src, r"^constexpr int SM_.*$") + "\n" + csrc_util.block(src, "struct StreamLayout")
+        + csrc_util.block(src, "__host__ __device__ inline StreamLayout stream_layout(") + """
+void show(int kind, StreamLayout L, int red) {
+  printf("%d %d %d %d %d %d %d %d %d %d %d %d\\n", kind, L.rows, L.wr, L.nb, L.stages, L.flight, L.w_st, L.x_st, L.off_x,
+         L.off_red, L.off_bar, L.total - 3 * SM_MAX_STAGES * 8);
+}
+int main() {
+  for (int r = 8; r <= SM_MAX_ROWS; r += 2) {
+    show(0, stream_layout(r, SM_NT * 128, SM_NT * SM_RP8 * 4, false), 0);
+    for (int o = 0; o < 2; ++o) show(1 + o, stream_layout(r, SM_NT * 512, 8 / (r > 32 ? 2 : 1) * SM_PART * 4, o), 0);
+  }
+}""")
+    assert len(rows) == 61 * 3
+    for kind, r, wr, nb, stages, flight, w_st, x_st, off_x, off_red, off_bar, end in (map(int, x) for x in rows):
+        lap = 16 // wr // 2
+        assert stages >= lap and stages % lap == 0 and stages <= 32 and 2 <= flight <= stages, r
+        assert nb <= 4 and nb * wr * 16 >= r and off_x == stages * w_st and w_st >= 128 * r
+        ring = off_x + stages * x_st
+        sums = 8 * 136 * 4 if kind == 0 else (4 if wr == 2 else 8) * 8 * 132 * 4
+        assert (off_red == 0 and kind == 2) or off_red >= ring
+        assert off_bar >= max(ring, off_red + sums) and off_bar % 8 == 0 and end == off_bar
+        assert end + 768 + 1024 <= 227 * 1024
+        assert (nb * wr * 16 - r) * 128 <= stages * x_st        # a ragged last block is read past its stage, never past the ring
+
+
+def _rows(rows, M):
+    """Channels that make a tile of `rows` on 148 SMs."""
+    return (148 - M) * rows
+
+
+# One and several stages, a ragged last one; the tile heights at which warps are split and blocks are added; several tiles per
+# block; ragged last tiles; one token and a full tile of eight.
+SHAPES = [(1, 128, 256), (8, 130, 288), (3, 200, 544), (8, 2048, 14336), (5, 4106, 1312)] + [
+    (8, _rows(r, 8), 800) for r in (16, 18, 32, 34, 48, 50, 64, 66, 96, 98, 128)] + [(8, _rows(128, 8) + 6, 576), (2, 40002, 288)]
+
+
+def _codes(rng, n, K):
+    return rng.integers(-8, 8, size=(n, K), dtype=np.int8)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K", SHAPES)
+def test_w4a4_stream_is_bit_exact(M, N, K):
+    from paper_2511_22316_b200 import binding as sq
+    rng = np.random.default_rng(M * 131 + N + K)
+    Xc, Wc = _codes(rng, M, K), _codes(rng, N, K)
+    Xc[0], Wc[0] = -8, -8
+    sx, sw = rng.uniform(0.01, 2.0, size=M).astype(np.float16), rng.uniform(0.001, 0.1, size=N).astype(np.float16)
+    y, acc = Guarded(M * N * 2), Guarded(M * N * 4)
+    sq.sq_w4a4_gemm(dev(ora.pack_int4(Xc)), dev(sx), dev(ora.pack_int4(Wc)), dev(sw), M, N, K, y, acc)
+    torch_mod().cuda.synchronize()
+    assert sq.sq_last_device_status() == sq.SQ_OK
+    y.check(), acc.check()
+    want = Xc.astype(np.float64) @ Wc.astype(np.float64).T                   # integers below 2^53
+    assert np.array_equal(acc.numpy(np.int32, (M, N)), want.astype(np.int32))
+    apart = y.numpy(np.float16, (M, N)).view(np.int16).astype(int) - ora.dequant(want.astype(np.int32), sx, sw).view(np.int16)
+    assert np.abs(apart).max() <= 1                                          # the steps' product is rounded to fp32
+
+
+# The same, and K over clusters of 2, 4 and 8 (few channels, long K).
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K", [s for s in SHAPES if s[0] > 1] + [(1, 5128, 4096), (8, 136, 8192), (8, 1024, 8192), (7, 4098, 14336),
+                                                                  (8, 8192, 28672)])
+def test_weight_only_stream_is_bit_exact_on_integers(M, N, K):
+    """Tokens in [-8, 8], steps powers of two: every partial sum is an integer below 2^24, so that any order gives the same."""
+    from paper_2511_22316_b200 import binding as sq
+    rng = np.random.default_rng(M * 137 + N + K)
+    Z, Wc = rng.integers(-8, 9, size=(M, K)).astype(np.float16), _codes(rng, N, K)
+    Z[0], Wc[0] = -8, -8
+    sw = (2.0 ** rng.integers(-12, -6, size=N)).astype(np.float16)
+    y = Guarded(M * N * 2)
+    sq.sq_w4a16_gemm(dev(Z), dev(ora.pack_int4_interleaved(Wc)), dev(sw), M, N, K, y)
+    torch_mod().cuda.synchronize()
+    assert sq.sq_last_device_status() == sq.SQ_OK
+    y.check()
+    want = (Z.astype(np.float32) @ Wc.astype(np.float32).T) * sw.astype(np.float32)         # exact: see above
+    assert np.array_equal(y.numpy(np.float16, (M, N)), want.astype(np.float16))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,K", [(1, 14336), (8, 4096), (8, 28672)])
+def test_weight_only_stream_stays_within_the_fp32_accumulation_bound(M, K):
+    """fp32 sums of K products, each addition off by at most one unit in the last place of a sum bounded by the sum of the
+    magnitudes, then one rounding to fp16; the same bits again on a second call."""
+    from paper_2511_22316_b200 import binding as sq
+    N = 1024
+    rng = np.random.default_rng(K + M)
+    Z, Wc = rng.standard_normal((M, K)).astype(np.float16), _codes(rng, N, K)
+    sw = rng.uniform(0.001, 0.1, size=N).astype(np.float16)
+    y, y2 = Guarded(M * N * 2), Guarded(M * N * 2)
+    args = (dev(Z), dev(ora.pack_int4_interleaved(Wc)), dev(sw), M, N, K)
+    sq.sq_w4a16_gemm(*args, y)
+    sq.sq_w4a16_gemm(*args, y2)
+    torch_mod().cuda.synchronize()
+    got, again = (g.numpy(np.float16, (M, N)) for g in (y, y2))
+    assert np.array_equal(got, again)
+    z, w, s = Z.astype(np.float64), Wc.astype(np.float64), sw.astype(np.float64)
+    want, mag = z @ w.T * s, np.abs(z) @ np.abs(w).T * s
+    assert np.all(np.abs(got - want) <= 2.0 ** -10 * np.abs(want) + K * 2.0 ** -23 * mag + 2.0 ** -24)
