@@ -201,6 +201,17 @@ __device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// kind::f16, weight-stationary form: D of M = 64 rows (A from shared memory) x N columns lies with columns [0, N / 2) on the lanes
+// 0 .. 63 and [N / 2, N) on 64 .. 127 of N / 2 TMEM columns; with M = 32, quarters of N on quarters of the lanes.
+__device__ __forceinline__ void umma_f16_ws(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.ws.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
 // 3-D tiled TMA load (x innermost; x * elemsize must be a multiple of 16 bytes).
 __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* tmap, uint64_t* bar, int32_t x,
                                             int32_t y, int32_t z) {

@@ -1,0 +1,49 @@
+"""Several tokens per accumulator in the rotate kernel (sq_rotate_quant_tc.cu) give the bits of one token at a time."""
+import numpy as np
+import pytest
+
+from gpu_util import Guarded, dev, torch_mod
+from oracle import singlequant_oracle as ora
+
+pytestmark = pytest.mark.gpu
+
+
+# Four tokens side by side and two, full and ragged lane ranges, both numbers of columns; four with n2 = 128 take the older way.
+@pytest.mark.parametrize("n1,n2", [(2, 64), (16, 64), (31, 64), (32, 64), (33, 64), (48, 64), (64, 64), (33, 128), (64, 128), (24, 128)])
+@pytest.mark.parametrize("M", [17, 301])
+def test_a_batch_has_the_bits_of_its_tokens(n1, n2, M):
+    """Rows up to 16 are rotated one to an accumulator; the same rows within a larger batch share one, and an infinity among
+    them stays in its own row (n1 = 24 with 128 columns: not so)."""
+    from paper_2511_22316_b200 import binding as sq
+    rng = np.random.default_rng(n1 * 131 + n2 + M)
+    K = n1 * n2
+    X = rng.standard_normal((M, K)).astype(np.float16)
+    X[:, rng.choice(K, 4, replace=False)] *= 50
+    bad = 5
+    R1, R2 = ora.build_rotation(X[:8].astype(np.float32), n1, n2, seed=1)
+    if n1 > 32 or n2 == 64:             # the older way multiplies a token's neighbours by zeros, which an infinity survives
+        X[bad, K // 2] = np.inf
+    rot = sq.sq_rotation_from_factors(R1, R2)
+    dX = dev(X)
+
+    def run(x, rows):
+        q, s, z = Guarded(rows * K // 2), Guarded(rows * 2), Guarded(rows * K * 2)
+        sq.sq_rotate_quant_act(rot, x, rows, q, s)
+        sq.sq_rotate_act_f16(rot, x, rows, z)
+        torch_mod().cuda.synchronize()
+        assert sq.sq_last_device_status() == sq.SQ_OK
+        for g in (q, s, z):
+            g.check()
+        return q.numpy(np.uint8, (rows, K // 2)), s.numpy(np.uint16, (rows,)), z.numpy(np.uint16, (rows, K))
+
+    whole = run(dX, M)
+    fine = np.arange(M) != bad
+    for r0 in range(0, M, 16):
+        rows = min(16, M - r0)
+        part = run(dX[r0:r0 + rows], rows)
+        keep = fine[r0:r0 + rows]
+        for a, b in zip(whole, part):
+            assert np.array_equal(a[r0:r0 + rows][keep], b[keep])
+    z = whole[2].view(np.float16)
+    assert np.all(np.isfinite(z[fine])) and np.all(np.isfinite(z[bad])) == np.all(np.isfinite(X[bad]))
+    rot.close()
