@@ -15,8 +15,8 @@
 // to global memory (16 bytes where it has 32 channels), and a warp's stores are contiguous.
 // 128 / LS tokens share one accumulator (LS = lanes per token, a power of two >= n1).  Stage 1 of all of them is one instruction
 // of the weight-stationary form: R1^T's LS rows times the tokens side by side, whose columns it lays on successive lane ranges.
-// (An MMA of 128 rows and 64 columns of an MN-major B takes 123 cycles, back to back into one accumulator, the form for two
-// tokens 126 -- and before it each token took an MMA of its own, with R1^T's image shifted to its lanes and zero rows elsewhere.
+// (Before it each token took MMAs of its own, with R1^T's image shifted to its lanes and zero rows elsewhere: two or four times
+// as many to issue and to run.
 // Same bits; 11008 x 4096 37.4 -> 33.6 us, 2048 x 4096 11.2 -> 10.2, 777 x 4096 7.1 -> 6.1, fp16 rows 41.3 -> 36.6, 11.6 -> 9.7,
 // 7.7 -> 6.6; packing 11008 x 4096 39.4 -> 35.5.)  Four tokens with n2 = 128 (n1 <= 32) have more columns than it takes and keep
 // the shifted image.  Both factors are stored pre-multiplied by 2^10 to keep
