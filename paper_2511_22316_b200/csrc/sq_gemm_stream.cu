@@ -57,8 +57,9 @@ __host__ __device__ inline StreamLayout stream_layout(int rows, int x_st, int re
   s = s > SM_MAX_STAGES ? SM_MAX_STAGES : s;
   const int lap = SM_WARPS / L.wr / 2;               // stages that the warps work on side by side
   L.stages = s / lap * lap;
-  const int f = SM_FLIGHT / L.w_st;
-  L.flight = f < 2 ? 2 : (f > L.stages ? L.stages : f);     // beyond a lap the phases could not be told apart
+  // Whole laps, one at least: block it - flight then is the same warps' as block it, see stream_loads.
+  const int f = SM_FLIGHT / L.w_st / lap * lap;
+  L.flight = f < lap ? lap : (f > L.stages ? L.stages : f);
   const int ring = L.stages * (L.w_st + L.x_st);       // (a ragged last block's fragments reach into the next stage, or the tokens')
   L.off_x = L.stages * L.w_st;
   L.off_red = overlay ? 0 : ring;
@@ -81,12 +82,16 @@ __device__ __forceinline__ void stream_loads(const StreamLayout& L, int total, i
   uint32_t idle = 0;
   while (__any_sync(0xFFFFFFFFu, left)) {
     bool go = left && (it < L.stages || mbar_test_wait(&empty[lane], ph));
-    // Noted once seen, and tested before any lane of this pass refills that block's stage: its phase cannot be missed.
+    // Block f = it - flight, which this lane looks at once it has issued block it - stages, is read by the same warps as block
+    // `it` (the flight is whole laps), after block it - stages or being that block.  So its stage is not free for a refill before
+    // this lane looks; and the tests of a pass come before its loads.  The phase cannot be missed, however far apart the warps are.
+    // (With flights of other lengths -- 9 of 12 stages -- a pair of warps a ring behind the others left this lane waiting for good.)
     if (left && !landed) {
       const int f = it - L.flight;
       landed = mbar_test_wait(&landed_bars[f % L.stages], (f / L.stages) & 1);
     }
     go = go && landed;
+    __syncwarp();
     if (go) {
       issue(it);
       it += L.stages;

@@ -7,13 +7,17 @@ from gpu_util import Guarded, dev, torch_mod
 from oracle import singlequant_oracle as ora
 
 
-def test_layouts_fit_and_their_rings_can_be_followed():
-    """Every warp meets every phase of its stages (the depth is a multiple of the stages worked on side by side), no more
-    stages are in flight than there are, and ring, sums and barriers lie apart inside the shared memory of a block."""
+def _layout_code():
     src = csrc_util.source("sq_gemm_stream.cu")
-    rows = csrc_util.run(
-        csrc_util.lines(src, r"^constexpr int SM_.*$") + "\n" + csrc_util.block(src, "struct StreamLayout")
-        + csrc_util.block(src, "__host__ __device__ inline StreamLayout stream_layout(") + """
+    return (csrc_util.lines(src, r"^constexpr int SM_.*$") + "\n" + csrc_util.block(src, "struct StreamLayout")
+            + csrc_util.block(src, "__host__ __device__ inline StreamLayout stream_layout(")
+            + csrc_util.block(src, "int stream_blocks("))                # and stream_rows, up to its closing brace
+
+
+def test_layouts_fit_and_their_rings_can_be_followed():
+    """Every warp meets every phase of its stages (the depth is a multiple of the stages worked on side by side), the loads in
+    flight are whole laps and no more than there are stages, and ring, sums and barriers lie apart inside a block's shared memory."""
+    rows = csrc_util.run(_layout_code() + """
 void show(int kind, StreamLayout L, int red) {
   printf("%d %d %d %d %d %d %d %d %d %d %d %d\\n", kind, L.rows, L.wr, L.nb, L.stages, L.flight, L.w_st, L.x_st, L.off_x,
          L.off_red, L.off_bar, L.total - 3 * SM_MAX_STAGES * 8);
@@ -27,7 +31,7 @@ int main() {
     assert len(rows) == 61 * 3
     for kind, r, wr, nb, stages, flight, w_st, x_st, off_x, off_red, off_bar, end in (map(int, x) for x in rows):
         lap = 16 // wr // 2
-        assert stages >= lap and stages % lap == 0 and stages <= 32 and 2 <= flight <= stages, r
+        assert stages >= lap and stages % lap == 0 and stages <= 32 and lap <= flight <= stages and flight % lap == 0, r
         assert nb <= 4 and nb * wr * 16 >= r and off_x == stages * w_st and w_st >= 128 * r
         ring = off_x + stages * x_st
         sums = 8 * 136 * 4 if kind == 0 else (4 if wr == 2 else 8) * 8 * 132 * 4
@@ -46,6 +50,26 @@ def _rows(rows, M):
 # block; ragged last tiles; one token and a full tile of eight.
 SHAPES = [(1, 128, 256), (8, 130, 288), (3, 200, 544), (8, 2048, 14336), (5, 4106, 1312)] + [
     (8, _rows(r, 8), 800) for r in (16, 18, 32, 34, 48, 50, 64, 66, 96, 98, 128)] + [(8, _rows(128, 8) + 6, 576), (2, 40002, 288)]
+# A ring that wraps with fewer loads in flight than it has stages: one tile per block, two, and two of nearly full height.
+SHAPES += [(1, 14336, 4096), (8, 28672, 8192), (8, 32000, 4096)]
+
+
+@pytest.mark.parametrize("kernel", ["w4a4", "weight-only"])
+def test_the_shapes_wrap_their_rings_with_a_limited_flight(kernel):
+    """Among the products below: rings that wrap while the loads in flight are limited, with one tile per block and with several."""
+    wide = [s for s in SHAPES if s[1] > 74 * 128]                 # more channels than a cluster per two SMs takes: K is not split
+    rows = csrc_util.run(_layout_code() + """
+int main(int n, char** v) {
+  for (int i = 1; i + 2 < n; i += 3) {
+    const int M = atoi(v[i]), N = atoi(v[i + 1]), K = atoi(v[i + 2]), blocks = stream_blocks(148, M), rows = stream_rows(N, blocks);
+    const int tiles = (N + rows - 1) / rows, waves = (tiles + blocks - 1) / blocks;
+    const StreamLayout L = W4A4 ? stream_layout(rows, SM_NT * 128, SM_NT * SM_RP8 * 4, false)
+                                : stream_layout(rows, SM_NT * 512, 8 / (rows > 32 ? 2 : 1) * SM_PART * 4, tiles <= blocks);
+    printf("%d %d %d %d\\n", waves, waves * ((K + 255) / 256), L.stages, L.flight);
+  }
+}""".replace("W4A4", "1" if kernel == "w4a4" else "0"), *(v for s in wide for v in s))
+    limited = {waves > 1 for waves, blocks, stages, flight in (map(int, r) for r in rows) if blocks > stages > flight}
+    assert limited == {False, True}
 
 
 def _codes(rng, n, K):
@@ -68,7 +92,7 @@ def test_w4a4_stream_is_bit_exact(M, N, K):
     want = Xc.astype(np.float64) @ Wc.astype(np.float64).T                   # integers below 2^53
     assert np.array_equal(acc.numpy(np.int32, (M, N)), want.astype(np.int32))
     apart = y.numpy(np.float16, (M, N)).view(np.int16).astype(int) - ora.dequant(want.astype(np.int32), sx, sw).view(np.int16)
-    assert np.abs(apart).max() <= 1                                          # the steps' product is rounded to fp32
+    assert np.abs(apart).max() <= 1       # its product with the steps is rounded to fp32 before fp16
 
 
 # The same, and K over clusters of 2, 4 and 8 (few channels, long K).

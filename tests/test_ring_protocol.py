@@ -1,4 +1,4 @@
-"""The rings of the W4A4 products, explored on the CPU.
+"""The rings of the products, explored on the CPU.
 
 Two groups of converter warps take the blocks of a ring in turn and tell the phases of a stage apart by their parity
 (mbarrier.try_wait.parity).  Loads that are in flight together may land in any order.  The model below walks every
@@ -89,3 +89,63 @@ int main() { pair<PairWide>("wide"); pair<PairNarrow>("narrow"); dec<16>(); dec<
 def test_no_group_is_let_through_before_its_load_has_landed(rings, name):
     stages, op_stages, groups, operand_first = rings[name]
     assert let_through_too_early(stages, op_stages, groups, bool(operand_first)) is None
+
+
+def left_waiting(stages, flight, pairs, blocks, held):
+    """The loading warp of the stream kernels (stream_loads): lane s owns stage s, block `it` is requested when its stage is free and
+    block it - flight has been seen landed; `pairs` pairs of warps take the blocks in turn.  Pair `held` does nothing until all the
+    others have come to a stop, then it goes on too.  Returns the pairs that do not come to their end."""
+    first = min(flight, blocks)
+    nxt = [s + stages if s < first else s for s in range(stages)]
+    landed, freed = [int(s < first) for s in range(stages)], [0] * stages              # phases completed per stage
+    seen, at = [False] * stages, list(range(pairs))
+
+    def passes(phases, parity):
+        return (phases - 1) & 1 == parity
+
+    def turn(active):
+        moved, go = False, []
+        for s, it in enumerate(nxt):
+            if it >= blocks:
+                continue
+            f = it - flight
+            if not seen[s] and passes(landed[f % stages], (f // stages) & 1):
+                seen[s] = moved = True
+            if seen[s] and (it < stages or passes(freed[s], (it // stages - 1) & 1)):
+                go.append(s)
+        for s in go:                                            # requested, and landed at once
+            landed[s], nxt[s], seen[s], moved = landed[s] + 1, nxt[s] + stages, False, True
+        for p in active:
+            s = at[p] % stages
+            if at[p] < blocks and landed[s] == at[p] // stages + 1:
+                freed[s], at[p], moved = freed[s] + 1, at[p] + pairs, True
+        return moved
+
+    for active in (set(range(pairs)) - {held}, range(pairs)):
+        while turn(active):
+            pass
+    return [p for p in range(pairs) if at[p] < blocks]
+
+
+def test_a_flight_of_parts_of_a_lap_can_leave_a_lane_waiting():
+    assert all(left_waiting(12, 9, 4, 64, held) for held in range(4))
+    assert left_waiting(28, 21, 4, 112, 0) and left_waiting(32, 25, 4, 200, 0)
+    assert not left_waiting(12, 8, 4, 64, 0) and not left_waiting(12, 12, 4, 64, 0)
+
+
+def test_no_lane_of_a_stream_ring_is_left_waiting():
+    src = source("sq_gemm_stream.cu")
+    rows = run(lines(src, r"^constexpr int SM_.*$") + "\n" + block(src, "struct StreamLayout")
+               + block(src, "__host__ __device__ inline StreamLayout stream_layout(") + """
+void show(const StreamLayout& L) { printf("%d %d %d\\n", L.stages, L.flight, SM_WARPS / L.wr / 2); }
+int main() {
+  for (int r = 8; r <= SM_MAX_ROWS; r += 2) {
+    show(stream_layout(r, SM_NT * 128, SM_NT * SM_RP8 * 4, false));
+    for (int o = 0; o < 2; ++o) show(stream_layout(r, SM_NT * 512, 8 / (r > 32 ? 2 : 1) * SM_PART * 4, o));
+  }
+}""")
+    rings = {tuple(int(v) for v in r) for r in rows}
+    assert len(rings) > 10
+    for stages, flight, pairs in rings:
+        for held in range(pairs):
+            assert left_waiting(stages, flight, pairs, 8 * stages, held) == [], (stages, flight, pairs, held)
