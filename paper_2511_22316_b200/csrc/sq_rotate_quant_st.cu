@@ -53,8 +53,8 @@ struct StCoef {
   float c0;        // 2^-10 (the image's pre-scale) x 1/sqrt(n2) when H is present
 };
 
-// An accumulator slot is 128 TMEM columns wide, so that every MMA has N = 128 (an MMA of N = 64 costs
-// the issuing thread as much as one of N = 128 and the tensor pipe three quarters of it).  Its lanes
+// An accumulator slot is 128 TMEM columns wide (an MMA of N = 64 costs the issuing thread as much as one of N = 128 and the
+// tensor pipe three quarters of it).  Its lanes
 // hold G = 128 / LS tokens side by side (LS = lanes per token, a power of two >= n1); its columns
 // hold CH = 128 / n2 tokens side by side: one "super-group" is TPS = G * CH consecutive tokens.
 struct StLayout {
@@ -197,12 +197,15 @@ rotate_quant_st_kernel(const __grid_constant__ StLayout L, int n1, int rows, con
   } else if (warp == 1) {
     // ------------------------------ MMA issuer: D[p'][q] = sum_p R1[p][p'] X~[p][q] --------------------
     if (elect_one()) {
-      // A K-major (shared: the image of R1^T shifted to the token's lanes), B MN-major (bit 16): the
-      // tokens' TMA tiles as they landed, two 64-column groups x_half apart.  Descriptors of one
-      // super-group differ only in the start-address field of their low word (no carry out of it).
+      // A K-major (shared: R1^T), B MN-major (bit 16): the tokens' TMA tiles as they landed.  One token on the lanes: both
+      // 64-column groups, x_half apart, in one instruction.  Several: one of the weight-stationary form (as in the dense kernel)
+      // per group, the tokens x_tile apart; with R1^T shifted to each token's lanes and zero rows elsewhere an infinity came out
+      // as NaN in the rows beside its own (and it took longer: 333 x 4096 5.54 -> 5.24 us, 2048 x 2048 7.18 -> 6.77).
+      // Descriptors of one super-group differ only in the start-address field of their low word (no carry out of it).
       constexpr uint32_t idesc1 = umma_idesc(/*c=f32*/ 1, /*a=f16*/ 0, /*b=f16*/ 0, 128, 128) | (1u << 16);
+      const uint32_t idesc_ws = umma_idesc(1, 0, 0, static_cast<uint32_t>(LS), static_cast<uint32_t>(64 * G)) | (1u << 16);
       const uint64_t a1_desc0 = umma_desc_sw128(smem_u32(a1s));
-      const uint64_t x_desc0 = umma_desc_sw128_mn(smem_u32(xs), static_cast<uint32_t>(L.x_half));
+      const uint64_t x_desc0 = umma_desc_sw128_mn(smem_u32(xs), static_cast<uint32_t>(G == 1 ? L.x_half : L.x_tile));
       const uint32_t a_hi = static_cast<uint32_t>(a1_desc0 >> 32), b_hi = static_cast<uint32_t>(x_desc0 >> 32);
       const uint32_t a_lo0 = static_cast<uint32_t>(a1_desc0), b_lo0 = static_cast<uint32_t>(x_desc0);
       const uint32_t lo_part = static_cast<uint32_t>(L.a1_part >> 4), a_tile = static_cast<uint32_t>(L.a1_tile >> 4);
@@ -216,18 +219,26 @@ rotate_quant_st_kernel(const __grid_constant__ StLayout L, int n1, int rows, con
         tc_fence_after_sync();
         const uint32_t d = tmem_base + slot * 128;
         uint32_t acc = 0;
-        for (int tk = 0; tk < G; ++tk) {
-          uint32_t b_lo = b_lo0 + static_cast<uint32_t>((xs_i * L.x_bytes + tk * L.x_tile) >> 4);
-          uint32_t a_lo = a_lo0 + static_cast<uint32_t>(((128 - LS - tk * LS) * 128) >> 4);
-          for (int k4 = 0; k4 < ksteps1; k4 += 4, a_lo += a_tile) {
+        uint32_t b_lo = b_lo0 + static_cast<uint32_t>((xs_i * L.x_bytes) >> 4);
+        uint32_t a_lo = a_lo0 + static_cast<uint32_t>(((128 - LS) * 128) >> 4);
+        for (int k4 = 0; k4 < ksteps1; k4 += 4, a_lo += a_tile) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              if (k4 + kk < ksteps1) {
-                umma_f16(d, desc_from(a_hi, a_lo + 2 * kk), desc_from(b_hi, b_lo), idesc1, acc);             // hi
-                umma_f16(d, desc_from(a_hi, a_lo + 2 * kk + lo_part), desc_from(b_hi, b_lo), idesc1, 1u);   // lo
-                acc = 1;
-                b_lo += 2048 >> 4;
+          for (int kk = 0; kk < 4; ++kk) {
+            if (k4 + kk < ksteps1) {
+              const uint64_t ah = desc_from(a_hi, a_lo + 2 * kk), al = desc_from(a_hi, a_lo + 2 * kk + lo_part);
+              if (G == 1) {
+                umma_f16(d, ah, desc_from(b_hi, b_lo), idesc1, acc);             // hi
+                umma_f16(d, al, desc_from(b_hi, b_lo), idesc1, 1u);              // lo
+              } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  const uint64_t bd = desc_from(b_hi, b_lo + static_cast<uint32_t>((h * L.x_half) >> 4));
+                  umma_f16_ws(d + 64 * h, ah, bd, idesc_ws, acc);
+                  umma_f16_ws(d + 64 * h, al, bd, idesc_ws, 1u);
+                }
               }
+              acc = 1;
+              b_lo += 2048 >> 4;
             }
           }
         }

@@ -18,8 +18,10 @@
 // (Before it each token took MMAs of its own, with R1^T's image shifted to its lanes and zero rows elsewhere: two or four times
 // as many to issue and to run.
 // Same bits; 11008 x 4096 37.4 -> 33.6 us, 2048 x 4096 11.2 -> 10.2, 777 x 4096 7.1 -> 6.1, fp16 rows 41.3 -> 36.6, 11.6 -> 9.7,
-// 7.7 -> 6.6; packing 11008 x 4096 39.4 -> 35.5.)  Four tokens with n2 = 128 (n1 <= 32) have more columns than it takes and keep
-// the shifted image.  Both factors are stored pre-multiplied by 2^10 to keep
+// 7.7 -> 6.6; packing 11008 x 4096 39.4 -> 35.5.)  Four tokens with n2 = 128 (n1 <= 32) have more columns than the 256 it takes:
+// one instruction for the first 64 columns of each and one for the others (2048 x 3072 12.1 -> 11.6, fp16 rows 11.2 -> 10.5).  The
+// zero rows let an infinity into the tokens beside its own, as NaN; now it stays in its row.  Both factors are stored
+// pre-multiplied by 2^10 to keep
 // the lo parts out of the fp16 subnormal range; every power-of-two factor is divided out exactly.
 //
 // Warp roles: warp 0 lane 0 = TMA producer, warp 1 lane 0 = MMA issuer, then the warps of the S
@@ -57,7 +59,7 @@ struct RqLayout {
   int LS, G, N1, KA1, XQ, S, XS, rowsA;
   int a1_tile, a1_part, a1_bytes, b2_tile, b2_part, b2_bytes, x_tile, x_token, x_bytes;
   int off_a1, off_b2, off_x, off_misc, total;
-  int ws;               // stage 1 of all of an accumulator's tokens in one instruction
+  int parts;            // instructions per step of stage 1 when several tokens share an accumulator
 };
 
 // `one_token`: one token per accumulator (the other lanes stay zero) instead of as many as fit.
@@ -65,7 +67,7 @@ __host__ __device__ inline RqLayout rq_layout(int n1, int n2, int budget = kMaxD
   RqLayout L;
   L.LS = n1 <= 32 ? 32 : (n1 <= 64 ? 64 : 128);   // TMEM lanes per token
   L.G = one_token ? 1 : 128 / L.LS;               // tokens per accumulator
-  L.ws = L.G > 1 && L.G * n2 <= 256;              // its N is the columns of all of them, 256 at most
+  L.parts = L.G * n2 <= 256 ? 1 : 2;              // the N of one is 256 at most
   L.N1 = (n1 + 15) & ~15;                         // K of stage 1, padded to the MMA's K = 16
   L.KA1 = (L.N1 + 63) / 64;                       // 64-wide K atoms of stage 1
   L.XQ = n2 / 64;                                 // 64-wide column blocks of a token
@@ -438,38 +440,38 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       // stage 1: A K-major (shared), B MN-major (bit 16); stage 2: A from TMEM, B K-major
       const uint32_t idesc1 = umma_idesc(/*c=f32*/ 1, /*a=f16*/ 0, /*b=f16*/ 0, 128, N2) | (1u << 16);
       const uint32_t idesc2 = umma_idesc(/*c=f32*/ 1, /*a=f16*/ 0, /*b=f16*/ 0, 128, N2);
-      // weight-stationary: M = LS rows, N = the columns of G tokens, whose tiles follow one another at the stride of a column block
-      const uint32_t idesc_ws = umma_idesc(1, 0, 0, static_cast<uint32_t>(LS), static_cast<uint32_t>(N2 * G)) | (1u << 16);
+      // weight-stationary: M = LS rows, N = the columns of G tokens, whose tiles follow one another at the stride of a column block,
+      // or 64 columns of each at the stride of a token
+      const bool halves = N2 == 128 && L.parts == 2;
+      const uint32_t idesc_ws = umma_idesc(1, 0, 0, static_cast<uint32_t>(LS), static_cast<uint32_t>((halves ? 64 : N2) * G)) | (1u << 16);
       const uint64_t a1_desc0 = umma_desc_sw128(smem_u32(a1s)), b2_desc0 = umma_desc_sw128(smem_u32(b2s));
-      const uint64_t x_desc0 = umma_desc_sw128_mn(smem_u32(xs), static_cast<uint32_t>(L.x_tile));
+      const uint64_t x_desc0 = umma_desc_sw128_mn(smem_u32(xs), static_cast<uint32_t>(halves ? L.x_token : L.x_tile));
       const int ksteps1 = L.N1 / 16;                 // K = p, 16 per MMA
       bool ok = mbar_wait(img_full, 0, RQ_IMG, limit);
       auto stage1 = [&](int i, int xs_i) {
         const int slot = i % S;
         tc_fence_after_sync();
         const uint32_t d1 = tmem_base + slot * SLOT_COLS;
-        uint32_t acc = 0;
         // descriptors differ only in their start-address field (16-byte units, no carry out of it)
-        if (L.ws) {                                    // the sums of every token are those of the loop below, in its order
-          uint64_t bd = x_desc0 + ((xs_i * L.x_bytes) >> 4);
-          const uint64_t ad = a1_desc0 + (((128 - LS) * 128) >> 4);
-          for (int ks = 0; ks < ksteps1; ++ks, bd += 2048 >> 4) {
-            const uint64_t ah = ad + (((ks >> 2) * L.a1_tile + (ks & 3) * 32) >> 4);
-            umma_f16_ws(d1, ah, bd, idesc_ws, acc);                        // hi
-            umma_f16_ws(d1, ah + (L.a1_part >> 4), bd, idesc_ws, 1u);      // lo
-            acc = 1;
+        const uint64_t ad = a1_desc0 + (((128 - LS) * 128) >> 4), bd0 = x_desc0 + ((xs_i * L.x_bytes) >> 4);
+        if (G > 1) {
+          for (int h = 0; h < (halves ? 2 : 1); ++h) {
+            uint64_t bd = bd0 + ((h * L.x_tile) >> 4);
+            uint32_t acc = 0;
+            for (int ks = 0; ks < ksteps1; ++ks, bd += 2048 >> 4) {
+              const uint64_t ah = ad + (((ks >> 2) * L.a1_tile + (ks & 3) * 32) >> 4);
+              umma_f16_ws(d1 + 64 * h, ah, bd, idesc_ws, acc);                       // hi
+              umma_f16_ws(d1 + 64 * h, ah + (L.a1_part >> 4), bd, idesc_ws, 1u);     // lo
+              acc = 1;
+            }
           }
-          umma_commit(&x_empty[xs_i]);
-          umma_commit(&d1_full[slot]);
-          return;
-        }
-        for (int tk = 0; tk < G; ++tk) {
-          uint64_t bd = x_desc0 + ((xs_i * L.x_bytes + tk * L.x_token) >> 4);
-          const uint64_t ad = a1_desc0 + (((128 - LS - tk * LS) * 128) >> 4);
+        } else {
+          uint64_t bd = bd0;
+          uint32_t acc = 0;
           for (int ks = 0; ks < ksteps1; ++ks, bd += 2048 >> 4) {
             const uint64_t ah = ad + (((ks >> 2) * L.a1_tile + (ks & 3) * 32) >> 4);
-            umma_f16(d1, ah, bd, idesc1, acc);                         // hi
-            umma_f16(d1, ah + (L.a1_part >> 4), bd, idesc1, 1u);       // lo
+            umma_f16(d1, ah, bd, idesc1, acc);
+            umma_f16(d1, ah + (L.a1_part >> 4), bd, idesc1, 1u);
             acc = 1;
           }
         }
@@ -636,9 +638,10 @@ bool rotate_quant_tc_prepare(sq_rotation* h) {
   const int n1 = h->n1, n2 = h->n2;
   const RqLayout L = rq_layout(n1, n2);
   std::vector<unsigned char> a1(L.a1_bytes, 0), b2(L.b2_bytes, 0);
-  // A1 (stage-1 A operand): rows = lanes, K = p.  R1^T sits at rows [128 - LS, 128 - LS + n1) of a
-  // (256 - LS)-row image; token slot g reads it from row (128 - LS) - g * LS on, which puts R1^T
-  // on lanes [g * LS, g * LS + n1) and zero rows on every other lane.
+  // A1 (stage-1 A operand): rows = lanes, K = p.  R1^T sits at rows [128 - LS, 128 - LS + n1) of a (256 - LS)-row image.  A
+  // single token takes 128 rows from there on, which leaves zeros on the lanes behind its own; several tokens side by side take
+  // LS.  (The zero rows ahead of R1^T belong to images shifted to the other tokens' lanes, which nothing uses any more; they
+  // are still copied into every CTA, and room for X is lost to them.)
   for (int pp = 0; pp < n1; ++pp)
     for (int p = 0; p < n1; ++p) {
       __half hi, lo;

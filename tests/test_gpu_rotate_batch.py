@@ -8,12 +8,13 @@ from oracle import singlequant_oracle as ora
 pytestmark = pytest.mark.gpu
 
 
-# Four tokens side by side and two, full and ragged lane ranges, both numbers of columns; four with n2 = 128 take the older way.
-@pytest.mark.parametrize("n1,n2", [(2, 64), (16, 64), (31, 64), (32, 64), (33, 64), (48, 64), (64, 64), (33, 128), (64, 128), (24, 128)])
+# Four tokens side by side and two, full and ragged lane ranges, both numbers of columns.
+@pytest.mark.parametrize("n1,n2", [(2, 64), (16, 64), (31, 64), (32, 64), (33, 64), (48, 64), (64, 64), (33, 128), (64, 128), (2, 128),
+                                   (24, 128), (32, 128)])
 @pytest.mark.parametrize("M", [17, 301])
 def test_a_batch_has_the_bits_of_its_tokens(n1, n2, M):
     """Rows up to 16 are rotated one to an accumulator; the same rows within a larger batch share one, and an infinity among
-    them stays in its own row (n1 = 24 with 128 columns: not so)."""
+    them stays in its own row."""
     from paper_2511_22316_b200 import binding as sq
     rng = np.random.default_rng(n1 * 131 + n2 + M)
     K = n1 * n2
@@ -21,8 +22,7 @@ def test_a_batch_has_the_bits_of_its_tokens(n1, n2, M):
     X[:, rng.choice(K, 4, replace=False)] *= 50
     bad = 5
     R1, R2 = ora.build_rotation(X[:8].astype(np.float32), n1, n2, seed=1)
-    if n1 > 32 or n2 == 64:             # the older way multiplies a token's neighbours by zeros, which an infinity survives
-        X[bad, K // 2] = np.inf
+    X[bad, K // 2] = np.inf
     rot = sq.sq_rotation_from_factors(R1, R2)
     dX = dev(X)
 
@@ -45,5 +45,27 @@ def test_a_batch_has_the_bits_of_its_tokens(n1, n2, M):
         for a, b in zip(whole, part):
             assert np.array_equal(a[r0:r0 + rows][keep], b[keep])
     z = whole[2].view(np.float16)
-    assert np.all(np.isfinite(z[fine])) and np.all(np.isfinite(z[bad])) == np.all(np.isfinite(X[bad]))
+    assert np.all(np.isfinite(z[fine])) and not np.all(np.isfinite(z[bad]))
+    rot.close()
+
+
+@pytest.mark.parametrize("n1,n2", [(16, 64), (48, 64), (64, 64), (24, 128), (64, 128)])
+def test_an_infinity_stays_in_its_row_with_the_structured_factor(n1, n2):
+    """Two or four tokens on the lanes of an accumulator (sq_rotate_quant_st.cu): the other rows have the bits that they have
+    without the infinity."""
+    from paper_2511_22316_b200 import binding as sq
+    M, K, bad = 37, n1 * n2, 5
+    X = np.random.default_rng(n1 + n2).standard_normal((M, K)).astype(np.float16)
+    rot = sq.sq_build_rotation(X[:8].astype(np.float32), n1, n2, flags=sq.SQ_ROT_DEFAULT | sq.SQ_ROT_APPLY_STRUCTURED, seed=1)
+    assert rot.structured
+    out = []
+    for value in (X[bad, K // 2], np.inf):
+        X[bad, K // 2] = value
+        q, s = Guarded(M * K // 2), Guarded(M * 2)
+        sq.sq_rotate_quant_act(rot, dev(X), M, q, s)
+        torch_mod().cuda.synchronize()
+        assert sq.sq_last_device_status() == sq.SQ_OK
+        q.check(), s.check()
+        out.append((np.delete(q.numpy(np.uint8, (M, K // 2)), bad, 0), np.delete(s.numpy(np.uint16, (M,)), bad)))
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
     rot.close()
