@@ -37,6 +37,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "sq_internal.h"
@@ -337,7 +338,10 @@ inline int rq_smem(const RqLayout& L, int ctas_per_sm) { return std::max(L.total
 
 // The kernel's body, for CTA `cta` of `ncta` that share the token groups (the fused decode kernel of
 // sq_linear_fused.cu runs it in its first CTAs, with more warps in the block than the roles below use).
-template <int N2, int S, int CW = 1, bool F16OUT = false>
+// `TOKENS`: one token per accumulator (1) or several (2), where that is known when the kernel is compiled; 0: by the layout.  With
+// the choice left to the kernel the MMA issuer lost time over it: 1 x 4096 3.65 us against 3.55, 50 x 14336 (112 x 128) 5.85
+// against 5.68, 2048 x 14336 32.8 against 31.1; three MLP layers of 50 tokens 49.8 against 47.9.
+template <int N2, int S, int CW = 1, bool F16OUT = false, int TOKENS = 0>
 __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, const RqLayout& L,
                                                      const unsigned char* __restrict__ a1_img,
                                                      const unsigned char* __restrict__ b2_img, int n1, int rows,
@@ -349,7 +353,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
   // The layout comes from the host (the same rq_layout call that sized the shared memory); group
   // counts are 32-bit: the set-up is on the critical path of a decode step.
   const int n = n1 * N2;
-  const int G = L.G, LS = L.LS;
+  const int G = TOKENS == 1 ? 1 : L.G, LS = L.LS;
 
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
@@ -442,7 +446,7 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
       const uint32_t idesc2 = umma_idesc(/*c=f32*/ 1, /*a=f16*/ 0, /*b=f16*/ 0, 128, N2);
       // weight-stationary: M = LS rows, N = the columns of G tokens, whose tiles follow one another at the stride of a column block,
       // or 64 columns of each at the stride of a token
-      const bool halves = N2 == 128 && L.parts == 2;
+      const bool halves = N2 == 128 && TOKENS != 1 && L.parts == 2;
       const uint32_t idesc_ws = umma_idesc(1, 0, 0, static_cast<uint32_t>(LS), static_cast<uint32_t>((halves ? 64 : N2) * G)) | (1u << 16);
       const uint64_t a1_desc0 = umma_desc_sw128(smem_u32(a1s)), b2_desc0 = umma_desc_sw128(smem_u32(b2s));
       const uint64_t x_desc0 = umma_desc_sw128_mn(smem_u32(xs), static_cast<uint32_t>(halves ? L.x_token : L.x_tile));
@@ -454,17 +458,19 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
         const uint32_t d1 = tmem_base + slot * SLOT_COLS;
         // descriptors differ only in their start-address field (16-byte units, no carry out of it)
         const uint64_t ad = a1_desc0 + (((128 - LS) * 128) >> 4), bd0 = x_desc0 + ((xs_i * L.x_bytes) >> 4);
-        if (G > 1) {
-          for (int h = 0; h < (halves ? 2 : 1); ++h) {
-            uint64_t bd = bd0 + ((h * L.x_tile) >> 4);
+        if (TOKENS == 2 || (TOKENS == 0 && G > 1)) {
+          auto steps = [&](uint32_t d, uint64_t bd) {
             uint32_t acc = 0;
+#pragma unroll 2                                       // 333 x 4096 4.76 us, 4.86 with the compiler's four
             for (int ks = 0; ks < ksteps1; ++ks, bd += 2048 >> 4) {
               const uint64_t ah = ad + (((ks >> 2) * L.a1_tile + (ks & 3) * 32) >> 4);
-              umma_f16_ws(d1 + 64 * h, ah, bd, idesc_ws, acc);                       // hi
-              umma_f16_ws(d1 + 64 * h, ah + (L.a1_part >> 4), bd, idesc_ws, 1u);     // lo
+              umma_f16_ws(d, ah, bd, idesc_ws, acc);                       // hi
+              umma_f16_ws(d, ah + (L.a1_part >> 4), bd, idesc_ws, 1u);     // lo
               acc = 1;
             }
-          }
+          };
+          steps(d1, bd0);
+          if (halves) steps(d1 + 64, bd0 + (L.x_tile >> 4));
         } else {
           uint64_t bd = bd0;
           uint32_t acc = 0;
@@ -602,12 +608,12 @@ __device__ __forceinline__ void rotate_quant_tc_body(const CUtensorMap& tmap_x, 
 
 // S accumulator slots (= compute groups) per CTA.  With S * 2 * N2 = 256 TMEM columns two CTAs share
 // an SM (each with its own producer and MMA issuer); with 512 a CTA has the SM to itself.
-template <int N2, int S, int CW = 1, bool F16OUT = false>
+template <int N2, int S, int CW = 1, bool F16OUT = false, int TOKENS = 0>
 __global__ void __launch_bounds__((2 + 4 * S * CW) * 32, (CW == 1 && S * 2 * N2 <= 256) ? 2 : 1)
 rotate_quant_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ RqLayout L,
                        const unsigned char* __restrict__ a1_img, const unsigned char* __restrict__ b2_img, int n1,
                        int rows, uint8_t* __restrict__ Xq, __half* __restrict__ scales, float* __restrict__ Zdbg) {
-  rotate_quant_tc_body<N2, S, CW, F16OUT>(tmap_x, L, a1_img, b2_img, n1, rows, Xq, scales, Zdbg, static_cast<int>(blockIdx.x),
+  rotate_quant_tc_body<N2, S, CW, F16OUT, TOKENS>(tmap_x, L, a1_img, b2_img, n1, rows, Xq, scales, Zdbg, static_cast<int>(blockIdx.x),
                               static_cast<int>(gridDim.x));
 }
 
@@ -702,29 +708,34 @@ sq_status_t launch_rotate_quant_tc(const sq_rotation* h, const void* X, int64_t 
   const long long ngroups = (rows + L.G - 1) / L.G;
   const unsigned char* a1 = static_cast<const unsigned char*>(h->dA1img);
   const unsigned char* b2 = static_cast<const unsigned char*>(h->dB2img);
-  auto launch = [&](auto kern, int slots, int ctas_per_sm, int cw = 1) -> bool {
+  auto launch = [&](auto n2_c, auto slots_c, auto cw_c, auto f16_c, int ctas_per_sm) -> bool {
+    constexpr int N2 = decltype(n2_c)::value, S = decltype(slots_c)::value, CW = decltype(cw_c)::value;
+    constexpr bool F16 = decltype(f16_c)::value;
+    auto kern = rotate_quant_tc_kernel<N2, S, CW, F16, 1>;
+    if constexpr (S == 2) {                          // one slot is one token at a time; four are for n1 > 64
+      if (L.G > 1) kern = rotate_quant_tc_kernel<N2, S, CW, F16, 2>;
+    }
     const int smem = rq_smem(L, ctas_per_sm);
     if (!ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem)) return false;
     const unsigned grid = static_cast<unsigned>(std::min<long long>(ngroups, static_cast<long long>(sms) * ctas_per_sm));
-    return launch_dependent(kern, dim3(grid), dim3((2 + 4 * slots * cw) * 32), static_cast<size_t>(smem), s, mx, L, a1, b2, n1,
+    return launch_dependent(kern, dim3(grid), dim3((2 + 4 * S * CW) * 32), static_cast<size_t>(smem), s, mx, L, a1, b2, n1,
                             static_cast<int>(rows), static_cast<uint8_t*>(Xq), static_cast<__half*>(scales),
                             Zdbg) == cudaSuccess;
   };
-  bool ok;
   // n2 = 128 (one CTA per SM, two slots): eight warps per slot, 18 in all instead of 10 -- measured 10 %
   // faster on 4096 x 8192 (39.7 -> 35.5 us) and 0.8 us on the decode batches (6.6 -> 5.8 us).  With n2 = 64
   // and two CTAs per SM the same split leaves 56 registers per thread and was slower (12.0 -> 15.9 us).
-  if (few) {
-    if (f16out) ok = n2 == 64 ? launch(rotate_quant_tc_kernel<64, 1, 2, true>, 1, 2, 2) : launch(rotate_quant_tc_kernel<128, 1, 2, true>, 1, 2, 2);
-    else ok = n2 == 64 ? launch(rotate_quant_tc_kernel<64, 1, 2>, 1, 1, 2) : launch(rotate_quant_tc_kernel<128, 1, 2>, 1, 1, 2);
-  } else if (f16out) {
-    // rotation only: Xq receives the rotated rows as fp16 [rows x n], `scales` is not touched
-    if (n2 == 64 && dual) ok = launch(rotate_quant_tc_kernel<64, 2, 1, true>, 2, 2);
-    else if (n2 == 64) ok = launch(rotate_quant_tc_kernel<64, 4, 1, true>, 4, 1);
-    else ok = launch(rotate_quant_tc_kernel<128, 2, 2, true>, 2, 1, 2);
-  } else if (n2 == 64 && dual) ok = launch(rotate_quant_tc_kernel<64, 2>, 2, 2);
-  else if (n2 == 64) ok = launch(rotate_quant_tc_kernel<64, 4>, 4, 1);
-  else ok = launch(rotate_quant_tc_kernel<128, 2, 2>, 2, 1, 2);
+  using std::integral_constant;
+  auto form = [&](auto f16) -> bool {                // rotation only: Xq receives the rotated rows as fp16, `scales` is not touched
+    const integral_constant<int, 64> c64;
+    const integral_constant<int, 128> c128;
+    const integral_constant<int, 1> one;
+    const integral_constant<int, 2> two;
+    if (few) return n2 == 64 ? launch(c64, one, two, f16, f16 ? 2 : 1) : launch(c128, one, two, f16, f16 ? 2 : 1);
+    if (n2 == 128) return launch(c128, two, two, f16, 1);
+    return dual ? launch(c64, two, one, f16, 2) : launch(c64, integral_constant<int, 4>(), one, f16, 1);
+  };
+  const bool ok = f16out ? form(std::true_type()) : form(std::false_type());
   if (!ok) return SQ_ERR_CUDA;
   count_launch();
   return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ERR_CUDA;
