@@ -434,9 +434,9 @@ sq_status_t launch_tc(const void* Xq, const void* sx, const void* Wq, const void
 
 }  // namespace
 
-// What the stream kernel does not take.  One or two tokens are pure streaming: dot products on the CUDA cores.  With three or
-// four the dot-product kernel is bound by its dp4a and shared-memory issue and the tensor-core decode kernel
-// (whose time does not depend on M up to 16) is as fast or faster, where it supports the shape.
+// What the stream kernel leaves.  One or two tokens: dot products on the CUDA cores.  With three or four the dot-product kernel is
+// bound by its dp4a and shared-memory issue and the tensor-core decode kernel (whose time does not depend on M up to 16) is as
+// fast or faster, where it supports the shape.
 static bool use_gemv(int64_t M, int64_t N, int64_t K) {
   return gemv_supported(M, N, K) && (M <= 2 || !gemm_decode_supported(M, N, K));
 }

@@ -547,13 +547,27 @@ int stream_rows(int N, int blocks) {
 
 }  // namespace
 
-// Against the kernels that took these calls before (layers over 18 shapes, K 512 to 28672, 1 / 2 / 4 / 8 tokens: 1.07 / 1.13 /
-// 1.15 / 1.13 on the geometric mean).  One token and 8 to 16 MB of weights stays with the dot products, which have all of them in
-// registers before the token exists: 3072 x 8192 7.28 us against 7.80, 5120 x 5120 8.10 and 8.35; above, 4096 x 11008 9.70 and 9.10,
-// and below, 2048 x 5632 6.34 and 6.22, this kernel is ahead.
+// Against the kernels that took these calls before: layers over 31 shapes, K 256 to 28672, 1 / 2 / 4 / 8 tokens, 1.07 / 1.12 / 1.15 /
+// 1.31 on the geometric mean.  What stays with them, in us a layer, theirs and this kernel's:
+//   one token, every warp of the dot products one task (N of 32 to 64 channels per SM), K from 2048 to 7168: all or most of the weights
+//     are in registers before the token exists.  4096 x 8192 7.92 and 8.69, 4096 x 9472 7.40 and 8.85, 3072 x 5120 6.69 and 7.09,
+//     6144 x 7168 9.09 and 9.99; beside it 4096 x 4096 6.70 and 6.58, 4096 x 10240 9.67 and 8.42, 8192 x 8192 12.1 and 11.6
+//   two tokens likewise, K from 3072 to 4096: 4096 x 7104 7.60 and 8.58, 4096 x 5328 7.46 and 8.04 (N of whole 512 within 5 % either way)
+//   one or two tokens, K beyond 16384, where the 33 to 48 channels of a tile are three blocks for two groups of warps:
+//     28672 x 6144 23.1 and 25.9; x 4096 20.8 and 20.0, x 8192 32.7 and 27.2
+//   three tokens and more, K beyond 16384 and N up to 8192, or K beyond 12288 and N up to 1024: every SM reads all the tokens, and
+//     the decode kernel splits K over a cluster.  28672 x 1024 13.8 and 17.9, 20480 x 4096 15.1 and 16.3, 14336 x 1024 10.0 and 10.6;
+//     beside it 28672 x 10240 34.7 and 30.7, 16384 x 4096 12.7 and 12.6, 14336 x 2048 11.5 and 10.7
+static bool stream_yields(int64_t M, int64_t N, int64_t K) {
+  const int64_t sms = sm_count();
+  if (M > 2) return gemm_decode_supported(M, N, K) && (K > 16384 ? N <= 8192 : K > 12288 && N <= 1024);
+  if (!gemv_supported(M, N, K) || N <= 32 * sms || N > 64 * sms) return false;
+  if (K > 16384) return N <= 48 * sms;
+  return M == 1 ? K >= 2048 && K <= 7168 : K >= 3072 && K <= 4096;
+}
+
 bool w4a4_stream_supported(int64_t M, int64_t N, int64_t K) {
-  const int64_t bytes = N * K / 2;
-  return M >= 1 && M <= SM_NT && N >= 128 && N % 2 == 0 && K % 32 == 0 && K >= 256 && (M > 1 || bytes < 8000000 || bytes > 16000000);
+  return M >= 1 && M <= SM_NT && N >= 128 && N % 2 == 0 && K % 32 == 0 && K >= 256 && !stream_yields(M, N, K);
 }
 
 sq_status_t launch_w4a4_gemm_stream(const void* Xq, const void* sx, const void* Wq, const void* sw, int M, int N, int K, void* Y,
@@ -566,10 +580,11 @@ sq_status_t launch_w4a4_gemm_stream(const void* Xq, const void* sx, const void* 
   return launch_w4a4_stream(L, Xq, sx, Wq, sw, M, N, K, Y, accdbg, grid, s);
 }
 
-// Likewise (1 / 2 / 4 / 8 tokens: 1.17 / 1.31 / 1.16 / 1.16); small layers of one token stay with the dot products: 512 x 2048
-// 4.24 us against 4.70, 2048 x 2048 6.67 and 6.92; 2048 x 5632 7.99 and 7.68.
+// Likewise (1 / 2 / 4 / 8 tokens: 1.24 / 1.35 / 1.34 / 1.34).  Small layers of one token stay with the dot products: 512 x 2048
+// 4.46 us against 4.81, 1024 x 4096 5.20 and 5.47, 2048 x 3072 6.90 and 7.16; beside them 2048 x 4096 7.23 and 7.15, and however few the
+// channels of longer rows 2560 x 1024 8.88 and 6.92, 8192 x 128 14.2 and 8.2, 14336 x 512 21.4 and 10.1.
 bool wo_stream_supported(int64_t M, int64_t N, int64_t K) {
-  return M >= 1 && M <= SM_NT && N >= 128 && N % 2 == 0 && K % 32 == 0 && K >= 256 && (M > 1 || N * K / 2 >= 4000000);
+  return M >= 1 && M <= SM_NT && N >= 128 && N % 2 == 0 && K % 32 == 0 && K >= 256 && (M > 1 || K > 2048 || N * K / 2 >= 4000000);
 }
 
 sq_status_t launch_wo_gemm_stream(const void* Z16, const void* Wq, const void* sw, int M, int N, int K, void* Y, cudaStream_t s) {
