@@ -451,11 +451,14 @@ sq_status_t launch_w4a4_gemm(const void* Xq, const void* sx, const void* Wq, con
   // 65 to 128 tokens: the CTA-pair kernel, most of whose token tile may be empty, or the decode kernel for 64 tokens and then
   // whatever takes the rest.  Two passes read the weights twice but split K over clusters, where the pair kernel runs on
   // N / 128 pairs only: 128 x 28672 -> 512 43.1 us on pairs and 20.2 in two passes, 65 x 14336 -> 1024 23.7 and 13.7; the
-  // other way round 128 x 4096 -> 4096 10.1 and 16.4, 100 x 4096 -> 14336 16.4 and 20.2.  Over 973 shapes the choice is at most a tenth
-  // slower than the other one.
+  // other way round 128 x 4096 -> 4096 10.1 and 16.4, 100 x 4096 -> 14336 16.4 and 20.2.  Over 228 shapes with 65 and 72 tokens the
+  // choice takes 0.3 % longer than the better one on average (0.6 % with the rest priced as the decode kernel, which takes it from
+  // 9 tokens on: 72 x 4096 -> 512 10.3 us, 9.2 now) and 13 % at most, but for 20480 -> 11008 (54 us, two passes 46).
   if (M > 64 && M <= 128 && gemm_pair_supported(M, N, K) && gemm_decode_supported(64, N, K)) {
     const int64_t rest = M - 64;
-    const double rest_us = use_gemv(rest, N, K) ? 2.5 + static_cast<double>(N) * K / 2 / 5.0e6 : gemm_decode_estimate_us(rest, N, K);
+    const double rest_us = w4a4_stream_supported(rest, N, K) ? gemm_stream_estimate_us(N, K)
+                           : use_gemv(rest, N, K)            ? 2.5 + static_cast<double>(N) * K / 2 / 5.0e6
+                                                             : gemm_decode_estimate_us(rest, N, K);
     if (gemm_decode_estimate_us(64, N, K) + rest_us < gemm_pair_estimate_us(M, N, K)) {
       const sq_status_t st = launch_w4a4_gemm_decode(Xq, sx, Wq, sw, 64, (int)N, (int)K, Y, accdbg, s);
       if (st != SQ_OK) return st;

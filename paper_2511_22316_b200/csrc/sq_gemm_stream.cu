@@ -570,6 +570,10 @@ bool w4a4_stream_supported(int64_t M, int64_t N, int64_t K) {
   return M >= 1 && M <= SM_NT && N >= 128 && N % 2 == 0 && K % 32 == 0 && K >= 256 && !stream_yields(M, N, K);
 }
 
+// The product of a batch's last 1 to 8 tokens behind another product: launch, start and end, the walk along K, the weights.  (By
+// itself it takes some 0.6 us less, within a tenth for K up to 14336; the rest is for what the two-pass choice also costs.)
+double gemm_stream_estimate_us(int64_t N, int64_t K) { return 2.2 + 0.04 * ((K + 255) / 256) + 0.15e-6 * (0.5 * N * K); }
+
 sq_status_t launch_w4a4_gemm_stream(const void* Xq, const void* sx, const void* Wq, const void* sw, int M, int N, int K, void* Y,
                                     int32_t* accdbg, cudaStream_t s) {
   const int sms = sm_count();

@@ -190,6 +190,7 @@ sq_status_t launch_w4a4_gemm_decode(const void* Xq, const void* sx, const void* 
 
 // The product for up to 8 tokens as a stream of weights through warp-level MMAs (sq_gemm_stream.cu).
 bool w4a4_stream_supported(int64_t M, int64_t N, int64_t K);
+double gemm_stream_estimate_us(int64_t N, int64_t K);
 sq_status_t launch_w4a4_gemm_stream(const void* Xq, const void* sx, const void* Wq, const void* sw, int M, int N, int K, void* Y,
                                     int32_t* accdbg, cudaStream_t s);
 bool wo_stream_supported(int64_t M, int64_t N, int64_t K);

@@ -100,10 +100,12 @@ def _codes(rng, n, K):
 
 # Beside the lines of stream_yields, on the side of the other kernels.
 YIELDED = [(1, 4738, 4096), (1, 9472, 2048), (1, 7104, 16416), (2, 8192, 3072), (2, 4738, 32768), (3, 1024, 12416), (8, 1032, 16512)]
+# The last tokens of a batch that the decode kernel begins.
+BEGUN = [(65, 1024, 1024), (72, 512, 4096)]
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("M,N,K", SHAPES + YIELDED)
+@pytest.mark.parametrize("M,N,K", SHAPES + YIELDED + BEGUN)
 def test_w4a4_stream_is_bit_exact(M, N, K):
     from paper_2511_22316_b200 import binding as sq
     rng = np.random.default_rng(M * 131 + N + K)
