@@ -43,20 +43,25 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 INT8_OVER_BF16 = 2.0      # nominal dense ratio (4.5 POPS int8 : 2.25 PFLOP/s bf16)
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised under
-# profiles/ (bytes; None until a capture exists for that kernel and workload).
+# profiles/: step, workload -> kernel captured, bytes.  None until a capture exists for that kernel and workload.
 NCU_TRAFFIC = {
-    ("gemm", "llama2_7b_qkvo_prefill"): 12632320,           # w4a4_gemm_pair_kernel: reads (Y stays in L2)
-    ("rotate_quant", "llama2_7b_qkvo_prefill"): 16887040,   # rotate_quant_tc_kernel
-    ("rotate_quant_st", "llama2_7b_qkvo_prefill"): 16875520,  # rotate_quant_st_kernel (--structured-r2)
-    ("gemm", "llama3_8b_up_decode_m16"): 29457152,          # w4a4_gemm_decode_kernel, K not split
-    ("gemm", "llama3_8b_down_decode_m16"): 29519104,        # w4a4_gemm_decode_kernel, K over clusters of 4
-    ("gemm", "llama3_8b_up_decode_m1"): 29410560,           # w4a4_gemv_kernel
-    ("rotate_quant", "llama2_7b_down_prefill"): 45460480,   # rotate_quant_pair_kernel
-    ("rotate_quant", "llama2_70b_gateup_prefill"): 70202624,   # rotate_quant_tc_kernel, n2 = 128
-    ("rotate_quant", "llama2_70b_down_prefill"): 276784640,    # rotate_quant_pair_kernel, n2 = 128
-    ("wo_gemm", "llama3_8b_up_decode_m16"): 29557760,       # wo_gemm_tmem_kernel<16, 4, 8> (W4A16)
-    ("wo_gemm", "llama2_7b_qkvo_prefill"): 25251584,        # wo_gemm_pair_kernel (W4A16; Y stayed in L2)
+    ("gemm", "llama2_7b_qkvo_prefill"): ("w4a4_gemm_pair_kernel", 12632320),           # reads (Y stays in L2)
+    ("rotate_quant", "llama2_7b_qkvo_prefill"): ("rotate_quant_tc_kernel", 16887040),
+    ("rotate_quant_st", "llama2_7b_qkvo_prefill"): ("rotate_quant_st_kernel", 16875520),   # --structured-r2
+    ("gemm", "llama3_8b_up_decode_m16"): ("w4a4_gemm_decode_kernel", 29457152),        # K not split
+    ("gemm", "llama3_8b_down_decode_m16"): ("w4a4_gemm_decode_kernel", 29519104),      # K over clusters of 4
+    ("gemm", "llama3_8b_up_decode_m1"): ("w4a4_gemm_stream_kernel", 29425408),
+    ("rotate_quant", "llama2_7b_down_prefill"): ("rotate_quant_pair_kernel", 45460480),
+    ("rotate_quant", "llama2_70b_gateup_prefill"): ("rotate_quant_tc_kernel", 70202624),   # n2 = 128
+    ("rotate_quant", "llama2_70b_down_prefill"): ("rotate_quant_pair_kernel", 276784640),  # n2 = 128
+    ("wo_gemm", "llama3_8b_up_decode_m16"): ("wo_gemm_tmem_kernel", 29557760),         # <16, 4, 8> (W4A16)
+    ("wo_gemm", "llama2_7b_qkvo_prefill"): ("wo_gemm_pair_kernel", 25251584),          # W4A16; Y stayed in L2
 }
+
+
+def ncu_traffic(step, workload, kernel):
+    captured, nbytes = NCU_TRAFFIC.get((step, workload), (None, None))
+    return nbytes if captured == kernel else None
 
 
 def peaks():
@@ -86,11 +91,24 @@ def gemm_bytes(w):
     return (w.M + w.N) * w.K / 2.0 + 2.0 * w.M * w.N + 2.0 * (w.M + w.N)
 
 
+def stream_kernel_takes(M, N, K, sms=148):
+    """Whether sq_w4a4_gemm runs the stream kernel (mirrors w4a4_stream_supported)."""
+    if not (1 <= M <= 8 and N >= 128 and N % 2 == 0 and K % 32 == 0 and K >= 256):
+        return False
+    if M > 2:
+        return not (K % 128 == 0 and N % 8 == 0 and (N <= 8192 if K > 16384 else K > 12288 and N <= 1024))
+    if K > 32768 or not 32 * sms < N <= 64 * sms:
+        return True
+    if K > 16384:
+        return N > 48 * sms
+    return not (2048 <= K <= 7168 if M == 1 else 3072 <= K <= 4096)
+
+
 def gemm_kernel_name(w):
     """The kernel sq_w4a4_gemm picks for this shape (mirrors the library's dispatch)."""
     fast = w.K % 128 == 0 and w.N % 8 == 0
     decode = fast and w.M <= 64 and w.N >= 128 and w.K >= 256
-    if w.M <= 8 and w.N >= 128 and w.N % 2 == 0 and w.K % 32 == 0 and w.K >= 256 and (w.M > 1 or not 8e6 <= w.N * w.K / 2 <= 16e6):
+    if stream_kernel_takes(w.M, w.N, w.K):
         return "w4a4_gemm_stream_kernel"
     if w.M <= 4 and w.K % 32 == 0 and w.K <= 32768 and (w.M <= 2 or not decode):
         return "w4a4_gemv_kernel"
@@ -99,6 +117,21 @@ def gemm_kernel_name(w):
     if fast and w.M > 64 and w.N >= 128:
         return "w4a4_gemm_pair_kernel"
     return "w4a4_gemm_tc_kernel" if fast else "w4a4_gemm_simple_kernel"
+
+
+def wo_gemm_kernel_name(M, N, K):
+    """The kernel sq_w4a16_gemm picks for this shape (mirrors the library's dispatch on 148 SMs)."""
+    if M <= 8 and N >= 128 and N % 2 == 0 and K % 32 == 0 and K >= 256 and (M > 1 or K > 2048 or N * K / 2 >= 4e6):
+        return "wo_gemm_stream_kernel"
+    if M <= 2 and K % 32 == 0 and M * K * 4 <= 200 * 1024:
+        return "wo_gemv_kernel"
+    if K % 64 != 0 or N % 8 != 0:
+        return "wo_gemm_simple_kernel"
+    if N < 128:
+        return "wo_gemm_tc_kernel"
+    tiles = (N + 255) // 256
+    pairs = M > 128 or -(-tiles // 74) < 2 * -(-tiles // 148)
+    return "wo_gemm_pair_kernel" if M > 64 and N >= 256 and pairs else "wo_gemm_tmem_kernel"
 
 
 def rotate_kernel_name(w, structured=False):
@@ -447,25 +480,26 @@ def rooflines(w, rq_ms, gemm_ms, pk, structured, yard=None):
     gemm_tops = ops_per_step(w) / (gemm_ms * 1e-3) / 1e12
     rq_gbs = rotate_quant_bytes(w) / (rq_ms * 1e-3) / 1e9
     int8_peak = pk["bf16_tflops"] * INT8_OVER_BF16
+    kernel, rotate_kernel = gemm_kernel_name(w), rotate_kernel_name(w, structured)
     if w.M <= 64:       # decode: bound by reading the packed weights once
         gemm_gbs = gemm_bytes(w) / (gemm_ms * 1e-3) / 1e9
-        roof_gemm = {"kernel": gemm_kernel_name(w), "bound": "hbm", "achieved": gemm_gbs, "peak": pk["hbm_gbs"],
+        roof_gemm = {"kernel": kernel, "bound": "hbm", "achieved": gemm_gbs, "peak": pk["hbm_gbs"],
                      "unit": "GB/s", "frac": gemm_gbs / pk["hbm_gbs"],
-                     "traffic": NCU_TRAFFIC.get(("gemm", w.name)),
+                     "traffic": ncu_traffic("gemm", w.name, kernel),
                      "peak_source": f"{pk['source']} copy bandwidth", "ms_per_launch": gemm_ms,
                      "algorithmic_bytes": gemm_bytes(w), "frac_of_spec_8000": gemm_gbs / 8000.0}
     else:
-        roof_gemm = {"kernel": gemm_kernel_name(w), "bound": "tensor", "achieved": gemm_tops, "peak": int8_peak,
+        roof_gemm = {"kernel": kernel, "bound": "tensor", "achieved": gemm_tops, "peak": int8_peak,
                      "unit": "TOP/s", "frac": gemm_tops / int8_peak,
-                     "traffic": NCU_TRAFFIC.get(("gemm", w.name)),
+                     "traffic": ncu_traffic("gemm", w.name, kernel),
                      "peak_source": f"{pk['source']} bf16 burst x{INT8_OVER_BF16:g} (nominal int8:bf16 ratio)",
                      "ms_per_launch": gemm_ms, "algorithmic_ops": ops_per_step(w),
                      "frac_of_spec_4500": gemm_tops / 4500.0}
         if yard is not None:
             roof_gemm["yardstick"] = dict(yard, frac=gemm_tops / yard["tops"])
-    roof_rq = {"kernel": rotate_kernel_name(w, structured), "bound": "hbm", "achieved": rq_gbs, "peak": pk["hbm_gbs"],
+    roof_rq = {"kernel": rotate_kernel, "bound": "hbm", "achieved": rq_gbs, "peak": pk["hbm_gbs"],
                "unit": "GB/s", "frac": rq_gbs / pk["hbm_gbs"],
-               "traffic": NCU_TRAFFIC.get(("rotate_quant_st" if structured else "rotate_quant", w.name)),
+               "traffic": ncu_traffic("rotate_quant_st" if structured else "rotate_quant", w.name, rotate_kernel),
                "peak_source": f"{pk['source']} copy bandwidth", "ms_per_launch": rq_ms,
                "algorithmic_bytes": rotate_quant_bytes(w), "frac_of_spec_8000": rq_gbs / 8000.0}
     return roof_gemm, roof_rq
@@ -549,19 +583,20 @@ def weight_only_entry(sq, torch, w, bits, pk, l2, quick=False):
     flops = 2.0 * M * N * K
     gemm_bytes_wo = N * K / 2.0 + 2.0 * M * K + 2.0 * M * N + 2.0 * N
     rot_bytes = 4.0 * M * K
+    kernel = wo_gemm_kernel_name(M, N, K)
+    traffic = ncu_traffic("wo_gemm", w.name, kernel) if bits == 4 else None
     if M <= 64:
         gbs = gemm_bytes_wo / (gemm_ms * 1e-3) / 1e9
-        roof = {"kernel": "wo_gemm_stream_kernel" if M <= 8 else "wo_gemm_tmem_kernel", "bound": "hbm", "achieved": gbs, "peak": pk["hbm_gbs"], "unit": "GB/s",
-                "frac": gbs / pk["hbm_gbs"], "traffic": NCU_TRAFFIC.get(("wo_gemm", w.name)) if bits == 4 else None,
+        roof = {"kernel": kernel, "bound": "hbm", "achieved": gbs, "peak": pk["hbm_gbs"], "unit": "GB/s",
+                "frac": gbs / pk["hbm_gbs"], "traffic": traffic,
                 "ms_per_launch": gemm_ms,
                 "algorithmic_bytes": gemm_bytes_wo}
     else:
         tf = flops / (gemm_ms * 1e-3) / 1e12
-        tc_ok = N >= 128 and K % 64 == 0 and N % 8 == 0
-        roof = {"kernel": ("wo_gemm_pair_kernel" if (M > 128 and N >= 256) else "wo_gemm_tmem_kernel") if tc_ok else "wo_gemm_tc_kernel",
+        roof = {"kernel": kernel,
                 "bound": "tensor", "achieved": tf, "peak": pk["bf16_tflops"],
                 "unit": "TFLOP/s", "frac": tf / pk["bf16_tflops"],
-                "traffic": NCU_TRAFFIC.get(("wo_gemm", w.name)) if bits == 4 else None, "ms_per_launch": gemm_ms,
+                "traffic": traffic, "ms_per_launch": gemm_ms,
                 "peak_source": f"{pk['source']} bf16 burst (fp16 runs at the same rate)", "algorithmic_flops": flops}
         try:
             if quick:

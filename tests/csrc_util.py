@@ -42,3 +42,19 @@ def wo_pair_widths(shapes, pairs=74):
             + "\nint main(int n, char** v) { for (int i = 1; i + 1 < n; i += 2)"
               " printf(\"%d\\n\", wo_pair_tile_m(atoi(v[i]), atoi(v[i + 1]), PAIRS)); }")
     return [int(row[0]) for row in run(code.replace("PAIRS", str(pairs)), *[v for s in shapes for v in s])]
+
+
+def stream_takes(shapes):
+    """For each (M, N, K) whether the stream kernels take the W4A4 and the weight-only product, on 148 SMs."""
+    src = source("sq_gemm_stream.cu")
+    rows = run(lines(src, r"^constexpr int SM_.*$") + "\nint sm_count() { return 148; }\n"
+               + block(source("sq_gemm_decode.cu"), "bool gemm_decode_supported(") + block(source("sq_gemv.cu"), "bool gemv_supported(")
+               + block(src, "static bool stream_yields(") + block(src, "bool w4a4_stream_supported(")
+               + block(src, "bool wo_stream_supported(") + """
+int main(int n, char** v) {
+  for (int i = 1; i + 2 < n; i += 3) {
+    const int M = atoi(v[i]), N = atoi(v[i + 1]), K = atoi(v[i + 2]);
+    printf("%d %d\\n", w4a4_stream_supported(M, N, K), wo_stream_supported(M, N, K));
+  }
+}""", *(v for s in shapes for v in s))
+    return [(row[0] == "1", row[1] == "1") for row in rows]

@@ -43,24 +43,13 @@ int main() {
 
 def test_what_the_stream_kernels_leave_to_the_others():
     """The lines that the measurements beside them draw, both sides of each, on 148 SMs."""
-    src = csrc_util.source("sq_gemm_stream.cu")
     cases = [(1, 4736, 4096, 1), (1, 4738, 4096, 0), (1, 9472, 4096, 0), (1, 9474, 4096, 1), (1, 8192, 2016, 1), (1, 8192, 2048, 0),
              (1, 8192, 7168, 0), (1, 8192, 7200, 1), (1, 7104, 16416, 0), (1, 7106, 16416, 1), (1, 6144, 16384, 1), (1, 6144, 32800, 1),
              (2, 8192, 3040, 1), (2, 8192, 3072, 0), (2, 8192, 4096, 0), (2, 8192, 4128, 1), (2, 9474, 4096, 1), (2, 6144, 28672, 0),
              (3, 8192, 4096, 1), (3, 1024, 12288, 1), (3, 1024, 12416, 0), (8, 1032, 12416, 1), (8, 8192, 16512, 0), (8, 8200, 16512, 1),
              (8, 8192, 16416, 1), (9, 4096, 4096, 0), (4, 126, 4096, 0), (4, 129, 4096, 0), (4, 4096, 224, 0), (4, 4096, 4112, 0)]
-    rows = csrc_util.run(
-        csrc_util.lines(src, r"^constexpr int SM_.*$") + "\nint sm_count() { return 148; }\n"
-        + csrc_util.block(csrc_util.source("sq_gemm_decode.cu"), "bool gemm_decode_supported(")
-        + csrc_util.block(csrc_util.source("sq_gemv.cu"), "bool gemv_supported(")
-        + csrc_util.block(src, "static bool stream_yields(") + csrc_util.block(src, "bool w4a4_stream_supported(")
-        + csrc_util.block(src, "bool wo_stream_supported(") + """
-int main(int n, char** v) {
-  for (int i = 1; i + 2 < n; i += 3)
-    printf("%d %d\\n", w4a4_stream_supported(atoi(v[i]), atoi(v[i + 1]), atoi(v[i + 2])), wo_stream_supported(atoi(v[i]), atoi(v[i + 1]), atoi(v[i + 2])));
-}""", *(v for c in cases for v in c[:3]), 1, 4096, 2048, 1, 3900, 2048, 1, 128, 2080)
-    assert [int(r[0]) for r in rows[:len(cases)]] == [c[3] for c in cases]
-    assert [int(r[1]) for r in rows[len(cases):]] == [1, 0, 1]
+    assert [w4a4 for w4a4, _ in csrc_util.stream_takes([c[:3] for c in cases])] == [bool(c[3]) for c in cases]
+    assert [wo for _, wo in csrc_util.stream_takes([(1, 4096, 2048), (1, 3900, 2048), (1, 128, 2080)])] == [True, False, True]
 
 
 def _rows(rows, M):
