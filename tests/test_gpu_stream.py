@@ -115,7 +115,7 @@ def test_w4a4_stream_is_bit_exact(M, N, K):
 # The same, and K over clusters of 2, 4 and 8 (few channels, long K).
 @pytest.mark.gpu
 @pytest.mark.parametrize("M,N,K", [s for s in SHAPES if s[0] > 1] + [(1, 5128, 4096), (8, 136, 8192), (8, 1024, 8192), (7, 4098, 14336),
-                                                                  (8, 8192, 28672)])
+                                                                  (8, 8192, 28672), (8, 136, 65536), (3, 2050, 65536)])
 def test_weight_only_stream_is_bit_exact_on_integers(M, N, K):
     """Tokens in [-8, 8], steps powers of two: every partial sum is an integer below 2^24, so that any order gives the same."""
     from paper_2511_22316_b200 import binding as sq
@@ -152,3 +152,106 @@ def test_weight_only_stream_stays_within_the_fp32_accumulation_bound(M, K):
     z, w, s = Z.astype(np.float64), Wc.astype(np.float64), sw.astype(np.float64)
     want, mag = z @ w.T * s, np.abs(z) @ np.abs(w).T * s
     assert np.all(np.abs(got - want) <= 2.0 ** -10 * np.abs(want) + K * 2.0 ** -23 * mag + 2.0 ** -24)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K", [(3, 130, 288), (8, 1024, 8192), (5, 4106, 1312)])
+def test_infinities_and_nan_stay_with_their_token_and_channel(M, N, K):
+    """An infinity or NaN among the tokens or in a step spoils its own row or column and no other bit."""
+    from paper_2511_22316_b200 import binding as sq
+    rng = np.random.default_rng(N + K)
+    Z, Wc = rng.standard_normal((M, K)).astype(np.float16), _codes(rng, N, K)
+    Xc = _codes(rng, M, K)
+    sx, sw = rng.uniform(0.01, 2.0, size=M).astype(np.float16), rng.uniform(0.001, 0.1, size=N).astype(np.float16)
+    wq, wi, xq = dev(ora.pack_int4(Wc)), dev(ora.pack_int4_interleaved(Wc)), dev(ora.pack_int4(Xc))
+
+    def both(z, steps_x, steps_w):
+        y, yw = Guarded(M * N * 2), Guarded(M * N * 2)
+        sq.sq_w4a4_gemm(xq, dev(steps_x), wq, dev(steps_w), M, N, K, y)
+        sq.sq_w4a16_gemm(dev(z), wi, dev(steps_w), M, N, K, yw)
+        torch_mod().cuda.synchronize()
+        assert sq.sq_last_device_status() == sq.SQ_OK
+        y.check(), yw.check()
+        return y.numpy(np.float16, (M, N)), yw.numpy(np.float16, (M, N))
+
+    clean = both(Z, sx, sw)
+    Z[1, K - 1], Z[2, 0], sx[1], sw[N - 1] = np.inf, np.nan, np.inf, np.nan
+    spoilt = both(Z, sx, sw)
+    rows = [np.arange(M) != 1, (np.arange(M) != 1) & (np.arange(M) != 2)]
+    for a, b, keep in zip(clean, spoilt, rows):
+        assert np.array_equal(a[keep, :-1], b[keep, :-1]) and np.all(np.isnan(b[:, -1]))
+        assert not np.any(np.isfinite(b[~keep]))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("bits", [0, 4])
+def test_a_product_right_behind_the_packing_reads_the_new_weights(bits):
+    """Queued without a wait, on a buffer that held other weights: the product asks for its first weights ahead of the kernel
+    before it, and must not be let go before they are written."""
+    from paper_2511_22316_b200 import binding as sq
+    torch = torch_mod()
+    n1, n2, M, N = 16, 64, 4, 4096
+    K = n1 * n2
+    rng = np.random.default_rng(bits)
+    rot = sq.sq_build_rotation(rng.standard_normal((8, K)).astype(np.float32), n1, n2, seed=1)
+    W = [dev(rng.standard_normal((N, K)).astype(np.float16)) for _ in range(2)]
+    x = dev(rng.standard_normal((M, K)).astype(np.float16)) if bits else dev(ora.pack_int4(_codes(rng, M, K)))
+    sx = dev(np.ones(M, np.float16))
+    Wq, sw = torch.empty(N * K // 2, dtype=torch.uint8, device="cuda"), torch.empty(N, dtype=torch.float16, device="cuda")
+    y = [torch.empty(M, N, dtype=torch.float16, device="cuda") for _ in range(4)]
+
+    def pack(w):
+        if bits:
+            sq.sq_pack_weight_wo(rot, w, N, K, bits, Wq, sw)
+        else:
+            sq.sq_pack_weight(rot, w, N, K, Wq, sw)
+
+    def product(out):
+        if bits:
+            sq.sq_w4a16_gemm(x, Wq, sw, M, N, K, out)
+        else:
+            sq.sq_w4a4_gemm(x, sx, Wq, sw, M, N, K, out)
+
+    for w, out in zip(W, y):                       # with a wait
+        pack(w)
+        torch.cuda.synchronize()
+        product(out)
+        torch.cuda.synchronize()
+    assert not torch.equal(y[0], y[1])
+    for turn in range(20):                         # without
+        for w, out in zip(W, y[2:]):
+            pack(w)
+            product(out)
+        torch.cuda.synchronize()
+        assert sq.sq_last_device_status() == sq.SQ_OK
+        assert torch.equal(y[0], y[2]) and torch.equal(y[1], y[3]), turn
+    rot.close()
+
+
+@pytest.mark.gpu
+def test_grouped_experts_of_few_rows_with_ragged_channels():
+    """K % 128 != 0: experts one by one, their steps and outputs at odd rows.  Same bits as expert by expert on its own."""
+    from paper_2511_22316_b200 import binding as sq
+    torch = torch_mod()
+    n1, n2, N = 33, 32, 136
+    K, offsets = n1 * n2, [0, 3, 4, 4, 9, 17]
+    M, E = offsets[-1], len(offsets) - 1
+    rng = np.random.default_rng(7)
+    X = dev(rng.standard_normal((M, K)).astype(np.float16))
+    rot = sq.sq_build_rotation(rng.standard_normal((8, K)).astype(np.float32), n1, n2, seed=1)
+    Wq = [dev(ora.pack_int4(_codes(rng, N, K))) for _ in range(E)]
+    sw = [dev(rng.uniform(0.001, 0.1, size=N).astype(np.float16)) for _ in range(E)]
+    nbytes = sq.sq_linear_workspace_bytes(M, K)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    y, one = Guarded(M * N * 2), Guarded(M * N * 2)
+    sq.sq_linear_grouped([rot] * E, offsets, X, Wq, sw, N, K, ws, nbytes, y)
+    out = one.view.view(torch.float16).view(M, N)
+    for e in range(E):
+        r0, r1 = offsets[e], offsets[e + 1]
+        if r1 > r0:
+            sq.sq_linear(rot, X[r0:r1], r1 - r0, Wq[e], sw[e], N, K, ws, nbytes, out[r0:r1])
+    torch.cuda.synchronize()
+    assert sq.sq_last_device_status() == sq.SQ_OK
+    y.check(), one.check()
+    assert np.array_equal(y.numpy(np.uint16, (M, N)), one.numpy(np.uint16, (M, N)))
+    rot.close()
