@@ -46,13 +46,13 @@ INT8_OVER_BF16 = 2.0      # nominal dense ratio (4.5 POPS int8 : 2.25 PFLOP/s bf
 # profiles/: step, workload -> kernel captured, bytes.  None until a capture exists for that kernel and workload.
 NCU_TRAFFIC = {
     ("gemm", "llama2_7b_qkvo_prefill"): ("w4a4_gemm_pair_kernel", 12632320),           # reads (Y stays in L2)
-    ("rotate_quant", "llama2_7b_qkvo_prefill"): ("rotate_quant_tc_kernel", 16887040),
-    ("rotate_quant_st", "llama2_7b_qkvo_prefill"): ("rotate_quant_st_kernel", 16875520),   # --structured-r2
+    ("rotate_quant", "llama2_7b_qkvo_prefill"): ("rotate_quant_tc_kernel", 16886272),
+    ("rotate_quant_st", "llama2_7b_qkvo_prefill"): ("rotate_quant_st_kernel", 16874752),   # --structured-r2
     ("gemm", "llama3_8b_up_decode_m16"): ("w4a4_gemm_decode_kernel", 29457152),        # K not split
     ("gemm", "llama3_8b_down_decode_m16"): ("w4a4_gemm_decode_kernel", 29519104),      # K over clusters of 4
     ("gemm", "llama3_8b_up_decode_m1"): ("w4a4_gemm_stream_kernel", 29425408),
     ("rotate_quant", "llama2_7b_down_prefill"): ("rotate_quant_pair_kernel", 45460480),
-    ("rotate_quant", "llama2_70b_gateup_prefill"): ("rotate_quant_tc_kernel", 70202624),   # n2 = 128
+    ("rotate_quant", "llama2_70b_gateup_prefill"): ("rotate_quant_tc_kernel", 71069952),   # n2 = 128
     ("rotate_quant", "llama2_70b_down_prefill"): ("rotate_quant_pair_kernel", 276784640),  # n2 = 128
     ("wo_gemm", "llama3_8b_up_decode_m16"): ("wo_gemm_tmem_kernel", 29557760),         # <16, 4, 8> (W4A16)
     ("wo_gemm", "llama2_7b_qkvo_prefill"): ("wo_gemm_pair_kernel", 25251584),          # W4A16; Y stayed in L2
