@@ -123,6 +123,7 @@ void sq_rotation_destroy(sq_rotation_t* rot);
  *   X             DEVICE fp16 [M x n]
  *   Xq            DEVICE uint8 [M x n/2]   (out)
  *   sx            DEVICE fp16 [M]          (out; Delta_t; 0 for an all-zero row)
+ * A row with an infinity or NaN has no defined codes; the other rows do not depend on it.
  *   Zdbg_or_null  DEVICE fp32 [M x n]      (out, optional: the rotated rows, for parity tests) */
 sq_status_t sq_rotate_quant_act(const sq_rotation_t* rot, const void* X, int64_t M,
                                 void* Xq, void* sx, void* Zdbg_or_null, void* stream);
@@ -144,8 +145,9 @@ sq_status_t sq_pack_weight(const sq_rotation_t* rot_or_null, const void* W, int6
  * No scratch memory: every kernel keeps its intermediates on chip (split-K partial tiles are
  * exchanged through cluster shared memory).
  * Supported: K even, K <= 65536 (so that the 256x-scaled int32 accumulator cannot overflow).
- * The tensor-core path needs K % 128 == 0 and N % 8 == 0; other shapes run a plain integer
- * kernel with the same results.
+ * Up to 8 tokens the fast kernels take K % 32 == 0 (three tokens and more: N even, N >= 128 and
+ * K >= 256 besides), above that the tensor-core path needs K % 128 == 0 and N % 8 == 0; other shapes
+ * run a plain integer kernel.  The results are the same bits whichever kernel runs.
  * Ordering: the kernel is queued as a programmatic dependent of the kernel before it in `stream`: it
  * may request its first blocks of Wq while that kernel still runs, and waits for it before it reads Xq
  * or sx or writes Y.  Weights packed by sq_pack_weight / sq_pack_weight_wo on the same stream are
@@ -235,8 +237,12 @@ sq_status_t sq_rotate_act_f16(const sq_rotation_t* rot, const void* X, int64_t M
 /* Step 3 of the variant: Y[t,c] = fp16((sum_k Z16[t,k] * code[c,k]) * sw[c]), fp32 accumulation.
  *   Z16 DEVICE fp16 [M x K]      Wq DEVICE uint8 [N x K/2] (weight-only order)     sw DEVICE fp16 [N]
  *   Y   DEVICE fp16 [M x N] (out)
- * K % 8 == 0, K <= 65536.  The tensor-core path needs K % 64 == 0 and N % 8 == 0; other shapes run a
- * plain fp32 kernel (same definition, another summation order). */
+ * K % 8 == 0, K <= 65536.  Up to 8 tokens the fast kernels take K % 32 == 0 (three tokens and more: N
+ * even, N >= 128 and K >= 256 besides), above that the tensor-core path needs K % 64 == 0 and N % 8 == 0;
+ * other shapes run a plain fp32 kernel (same definition, another summation order).
+ * The order of the fp32 sums is fixed for given M, N and K, and a second call gives the same bits; it
+ * depends on M, also within 1 to 8 tokens (how many SMs share the channels and K), so a token's last bit
+ * may depend on how many tokens are multiplied with it. */
 sq_status_t sq_w4a16_gemm(const void* Z16, const void* Wq, const void* sw, int64_t M, int64_t N, int64_t K,
                           void* Y, void* stream);
 

@@ -7,9 +7,11 @@
 // the rest afterwards; here every SM holds up to 200 KB.  The weights go from shared memory to registers, where the nibbles are
 // widened, and on to the MMA: no operand ring and no hand-overs between roles, one wait per 256 channels.  What follows the
 // tokens is bound by the widening (logic pipe, half rate) and the latency of its chain with four warps per scheduler: 8 x 8192
-// -> 28672 in fp16 35 us, 37 % of the issue slots.  Layers: 1 x 4096 -> 14336 10.4 -> 9.9 us, 1 x 14336 -> 4096 13.8 -> 11.4, 8 x
-// 4096 -> 4096 8.0 -> 7.1; weight-only 1 x 4096 -> 14336 18.2 -> 13.6, 2 x 8192 -> 8192 23.7 -> 16.7, 8 x 4096 -> 11008 14.6 ->
-// 12.7.  16 tokens were tried too: INT4 12.1 us a layer against 11.7, fp16 17.3 and 16.6 (twice the MMAs and token fragments).
+// -> 28672 in fp16 34 us, 42 % of the issue slots.  Layers: 1 x 4096 -> 14336 10.4 -> 9.6 us, 1 x 14336 -> 4096 13.8 -> 11.5, 8 x
+// 4096 -> 4096 8.0 -> 7.0; weight-only 1 x 4096 -> 14336 18.5 -> 13.2, 2 x 8192 -> 8192 24.7 -> 16.4, 8 x 4096 -> 11008 14.9 ->
+// 12.5.  16 tokens were tried too: INT4 12.1 us a layer against 11.7, fp16 17.3 and 16.6 (twice the MMAs and token fragments).
+// Both kernels are at 96 registers, all that 18 warps (allocated as 20) leave a thread; the fp16 one spills ten words there, and
+// was tried for 16 tokens under that limit.
 //
 // A block takes a tile of up to 128 output channels, as many as give every SM the same share; its sixteen warps split K, and the
 // channels where there are more than 32, and add up at the end.  The weights are the A operand (16 channels x 32 or 16 of K), the

@@ -959,9 +959,8 @@ wo_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_z, const __grid_con
   }
 }
 
-// One or two tokens: dot products on the CUDA cores.  The product is pure streaming then (29 MB of
-// packed weights against a few MFLOP), and the tensor-core forms pay more in hand-overs than the read
-// costs.  Each warp takes four weight rows at a time; every lane reads 16-byte pieces of them straight
+// One token with a small layer (less than 4 MB, K up to 2048), and one or two tokens of shapes that the stream kernel does not
+// take: dot products on the CUDA cores.  Each warp takes four weight rows at a time; every lane reads 16-byte pieces of them straight
 // from global memory (coalesced, several in flight), widens the nibbles to half2 as above, converts to
 // fp32 and multiplies with the tokens, which the CTA holds in shared memory as fp32.  Accumulation is
 // fp32 throughout; a row's sum is completed by one warp (shuffle reduction): deterministic.
@@ -1257,7 +1256,7 @@ sq_status_t launch_wo_gemm(const void* Z16, const void* Wq, const void* sw, int6
   const bool tc_ok = (K % 64 == 0) && (N % 8 == 0);
   if (wo_stream_supported(M, N, K)) return launch_wo_gemm_stream(Z16, Wq, sw, (int)M, (int)N, (int)K, Y, s);
   if (M <= 2 && K % 32 == 0 && static_cast<int64_t>(M) * K * 4 <= 200 * 1024) {
-    // one or two tokens: dot products on the CUDA cores
+    // one or two tokens that the stream kernel leaves: dot products on the CUDA cores
     if (M == 1) return launch_wo_gemv<1>(Z16, Wq, sw, (int)M, (int)N, (int)K, Y, s);
     return launch_wo_gemv<2>(Z16, Wq, sw, (int)M, (int)N, (int)K, Y, s);
   }

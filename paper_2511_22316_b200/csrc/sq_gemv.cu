@@ -1,8 +1,9 @@
-// Step 3 for one to four tokens: the INT4 x INT4 product as dot products on the CUDA cores.
+// Step 3 for one to four tokens where the stream kernel leaves it to this one (stream_yields, sq_gemm_stream.cu): the INT4 x INT4
+// product as dot products on the CUDA cores.
 //
-// With M <= 4 the work is 2 M N K <= 0.5 GOP against 29 MB of packed weights: pure streaming, and
-// every tensor-core arrangement pays more in pipeline hand-overs and MMA issue than the whole
-// read costs.  Here each warp takes two weight rows at a time, every lane reads 16-byte pieces of
+// One or two tokens and 32 to 64 channels per SM: every warp has one task, and most or all of its weights are in registers before
+// the token exists.  Also three or four tokens, and one or two, of shapes that no other kernel takes (N odd or below 128).
+// Each warp takes two or four weight rows at a time, every lane reads 16-byte pieces of
 // them straight from global memory (coalesced, several in flight), widens the nibbles to
 // 16 x code in the top of each byte -- the same trick as the tensor-core kernels, so the dp4a
 // accumulator holds 256 x acc and the shift at the end is exact -- and multiplies them with the
