@@ -69,3 +69,30 @@ def test_an_infinity_stays_in_its_row_with_the_structured_factor(n1, n2):
         out.append((np.delete(q.numpy(np.uint8, (M, K // 2)), bad, 0), np.delete(s.numpy(np.uint16, (M,)), bad)))
     assert all(np.array_equal(a, b) for a, b in zip(*out))
     rot.close()
+
+
+@pytest.mark.parametrize("n1,n2,M", [(24, 128, 33), (32, 128, 64), (16, 64, 33)])
+def test_the_one_launch_layer_rotates_its_batch_alike(n1, n2, M):
+    """Its rotating blocks find out at run time how many tokens share an accumulator: codes, steps and outputs are those of the
+    kernels one after the other, an infinity in one row or not."""
+    from paper_2511_22316_b200 import binding as sq
+    torch, K, N, bad = torch_mod(), n1 * n2, 256, 5
+    rng = np.random.default_rng(n1 + M)
+    X = rng.standard_normal((M, K)).astype(np.float16)
+    rots = [sq.sq_build_rotation(X[:8].astype(np.float32), n1, n2, seed=1, flags=sq.SQ_ROT_DEFAULT | f) for f in (0, sq.SQ_ROT_FUSE_DECODE)]
+    Wq, sw = dev(rng.integers(0, 256, (N, K // 2), dtype=np.uint8)), dev(np.ones(N, np.float16))
+    nb = sq.sq_linear_workspace_bytes(M, K)
+    X[bad, K // 2] = np.inf
+    before, out = sq.sq_kernel_launch_count(), []
+    for rot in rots:
+        ws, y = torch.zeros(nb, dtype=torch.uint8, device="cuda"), Guarded(M * N * 2)
+        sq.sq_linear(rot, dev(X), M, Wq, sw, N, K, ws, nb, y)
+        torch.cuda.synchronize()
+        assert sq.sq_last_device_status() == sq.SQ_OK
+        y.check()
+        codes = ws[:M * K // 2].cpu().numpy().reshape(M, K // 2)
+        out.append([np.delete(a, bad, 0) for a in (codes, y.numpy(np.uint16, (M, N)))])
+    assert sq.sq_kernel_launch_count() - before == 3
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
+    for rot in rots:
+        rot.close()
